@@ -16,6 +16,7 @@
 
 #include "qm_internal.h"
 #include "qm_community.cuh"
+#include "qm_count.cuh"
 #include "qm_expand.cuh"
 #include "qm_finalize.cuh"
 
@@ -23,7 +24,7 @@ namespace qm {
 using namespace qmk;
 
 enum { C_BIG_COUNT = 0, C_BIG_NEXT = 1, C_SMALL_NEXT = 2, C_OVF_COUNT = 3, C_OVF_NEXT = 4, C_SMALL_COUNT = 5,
-       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_COUNT = 9, C_BX_BAD = 10 };
+       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_COUNT = 9, C_BX_BAD = 10, C_MID_NEXT = 11 };
 
 constexpr int SCAN_TILE = 4096;   // elements per block in the multi-block scan
 constexpr int SCAN_SINGLE_MAX = 1 << 16;
@@ -1137,6 +1138,163 @@ __global__ void __launch_bounds__(1024) k_count(CountKArgs a)
     }
 }
 
+// Phase B with one-word tables (qm_count.cuh), for fewer than CT_MAX_K label ids.
+// k_count_tab takes the runs of up to CT_FILL_GROUP entries: whole blocks (of
+// four warps) the longer ones, claimed one at a time, then single warps the
+// others, claim_chunk headers at a time, each with a quarter of the table.
+struct CountTabArgs {
+    CountCtx x;
+    const RunHdr *mid;    // runs for whole blocks of k_count_tab
+    const RunHdr *small;  // runs for single warps
+    const RunHdr *big;    // runs for k_count_big, staged
+    const RunHdr *lng;    // runs longer than those, counted in hash classes
+    int *counters;
+    const int *status;
+    int cb;               // bits of a table word left for the repeats
+    unsigned stage_wait;  // k_count_big: polls of each staging wait before the block gives up
+    SmemPlan plan;        // k_count_big: tables of the hash-class count
+};
+
+template <int MODE>
+__global__ void __launch_bounds__(CT_THREADS, CT_BLOCKS) k_count_tab(CountTabArgs a)
+{
+    __shared__ __align__(16) unsigned slot[CT_WORDS];
+    __shared__ unsigned late[CT_THREADS / 32][CT_LATE];
+    __shared__ unsigned long long red[8 * (CT_THREADS / 32)];
+    __shared__ int s_i;
+    if (*a.status) return;
+    constexpr int W = CT_THREADS / 32;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < CT_WORDS / 4; i += CT_THREADS)
+        reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const int nmid = a.counters[C_MID_COUNT];
+    for (;;) {
+        if (tid == 0) s_i = atomicAdd(&a.counters[C_MID_NEXT], 1);
+        block_sync();
+        const int i = s_i;
+        if (i >= nmid) break;
+        const RunHdr h = a.mid[i];
+        ct_count_run<MODE, false, CT_THREADS>(a.x, h, a.x.nbr + h.a0, slot, a.cb, tid, late[wid], red);
+    }
+    const int nsmall = a.counters[C_SMALL_COUNT];
+    const int chunk = claim_chunk(nsmall, (long long)gridDim.x * W);
+    unsigned *const ws = slot + wid * (CT_WORDS / W);
+    for (;;) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&a.counters[C_SMALL_NEXT], chunk);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (base >= nsmall) break;
+        RunHdr mine{-1, 0u, 0u, 0u};
+        if (lane < chunk && base + lane < nsmall) mine = a.small[base + lane];
+        const int cnt = min(chunk, nsmall - base);
+        for (int j = 0; j < cnt; ++j) {
+            const RunHdr h{__shfl_sync(0xffffffffu, mine.c, j), __shfl_sync(0xffffffffu, mine.a0, j),
+                           __shfl_sync(0xffffffffu, mine.m, j), __shfl_sync(0xffffffffu, mine.vol, j)};
+            ct_count_run<MODE, false, 32>(a.x, h, a.x.nbr + h.a0, ws, a.cb, lane, late[wid], red);
+        }
+    }
+}
+
+// The longer runs.  Runs of up to CB_FILL entries are counted with the same
+// tables while the block's next run is on its way into shared memory (a bulk
+// copy into the other of two buffers, completing on an mbarrier with a bounded
+// wait; the next copy is issued only after the current one has landed, so at
+// most one is in flight when a wait expires).  Then the list of the runs beyond
+// that: up to CB_FILL_LONG entries (and below 2^cb) with one table in the whole
+// shared memory, longer ones by hash classes (count_run_general).
+constexpr int CB_SMEM = 16 + CB_WORDS * 4 + 2 * CB_STAGE * 4;
+static_assert(CB_SMEM >= 16 + CB_WORDS_LONG * 4, "the unstaged table fits");
+
+template <int MODE>
+__global__ void __launch_bounds__(CB_THREADS, 2) k_count_big(CountTabArgs a)
+{
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ unsigned late[CB_THREADS / 32][CT_LATE];
+    __shared__ unsigned long long red[256];
+    __shared__ RunHdr ring[3];
+    __shared__ int s_timeout;
+    if (*a.status) return;
+    const int nbig = a.counters[C_BIG_COUNT], nlong = a.counters[C_LONG_COUNT];
+    const long long G = gridDim.x, b = blockIdx.x;
+    if (b >= nbig && b >= nlong) return;
+    unsigned long long *bars = (unsigned long long *)sm;
+    unsigned *slot = (unsigned *)(sm + 16);
+    int *stage = (int *)(sm + 16 + CB_WORDS * 4);
+    const int tid = threadIdx.x;
+    const RunHdr none{-1, 0u, 0u, 0u};
+    auto issue = [&](const RunHdr &h, int k) {
+        const unsigned lo = h.a0 & ~3u;
+        bulk_load_smem(stage + k * CB_STAGE, a.x.nbr + lo, ((h.a0 - lo) + h.m + 3u) / 4u * 16u, &bars[k]);
+    };
+    if (b < nbig) {
+        for (int i = tid; i < CB_WORDS / 4; i += CB_THREADS)
+            reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid == 0) {
+            s_timeout = 0;
+            mbar_init(&bars[0], 1);
+            mbar_init(&bars[1], 1);
+            fence_proxy_async_smem();
+            ring[0] = a.big[b];
+            ring[1] = b + G < nbig ? a.big[b + G] : none;
+            issue(ring[0], 0);
+        }
+        block_sync();
+        for (int it = 0;; ++it) {
+            const RunHdr h = ring[it % 3];
+            if (h.c < 0) break;
+            const int k = it & 1;
+            RunHdr nn = none;
+            if (tid == 0) {
+                if (mbar_wait(&bars[k], (unsigned)(it >> 1) & 1u, a.stage_wait)) {
+                    const RunHdr hn = ring[(it + 1) % 3];
+                    if (hn.c >= 0) {
+                        fence_proxy_async_smem();
+                        issue(hn, k ^ 1);
+                    }
+                    const long long idx = b + (long long)(it + 2) * G;
+                    if (idx < nbig) nn = a.big[idx];
+                } else {
+                    s_timeout = 1;
+                    atomicOr(a.x.err, 4);
+                    // the copy in flight lands before the block (and its shared memory) goes away
+                    mbar_wait(&bars[k], (unsigned)(it >> 1) & 1u, STAGE_WAIT_LIMIT);
+                }
+            }
+            block_sync();
+            if (s_timeout) return;
+            ct_count_run<MODE, true, CB_THREADS>(a.x, h, stage + k * CB_STAGE + (h.a0 & 3u), slot, a.cb, tid,
+                                                late[tid >> 5], red);
+            if (tid == 0) ring[(it + 2) % 3] = nn;
+            block_sync();
+        }
+    }
+    if (b >= nlong) return;
+    block_sync();
+    const unsigned most = min((unsigned)CB_FILL_LONG, (1u << a.cb) - 1u);
+    bool general = false;
+    for (int i = tid; i < CB_WORDS_LONG / 4; i += CB_THREADS)
+        reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
+    block_sync();
+    for (long long i = b; i < nlong; i += G) {
+        const RunHdr h = a.lng[i];
+        if (h.m <= most) ct_count_run<MODE, false, CB_THREADS>(a.x, h, a.x.nbr + h.a0, slot, a.cb, tid, late[tid >> 5], red);
+        else general = true;
+    }
+    if (!general) return;
+    block_sync();
+    const SmemPlan &p = a.plan;
+    int *ctl = (int *)(sm + p.ctl_off);
+    unsigned long long *lslot = (unsigned long long *)(sm + p.slot_off);
+    int *used = (int *)(sm + p.used_off);
+    for (int i = tid; i < p.cap; i += CB_THREADS) lslot[i] = 0ull;
+    if (tid < 2) ctl[tid] = 0;
+    block_sync();
+    const SmemTable tb{lslot, used, &ctl[0], &ctl[1], p.cap, p.max_used};
+    for (long long i = b; i < nlong; i += G)
+        if (a.lng[i].m > most)
+            count_run_general(a.x, a.lng[i], tb, tid, CB_THREADS, (unsigned long long *)(sm + p.red_off));
+}
+
 // Runs longer than the block tables of k_count hold at 3/4 load (and any run
 // of 2^24 entries or more), one block each, with 64-bit counts
 // (count_run_general).
@@ -1415,6 +1573,9 @@ void prepare_kernels()
     cudaFuncSetAttribute(k_count<EpochTable32V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count<EpochTable, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count<EpochTable32V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
+    cudaFuncSetAttribute(k_count_big<CT_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM);
+    cudaFuncSetAttribute(k_count_big<CT_ABOVE>, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM);
+    cudaFuncSetAttribute(k_count_big<CT_FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM);
     cudaFuncSetAttribute(k_count_long, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
@@ -1860,8 +2021,18 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     const CountPlan cp = plan_count(sh.threads, sh.smem_bytes);
     const bool sorted = sh.algo == ALGO_SORT;
     const SortPlan sp = plan_sort(sh.threads, sh.smem_bytes);
+    // phase B: one-word tables (qm_count.cuh) while the ids leave room for the
+    // repeats in a word, else the two-word or 64-bit tables of k_count
+    const bool tab = !sorted && K < CT_MAX_K;
+    const int cb = ct_count_bits(K);
+    const int most = tab ? (int)std::min<long long>(INT_MAX, (1LL << cb) - 1) : 0;
     TRACE("k_classify");
-    if (sorted)  // warps sort runs up to SORT_WARP_CAP, blocks up to their buffers
+    if (tab)
+        k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
+            ws.start, ws.aoff, packed_len, K, std::min(CT_FILL_WARP, most), std::min(CT_FILL_GROUP, most),
+            std::min(CB_FILL, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
+            half ? ws.inter : nullptr);
+    else if (sorted)  // warps sort runs up to SORT_WARP_CAP, blocks up to their buffers
         k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(ws.start, ws.aoff, packed_len, K, SORT_WARP_CAP,
                                                                 SORT_WARP_CAP, sp.cap, ws.hdr_big, ws.hdr_small,
                                                                 ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
@@ -1891,7 +2062,31 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     const int count_grid = community_grid(K, num_sms, sh);  // sh.blocks_per_sm: occupancy resolved by the caller
     // S_c of every community only when its per-community Qds term is asked for
     a.x.full = (pc && pc->qds) ? 1 : 0;
-    if (sorted) {
+    if (tab) {
+        CountTabArgs t;
+        t.x = a.x;
+        t.mid = ws.hdr_mid;
+        t.small = ws.hdr_small;
+        t.big = ws.hdr_big;
+        t.lng = ws.hdr_long;
+        t.counters = ws.counters;
+        t.status = ws.status;
+        t.cb = cb;
+        t.stage_wait = a.stage_wait;
+        t.plan = plan_smem(CB_THREADS, CB_SMEM);
+        const int tg = (int)std::min<long long>((long long)num_sms * CT_BLOCKS, K), bg = std::min(2 * num_sms, K);
+        TRACE("k_count_tab");
+        // the binned gathers pack every label, the others only those counted
+        const int mode = a.x.full ? CT_FULL : ws.bin_pool ? CT_MIXED : CT_ABOVE;
+        TRACE("k_count_tab");
+        if (mode == CT_FULL) k_count_tab<CT_FULL><<<tg, CT_THREADS, 0, s>>>(t);
+        else if (mode == CT_ABOVE) k_count_tab<CT_ABOVE><<<tg, CT_THREADS, 0, s>>>(t);
+        else k_count_tab<CT_MIXED><<<tg, CT_THREADS, 0, s>>>(t);
+        TRACE("k_count_big");
+        if (mode == CT_FULL) k_count_big<CT_FULL><<<bg, CB_THREADS, CB_SMEM, s>>>(t);
+        else if (mode == CT_ABOVE) k_count_big<CT_ABOVE><<<bg, CB_THREADS, CB_SMEM, s>>>(t);
+        else k_count_big<CT_MIXED><<<bg, CB_THREADS, CB_SMEM, s>>>(t);
+    } else if (sorted) {
         CountSortArgs sa;
         sa.x = a.x;
         sa.big = ws.hdr_big;
@@ -1914,9 +2109,11 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
         if (a.x.full) k_count<EpochTable, true><<<count_grid, sh.threads, sh.smem_bytes, s>>>(a);
         else k_count<EpochTable, false><<<count_grid, sh.threads, sh.smem_bytes, s>>>(a);
     }
-    TRACE("k_count_long");
-    k_count_long<<<std::min(num_sms, K), 1024, MAX_DYN_SMEM, s>>>(a.x, ws.hdr_long, ws.counters, plan_smem(1024, MAX_DYN_SMEM),
-                                                      ws.status);
+    if (!tab) {
+        TRACE("k_count_long");
+        k_count_long<<<std::min(num_sms, K), 1024, MAX_DYN_SMEM, s>>>(a.x, ws.hdr_long, ws.counters,
+                                                                      plan_smem(1024, MAX_DYN_SMEM), ws.status);
+    }
     launches += 2;
     PerCommDev pcd{};
     if (pc) pcd = *pc;
