@@ -549,6 +549,42 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned pari
     return false;
 }
 
+// ---------------------------------------------------------------- community volumes
+
+// A community's members (above) and arcs (below) in one word: n < 2^31 nodes,
+// fewer than 2^32 arcs.
+constexpr int VOL_BITS = 33;
+constexpr unsigned long long VOL_MASK = (1ull << VOL_BITS) - 1ull;
+
+// Adds the warp's nodes (label l, degree d, `ok` lanes only) to the
+// communities' words: lanes of equal consecutive labels are summed first, so
+// that in an order that follows the communities a warp issues few atomics.
+// All 32 lanes call this.
+__device__ __forceinline__ void vol_add_warp(unsigned long long *cv, int l, unsigned d, bool ok)
+{
+    const int lane = threadIdx.x & 31;
+    const int key = ok ? l : -1;
+    const int key0 = __shfl_sync(0xffffffffu, key, 0);
+    if (__all_sync(0xffffffffu, key >= 0 && key == key0)) {  // one community
+        const unsigned sum = __reduce_add_sync(0xffffffffu, d);
+        if (lane == 0) atomicAdd(&cv[l], (32ull << VOL_BITS) | (unsigned long long)sum);
+        return;
+    }
+    unsigned inc = ok ? d : 0u;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, inc, s);
+        if (lane >= s) inc += t;
+    }
+    const int prev = __shfl_up_sync(0xffffffffu, key, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || key != prev);
+    const unsigned later = heads & ~((2u << lane) - 1u);  // heads after this lane
+    const int end = later ? __ffs(later) - 2 : 31;        // last lane of this lane's stretch
+    const unsigned upto = __shfl_sync(0xffffffffu, inc, end);
+    if (ok && ((heads >> lane) & 1u))
+        atomicAdd(&cv[l], ((unsigned long long)(end - lane + 1) << VOL_BITS) | (unsigned long long)(upto - inc + d));
+}
+
 // ---------------------------------------------------------------- misc
 
 // How many items a warp claims at a time from a shared list of n items when

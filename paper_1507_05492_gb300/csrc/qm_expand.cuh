@@ -61,24 +61,22 @@ __device__ __forceinline__ int ld_label3(const unsigned long long *plab, int v, 
 
 // Block encoding of the labels of a renumbered graph, for the far-end gathers
 // (built per call by k_pack_blocks).  Along the stored node order the labels
-// of a partition that follows the graph's clusters change rarely, so 16
-// consecutive nodes mostly carry one or two labels: one 64-bit word per 16
-// nodes holds labels A ([0, 21)) and B ([21, 42)) and a 16-bit mask ([42, 58))
-// whose bit i selects B for the block's node i.  A block of three or more
-// labels has bit 63 set and, in bits [0, 32), the offset (in 32-bit words from
-// the array's start) of its 16 labels in the exception area after the block
-// words.  Half a byte a node instead of the packed copy's 8/3, so that the
-// whole encoding of 10^8 nodes stays in L2.
+// of a partition that follows the graph's clusters change rarely, so most
+// blocks of 16 consecutive nodes carry one label: one 32-bit word per block
+// holds it.  A block of two labels has its word point (BLK_PAIR) at a 64-bit
+// entry with labels A ([0, 21)) and B ([21, 42)) and a 16-bit mask that selects
+// B; a block of more at a slot of its 16 labels (BLK_SLOT).  The words of 10^8
+// nodes take 25 MB (the packed copy 267 MB), so the encoding stays in L2, and
+// most gathers are one 32-bit load and a sign test.
 constexpr int BLK_NODES = 16;
+constexpr unsigned BLK_SLOT = 0x80000000u, BLK_PAIR = 0xC0000000u, BLK_INDEX = 0x3FFFFFFFu;
 
-__device__ __forceinline__ int ld_label_blk(const unsigned long long *blab, int v, unsigned long long pol)
+// Where the pairs and the slots begin, in 32-bit words from the array's start.
+__host__ __device__ inline unsigned blk_pairs_at(long long n)
 {
-    unsigned long long w;
-    asm("ld.global.nc.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(w) : "l"(blab + ((unsigned)v >> 4)), "l"(pol));
-    const unsigned i = (unsigned)v & 15u;
-    if (!(w >> 63)) return (int)((w >> (((w >> (42u + i)) & 1ull) ? PACK_BITS : 0)) & 0x1FFFFFull);
-    return ld_hint((const int *)blab + ((unsigned)w + i), pol);
+    return (unsigned)(((n + BLK_NODES - 1) / BLK_NODES + 31) / 32 * 32);
 }
+__host__ __device__ inline unsigned blk_slots_at(long long n) { return 3u * blk_pairs_at(n); }
 
 // Label sources of the far-end gathers: the labels as given, the packed copy,
 // or the block encoding.
@@ -113,9 +111,7 @@ __device__ __forceinline__ void expand_range(unsigned e_lo, unsigned e_hi, int c
 #pragma unroll
         for (int k = 0; k < EXPAND_UNROLL; ++k)
             if (lab[k] >= 0)
-                lab[k] = LAB == LAB_BLOCKS  ? ld_label_blk(plab, lab[k], keep)
-                         : LAB == LAB_PACK3 ? ld_label3(plab, lab[k], keep)
-                                            : ld_hint(&labels[lab[k]], keep);
+                lab[k] = LAB == LAB_PACK3 ? ld_label3(plab, lab[k], keep) : ld_hint(&labels[lab[k]], keep);
         if (WT) {
 #pragma unroll
             for (int k = 0; k < EXPAND_UNROLL; ++k)
@@ -161,85 +157,6 @@ __device__ __forceinline__ void flush_weights(unsigned long long *wl, int c, u12
         if (w_out) limbs_add(wl + (size_t)c * 6 + 3, (i128)w_out);
     }
 }
-
-// One warp's share of phase A: the 32 member positions from p0 (fewer at the
-// end), their runs of one community each, and the gathers of those runs'
-// arcs.  offw (33 entries), rsw and cw (32 each) are the warp's shared-memory
-// slices.
-template <bool WT, int LAB, bool HI>
-__device__ __forceinline__ void expand_chunk(long long p0, long long n, const long long *__restrict__ row_ptr,
-                                             const int *__restrict__ col, const int *__restrict__ labels,
-                                             const unsigned long long *__restrict__ plab,
-                                             const int *__restrict__ members, const unsigned *__restrict__ aoff,
-                                             const int *__restrict__ start, int *inter, int *inter_hi,
-                                             int *__restrict__ nbr, Shard own, const float *__restrict__ wt,
-                                             float *__restrict__ nbrw, unsigned long long *wl, unsigned *offw,
-                                             long long *rsw, int *cw, unsigned long long keep, int lane)
-{
-    const int nm = (int)min(32LL, n - p0);
-    const unsigned base = __ldg(&aoff[p0]);
-    int u = -2;
-    if (lane < nm) {
-        u = __ldcs(&members[p0 + lane]);
-        offw[lane] = __ldg(&aoff[p0 + lane]) - base;
-        rsw[lane] = __ldg(&row_ptr[u]);
-        cw[lane] = ld_hint(&labels[u], keep);
-    }
-    if (lane == 0) offw[nm] = __ldg(&aoff[p0 + nm]) - base;
-    __syncwarp();
-    const int u_prev = __shfl_up_sync(0xffffffffu, u, 1);
-    const bool valid = lane < nm;
-    const bool newrun = valid && (lane == 0 || cw[lane] != cw[lane - 1]);
-    unsigned runs = __ballot_sync(0xffffffffu, newrun);
-    const unsigned segs = __ballot_sync(0xffffffffu, newrun || (valid && u != u_prev + 1));
-    int cur_c = -1;
-    unsigned cbase = 0;
-    if (__popc(segs) <= EXPAND_MAX_SEGS) {
-        unsigned rem = segs;
-        while (rem) {
-            const int lo = __ffs(rem) - 1;
-            rem &= rem - 1;
-            const int hi = rem ? __ffs(rem) - 1 : nm;
-            const unsigned e_lo = offw[lo], e_hi = offw[hi];
-            if (e_lo == e_hi) continue;
-            const int c = cw[lo];
-            if (!own.owns(c)) continue;
-            if (c != cur_c) {
-                cur_c = c;
-                if (lane == 0) cbase = __ldg(&aoff[__ldg(&start[c])]);
-                cbase = __shfl_sync(0xffffffffu, cbase, 0);
-            }
-            const long long cs = rsw[lo] - (long long)e_lo;  // CSR index of arc e is cs + e
-            u128 w_in = 0, w_out = 0;
-            expand_range<WT, LAB, HI>(e_lo, e_hi, c, cbase, [cs](unsigned e) { return cs + (long long)e; }, col,
-                                       labels, plab, inter, inter_hi, nbr, keep, lane, wt, nbrw, w_in, w_out);
-            if (WT) flush_weights(wl, c, w_in, w_out, lane);
-        }
-    } else {
-        while (runs) {
-            const int m_lo = __ffs(runs) - 1;
-            runs &= runs - 1;
-            const int m_hi = runs ? __ffs(runs) - 1 : nm;
-            const unsigned e_lo = offw[m_lo], e_hi = offw[m_hi];
-            if (e_lo == e_hi) continue;
-            const int c = cw[m_lo];
-            if (!own.owns(c)) continue;
-            if (lane == 0) cbase = __ldg(&aoff[__ldg(&start[c])]);
-            cbase = __shfl_sync(0xffffffffu, cbase, 0);
-            u128 w_in = 0, w_out = 0;
-            expand_range<WT, LAB, HI>(
-                e_lo, e_hi, c, cbase,
-                [=](unsigned e) {
-                    const int o = m_lo + upper_bound_smem(offw + m_lo, m_hi - m_lo, e) - 1;
-                    return rsw[o] + (long long)(e - offw[o]);
-                },
-                col, labels, plab, inter, inter_hi, nbr, keep, lane, wt, nbrw, w_in, w_out);
-            if (WT) flush_weights(wl, c, w_in, w_out, lane);
-        }
-    }
-    __syncwarp();
-}
-
 
 // ---------------------------------------------------------------- half-edge gathers
 //

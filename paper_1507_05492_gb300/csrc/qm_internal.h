@@ -93,6 +93,8 @@ struct ScoreWs {
     unsigned *aoff;             // two-phase only: [n + 1] arc offsets of member positions
     int *inter;                 // two-phase only: [K] cut arcs of each community (zeroed)
     int *inter_hi;              // two-phase only: [K] packed labels above c of each community (zeroed)
+    unsigned long long *cv = nullptr;    // two-phase, node order: [K] members << 33 | arcs (zeroed)
+    unsigned long long *curs = nullptr;  // two-phase, node order: [K] cut arcs << 32 | packed labels (zeroed)
     qmk::RunHdr *hdr_big;       // two-phase only: [K] run headers for whole blocks
     qmk::RunHdr *hdr_small;     // two-phase only: [K] run headers for single warps
     qmk::RunHdr *hdr_long;      // two-phase only: [K] run headers for k_count_long
@@ -189,10 +191,15 @@ int launch_score(const GraphDev &g, const int *labels, int K, const ScoreWs &ws,
 int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh,
                   const PerCommDev *pc, int num_sms, cudaStream_t s, TraceFn tr, int shard_r = 0,
                   int shard_p = 1, bool sizes_ready = false);
+// Whether the two-phase pipeline of a call walks the rows in stored node order
+// (algorithms 1, 4, 5 and 6, weighted graphs, and 7 where the half-edge pass does
+// not apply) rather than the members in community order.
+bool score_rows(const GraphDev &g, int algo, int shard_p);
 // For a renumbered graph: out[j] = labels[inv[j]] and the community sizes into
-// ws.size (zeroed), with the label range check of k_hist.  Returns 1 or -1.
-int launch_permute_hist(const int *labels, const int *inv, long long n, int *out, int K, const ScoreWs &ws,
-                        int num_sms, cudaStream_t s);
+// ws.size, or (rows) members and arcs into ws.cv (zeroed), with the label range
+// check of k_hist.  Returns 1 or -1.
+int launch_permute_hist(const int *labels, const int *inv, const long long *row_ptr, long long n, int *out, int K,
+                        const ScoreWs &ws, bool rows, int num_sms, cudaStream_t s);
 // k_score_fin on an accumulator array of GS_COUNT words (a combined set of shard
 // partials): status must point at a zero int.  Returns 1 (launches) or -1.
 int launch_score_fin(const unsigned long long *gacc, const int *status, long long n, long long E, qm_quality *out,
@@ -238,10 +245,11 @@ int build_perm_buckets(const int *inv, long long n, int wb, int tb, int num_sms,
 void free_perm_buckets(PermBuckets *pb);
 // out[j] = labels[inv[j]] by the two passes (tmp: n ints), labels outside
 // [0, K) flagged in bit 0 of *status; with `size`, also the community sizes,
-// as k_hist.  Returns launches, 0 when K is too large for the passes' shared
-// memory (nothing launched: gather the labels instead), or -1.
-int launch_permute_buckets(const int *labels, const PermBuckets &pb, long long n, int *tmp, int *out, int *size,
-                           int K, int *status, int num_sms, cudaStream_t s,
+// as k_hist, or with `cv` the members and arcs (from row_ptr, stored order).
+// Returns launches, 0 when K is too large for the passes' shared memory
+// (nothing launched: gather the labels instead), or -1.
+int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long long *row_ptr, long long n, int *tmp,
+                           int *out, int *size, unsigned long long *cv, int K, int *status, int num_sms, cudaStream_t s,
                            void (*tr)(const char *, cudaStream_t) = nullptr);
 // Builds the renumbered CSR (row_ptr, col: new device allocations) and inv
 // (new id -> old id) of g from `rounds` label-propagation rounds.  Returns 0,

@@ -24,7 +24,8 @@ namespace qm {
 using namespace qmk;
 
 enum { C_BIG_COUNT = 0, C_BIG_NEXT = 1, C_SMALL_NEXT = 2, C_OVF_COUNT = 3, C_OVF_NEXT = 4, C_SMALL_COUNT = 5,
-       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_COUNT = 9, C_BX_BAD = 10, C_MID_NEXT = 11 };
+       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_BAD = 9, C_MID_NEXT = 10,
+       C_BX_COUNT = 12 /* two words */ };
 
 constexpr int SCAN_TILE = 4096;   // elements per block in the multi-block scan
 constexpr int SCAN_SINGLE_MAX = 1 << 16;
@@ -793,28 +794,30 @@ __global__ void k_pack3(const int *__restrict__ labels, long long n, unsigned lo
     }
 }
 
-// The block encoding of the labels (ld_label_blk in qm_expand.cuh) in the
+// The block encoding of the labels (see BLK_NODES in qm_expand.cuh) in the
 // buffer of the packed copy, which is larger: a half-warp per block of 16
 // nodes, each warp taking PACKB_UNROLL pairs of blocks a step with all their
-// loads issued first.  Blocks of three or more labels take exception slots
-// (one atomic per warp and block pair; the order is whatever the atomics give)
-// while fewer than xcap are taken; a warp that finds them gone sets *bad and
-// stops (as does every later one that needs a slot), and the packed copy
-// replaces the encoding.
+// loads issued first and one atomic for all the entries the step needs (their
+// order is whatever the atomics give).  A warp that needs a slot of 16 labels
+// when xcap are taken sets *bad and stops (as does every later one), and the
+// packed copy replaces the encoding.  count: slots above, pairs below.
 constexpr int PACKB_UNROLL = 4;
 
-__global__ void k_pack_blocks(const int *__restrict__ labels, long long n, unsigned long long *__restrict__ blab,
-                              long long xcap, int *xcount, int *bad, const int *status)
+__global__ void k_pack_blocks(const int *__restrict__ labels, long long n, unsigned *__restrict__ blab, long long xcap,
+                              unsigned long long *count, int *bad, const int *status)
 {
     if (*status) return;
     const int lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15;
-    const unsigned hmask = 0xFFFFu << (16 * half);
+    const unsigned hmask = 0xFFFFu << (16 * half), before = (1u << (16 * half)) - 1u;
     const long long nb = (n + BLK_NODES - 1) / BLK_NODES;
-    const unsigned xbase = (unsigned)(2 * nb);  // first word of the exception area
+    unsigned long long *const pairs = (unsigned long long *)(blab + blk_pairs_at(n));
+    int *const slots = (int *)blab + blk_slots_at(n);
     const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
     const long long wg = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     for (long long b0 = wg * 2 * PACKB_UNROLL; b0 < nb; b0 += 2 * PACKB_UNROLL * nwarps) {
-        int lv[PACKB_UNROLL];
+        int lv[PACKB_UNROLL], A[PACKB_UNROLL], B[PACKB_UNROLL];
+        unsigned isB[PACKB_UNROLL], m2[PACKB_UNROLL], m3[PACKB_UNROLL];
+        unsigned n2 = 0, n3 = 0;
 #pragma unroll
         for (int q = 0; q < PACKB_UNROLL; ++q) {
             const long long i = (b0 + 2 * q + half) * BLK_NODES + hl;
@@ -823,83 +826,62 @@ __global__ void k_pack_blocks(const int *__restrict__ labels, long long n, unsig
 #pragma unroll
         for (int q = 0; q < PACKB_UNROLL; ++q) {
             const long long b = b0 + 2 * q + half;
-            const bool inb = b < nb, real = inb && b * BLK_NODES + hl < n;
-            int l = lv[q];
-            const int A = __shfl_sync(0xffffffffu, l, 16 * half);
-            if (!real) l = A;  // nodes past the end take the block's first label
-            const unsigned notA = __ballot_sync(0xffffffffu, l != A) & hmask;
-            const int B = __shfl_sync(0xffffffffu, l, notA ? __ffs(notA) - 1 : 16 * half);
-            const bool exc = (__ballot_sync(0xffffffffu, l != A && l != B) & hmask) != 0;
-            const unsigned isB = (__ballot_sync(0xffffffffu, l == B && B != A) & hmask) >> (16 * half);
-            const unsigned need = __ballot_sync(0xffffffffu, hl == 0 && inb && exc);
-            int x0 = 0;
-            if (lane == 0 && need) x0 = atomicAdd(xcount, __popc(need));
-            x0 = __shfl_sync(0xffffffffu, x0, 0);
-            if (need && x0 >= xcap) {  // the slots ran out (here or in another warp): give up the encoding
+            A[q] = __shfl_sync(0xffffffffu, lv[q], 16 * half);
+            if (b * BLK_NODES + hl >= n) lv[q] = A[q];  // nodes past the end take the block's first label
+            const unsigned notA = __ballot_sync(0xffffffffu, lv[q] != A[q]) & hmask;
+            B[q] = __shfl_sync(0xffffffffu, lv[q], notA ? __ffs(notA) - 1 : 16 * half);
+            const unsigned other = __ballot_sync(0xffffffffu, lv[q] != A[q] && lv[q] != B[q]) & hmask;
+            isB[q] = notA >> (16 * half);
+            m2[q] = __ballot_sync(0xffffffffu, hl == 0 && b < nb && notA && !other);
+            m3[q] = __ballot_sync(0xffffffffu, hl == 0 && b < nb && other);
+            n2 += __popc(m2[q]);
+            n3 += __popc(m3[q]);
+        }
+        unsigned i2 = 0, i3 = 0;
+        if (n2 | n3) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(count, ((unsigned long long)n3 << 32) | n2);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            i2 = (unsigned)at;
+            i3 = (unsigned)(at >> 32);
+            if (n3 && (long long)i3 + n3 > xcap) {  // the slots ran out: give up the encoding
                 if (lane == 0) atomicExch(bad, 1);
                 return;
             }
-            const int x = x0 + __popc(need & ((1u << (16 * half)) - 1u));
-            unsigned long long word;
-            if (!exc) {
-                word = (unsigned long long)(A & 0x1FFFFF) | ((unsigned long long)(B & 0x1FFFFF) << PACK_BITS) |
-                       ((unsigned long long)isB << 42);
-            } else {
-                if (x < xcap) {
-                    if (inb) ((int *)blab)[xbase + (unsigned)x * BLK_NODES + hl] = l;
-                } else if (hl == 0 && inb) {
-                    atomicExch(bad, 1);
-                }
-                word = (1ull << 63) | (unsigned long long)(xbase + (unsigned)min((long long)x, xcap) * BLK_NODES);
+        }
+#pragma unroll
+        for (int q = 0; q < PACKB_UNROLL; ++q) {
+            const long long b = b0 + 2 * q + half;
+            const unsigned me = 1u << (16 * half);
+            unsigned word = (unsigned)A[q];
+            if (m3[q] & me) {
+                const unsigned x = i3 + __popc(m3[q] & before);
+                slots[x * BLK_NODES + hl] = lv[q];
+                word = BLK_SLOT | x;
+            } else if (m2[q] & me) {
+                const unsigned x = i2 + __popc(m2[q] & before);
+                if (hl == 0)
+                    pairs[x] = (unsigned long long)(unsigned)A[q] | ((unsigned long long)(unsigned)B[q] << PACK_BITS) |
+                               ((unsigned long long)isB[q] << (2 * PACK_BITS));
+                word = BLK_PAIR | x;
             }
-            if (inb && hl == 0) blab[b] = word;
+            i2 += __popc(m2[q]);
+            i3 += __popc(m3[q]);
+            if (b < nb && hl == 0) blab[b] = word;
         }
     }
 }
 
-// Exception slots of the block encoding: a sixteenth of the blocks, and what
-// the packed copy's buffer leaves after the block words.
+// Slots of the block encoding: a sixth of the blocks (at 10^8 nodes the words,
+// pairs and slots then still take about L2), and what the packed copy's buffer
+// leaves.
 static long long blocks_xcap(long long n)
 {
-    const long long nb = (n + BLK_NODES - 1) / BLK_NODES, words = (n + 2) / 3;
-    return std::max(0LL, std::min(nb / 16, (2 * words - 2 * nb) / BLK_NODES));
+    const long long nb = (n + BLK_NODES - 1) / BLK_NODES, ints = 2 * ((n + 2) / 3);
+    return std::max(0LL, std::min(nb / 6, (ints - (long long)blk_slots_at(n)) / BLK_NODES));
 }
 
-// Phase A (the far-end label gathers) lives in qm_expand.cuh: expand_chunk is one
-// warp's share of it.  LAB is the label source of the gathers; with bx_bad (the
-// block encoding was tried) the LAB_BLOCKS launch runs when it fits and the
-// LAB_PACK3 launch when it does not.  Register budgets: 40 for the block
-// encoding (six resident blocks; its gathers hit L2 and wait on latency), 48
-// for the others (64 with weights).
-
-template <bool WT, int LAB, bool HI>
-__global__ void __launch_bounds__(EXPAND_THREADS, LAB == LAB_BLOCKS ? 6 : WT ? 4 : 5) k_expand(const long long *__restrict__ row_ptr,
-                                                           const int *__restrict__ col,
-                                                           const int *__restrict__ labels,
-                                                           const unsigned long long *__restrict__ plab,
-                                                           const int *__restrict__ members,
-                                                           const unsigned *__restrict__ aoff,
-                                                           const int *__restrict__ start, long long n,
-                                                           int *inter, int *inter_hi, int *__restrict__ nbr,
-                                                           const int *status,
-                                                           Shard own, const float *__restrict__ wt,
-                                                           float *__restrict__ nbrw, unsigned long long *wl,
-                                                           const int *bx_bad = nullptr)
-{
-    __shared__ unsigned offs_s[EXPAND_THREADS / 32][33];
-    __shared__ long long rs_s[EXPAND_THREADS / 32][32];
-    __shared__ int cw_s[EXPAND_THREADS / 32][32];
-    if (*status) return;
-    if (bx_bad && (LAB == LAB_BLOCKS) == (*bx_bad != 0)) return;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned long long keep = l2_policy_evict_last();
-    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long p0 = ((long long)blockIdx.x * (blockDim.x >> 5) + w) * 32; p0 < n; p0 += nwarps * 32)
-        expand_chunk<WT, LAB, HI>(p0, n, row_ptr, col, labels, plab, members, aoff, start, inter, inter_hi, nbr,
-                                   own, wt, nbrw, wl, offs_s[w], rs_s[w], cw_s[w], keep, lane);
-}
-
-// Half-edge phase A (ALGO_HALF): as k_expand over the upper rows; same2 (the
+// Half-edge phase A (ALGO_HALF): members in community order, their upper rows; same2 (the
 // `inter` array) receives 2|E_c^in| and cursor (`inter_hi`) the run lengths.
 template <bool PACK, bool FULL>
 __global__ void __launch_bounds__(EXPAND_THREADS) k_expand_half(const long long *__restrict__ up_ptr,
@@ -933,6 +915,7 @@ __global__ void k_cbase(const int *start, const unsigned *aoff, int K, unsigned 
 }
 
 #include "qm_binned.cuh"
+#include "qm_rows.cuh"
 
 // One header per non-empty community, sorted into four lists by run length
 // m (the community's packed entries, an upper bound on the distinct keys its
@@ -1534,7 +1517,7 @@ __device__ __forceinline__ void flush_score_threads(const ScoreAcc &acc, unsigne
 }
 
 // FP64 terms of every community from the phase-B records, all in parallel.
-__global__ void k_score_terms(const int *start, const unsigned long long *rec, int K, long long E, PerCommDev pc,
+__global__ void k_score_terms(const int *start, const unsigned long long *cv, const unsigned long long *rec, int K, long long E, PerCommDev pc,
                               unsigned long long *g, const int *status, Shard own)
 {
     __shared__ unsigned long long red[72];
@@ -1542,7 +1525,7 @@ __global__ void k_score_terms(const int *start, const unsigned long long *rec, i
     ScoreAcc acc;
     score_acc_zero(acc);
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < K; c += gridDim.x * blockDim.x) {
-        const long long size = start[c + 1] - start[c];
+        const long long size = cv ? (long long)(cv[c] >> VOL_BITS) : start[c + 1] - start[c];
         if (size == 0 || !own.owns(c)) continue;
         double pen, qs, dens, contr, expn, cond;
         const unsigned long long *rc = rec + (size_t)c * REC_WORDS;
@@ -1734,6 +1717,10 @@ ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool w
     p += align_up((size_t)K * 4, 256);
     w.inter_hi = (int *)p;
     p += align_up((size_t)K * 4, 256);
+    w.cv = (unsigned long long *)p;
+    p += align_up((size_t)K * 8, 256);
+    w.curs = (unsigned long long *)p;
+    p += align_up((size_t)K * 8, 256);
     if (weighted) {
         w.wl = (unsigned long long *)p;
         p += align_up((size_t)K * 6 * 8, 256);
@@ -1797,9 +1784,14 @@ ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool w
     return w;
 }
 
-int launch_permute_hist(const int *labels, const int *inv, long long n, int *out, int K, const ScoreWs &ws,
-                        int num_sms, cudaStream_t s)
+int launch_permute_hist(const int *labels, const int *inv, const long long *row_ptr, long long n, int *out, int K,
+                        const ScoreWs &ws, bool rows, int num_sms, cudaStream_t s)
 {
+    if (rows) {
+        k_permute_vol<<<grid_for((n + HIST_UNROLL - 1) / HIST_UNROLL, 256, num_sms, 8), 256, 0, s>>>(
+            labels, inv, row_ptr, n, out, K, ws.cv, ws.status);
+        return cudaGetLastError() == cudaSuccess ? 1 : -1;
+    }
     const int hist_smem = (K <= 12288) ? K * 4 : 0;
     k_permute_hist<<<grid_for(n, 512, num_sms, 8), 512, hist_smem, s>>>(labels, inv, n, out, K, ws.size, ws.status,
                                                                        hist_smem ? 1 : 0);
@@ -1812,14 +1804,8 @@ static int community_grid(long long K, int num_sms, const Shape &sh)
     return (int)std::max<long long>(1, std::min<long long>(resident, K));
 }
 
-// k_expand: 8 blocks per SM, or fewer when the graph has fewer member chunks
-// (32 member positions per warp, EXPAND_THREADS / 32 warps per block).
-// k_expand: per_sm blocks per SM, or fewer when the graph has fewer member
-// chunks.  The gathers from the block encoding (L2-resident, bound by latency)
-// take one wave of resident blocks: each block has an equal grid-stride share,
-// so blocks of a second wave would start late and end the kernel late.  The
-// DRAM-bound gathers from the packed copy keep 8 blocks per SM (measured
-// faster there).
+// Blocks of the phase A kernels: per_sm per SM, or fewer when the graph has
+// fewer chunks (32 nodes per warp, EXPAND_THREADS / 32 warps per block).
 static int expand_grid(long long n, int num_sms, int per_sm = 8)
 {
     const long long per_block = 32LL * (EXPAND_THREADS / 32);
@@ -1827,19 +1813,22 @@ static int expand_grid(long long n, int num_sms, int per_sm = 8)
                                     std::min<long long>((long long)num_sms * per_sm, (n + per_block - 1) / per_block));
 }
 
+// k_rows takes one wave of resident blocks: each block has an equal
+// grid-stride share, so blocks of a second wave would start late and end the
+// kernel late.
 template <bool WT, int LAB, bool HI>
-static int expand_per_sm()
+static void launch_rows(const RowsArgs &a, int num_sms, cudaStream_t s)
 {
-    static std::atomic<int> v{0};
-    if (!v.load()) {
-        int nb = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_expand<WT, LAB, HI>, EXPAND_THREADS, 0);
-        v.store(std::max(1, std::min(nb, 8)));
+    static std::atomic<int> per_sm{0};
+    int nb = per_sm.load();
+    if (!nb) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_rows<WT, LAB, HI>, ROWS_THREADS, 0);
+        per_sm.store(nb = std::max(1, nb));
     }
-    return v.load();
+    k_rows<WT, LAB, HI><<<expand_grid(a.n, num_sms, nb), ROWS_THREADS, 0, s>>>(a);
 }
 
-// Weighted graphs after k_expand<true>: one block per community counts and
+// Weighted graphs after k_rows<true>: one block per community counts and
 // forms the weighted pair sums, then the weighted terms and the result.
 
 static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, const PerCommDev *pc, int num_sms,
@@ -1858,11 +1847,12 @@ static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, con
     TRACE("k_count_w");
     k_count_w<<<(int)std::min<long long>((long long)num_sms * g_count_w_blocks_per_sm, K), COUNT_W_THREADS,
                 COUNT_W_SMEM, s>>>(
-        x, ws.nbrw, ws.recw, plan_smem(COUNT_W_THREADS, COUNT_W_SMEM), ws.status, own);
+        x, ws.nbrw, ws.recw, ws.cv, (const unsigned *)ws.cursor, ws.curs, plan_smem(COUNT_W_THREADS, COUNT_W_SMEM),
+        ws.status, own);
     PerCommDev pcd{};
     if (pc) pcd = *pc;
     TRACE("k_score_terms_w");
-    k_score_terms_w<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(ws.start, ws.rec, ws.recw, ws.wl, K, g.n_arcs / 2,
+    k_score_terms_w<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(ws.cv, ws.rec, ws.recw, ws.wl, K, g.n_arcs / 2,
                                                                  g.w_lo, g.w_hi, pcd, ws.gacc, ws.status, own);
     launches += 2;
     if (own.p == 1) {
@@ -1874,9 +1864,94 @@ static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, con
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
-// The two-phase plain scoring pipeline (see k_expand / count_community):
+bool score_rows(const GraphDev &g, int algo, int shard_p)
+{
+    if (g.wt) return algo != 0;
+    return algo != 0 && !bin_mode_of(algo, false) && !(algo == ALGO_HALF && g.up_ptr && shard_p == 1);
+}
+
+// Phase A in stored node order: volumes (unless the label permutation has
+// counted them), segment bases, the walk.  Returns its launches.
+static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh, bool hi,
+                             int num_sms, cudaStream_t s, TraceFn tr, Shard own, bool sizes_ready)
+{
+    int launches = 0;
+    const long long n = g.n;
+    if (!sizes_ready) {
+        const int smem = K <= 6144 ? K * 8 : 0;  // two words an id within 48 KB
+        TRACE("k_hist_vol");
+        k_hist_vol<<<grid_for((n + HIST_UNROLL - 1) / HIST_UNROLL, 256, num_sms, 8), 256, smem, s>>>(
+            labels, g.row_ptr, n, K, ws.cv, ws.status, smem ? 1 : 0);
+        ++launches;
+    }
+    const int tiles = (K + VSCAN_TILE - 1) / VSCAN_TILE;
+    unsigned *base = (unsigned *)ws.cursor, *sums = (unsigned *)ws.scan_tmp;
+    if (tiles > 1) {
+        TRACE("k_vscan_tiles");
+        k_vscan_tiles<<<tiles, VSCAN_THREADS, 0, s>>>(ws.cv, K, sums, ws.status);
+        ++launches;
+    }
+    TRACE("k_vscan_apply");
+    k_vscan_apply<<<tiles, VSCAN_THREADS, 0, s>>>(ws.cv, K, sums, base, ws.recip, ws.status);
+    ++launches;
+    RowsArgs a;
+    a.row_ptr = g.row_ptr;
+    a.col = g.col;
+    a.labels = labels;
+    a.plab = ws.plab;
+    a.n = n;
+    a.base = base;
+    a.curs = ws.curs;
+    a.nbr = ws.nbr;
+    a.status = ws.status;
+    a.bx_bad = nullptr;
+    a.own = own;
+    a.wt = g.wt;
+    a.nbrw = ws.nbrw;
+    a.wl = ws.wl;
+    if (g.wt) {
+        TRACE("k_rows");
+        launch_rows<true, LAB_PLAIN, false>(a, num_sms, s);
+        return launches + 1;
+    }
+    // on a renumbered graph above BLOCKS_MIN_NODES nodes (any size with
+    // algorithm 4) the block encoding is tried first (the packed copy, in the
+    // same buffer, only when it does not fit)
+    const bool blocks = ws.plab && g.inv && label_blocks(sh.algo, n) && blocks_xcap(n) > 0;
+    int *const bx_bad = blocks ? &ws.counters[C_BX_BAD] : nullptr;
+    a.bx_bad = bx_bad;
+    if (blocks) {
+        TRACE("k_pack_blocks");
+        const long long nb = (n + BLK_NODES - 1) / BLK_NODES;
+        k_pack_blocks<<<grid_for((nb + 2 * PACKB_UNROLL - 1) / (2 * PACKB_UNROLL) * 32, 256, num_sms, 8), 256, 0, s>>>(
+            labels, n, (unsigned *)ws.plab, blocks_xcap(n), (unsigned long long *)&ws.counters[C_BX_COUNT], bx_bad,
+            ws.status);
+        ++launches;
+    }
+    if (ws.plab) {
+        TRACE("k_pack3");
+        k_pack3<<<grid_for((n + 2) / 3, 256, num_sms, 8), 256, 0, s>>>(labels, n, ws.plab, ws.status, bx_bad);
+        ++launches;
+    }
+    TRACE("k_rows");
+    if (blocks) {
+        if (hi) launch_rows<false, LAB_BLOCKS, true>(a, num_sms, s);
+        else launch_rows<false, LAB_BLOCKS, false>(a, num_sms, s);
+        ++launches;
+    }
+    if (ws.plab && hi) launch_rows<false, LAB_PACK3, true>(a, num_sms, s);
+    else if (ws.plab) launch_rows<false, LAB_PACK3, false>(a, num_sms, s);
+    else if (hi) launch_rows<false, LAB_PLAIN, true>(a, num_sms, s);
+    else launch_rows<false, LAB_PLAIN, false>(a, num_sms, s);
+    return launches + 1;
+}
+
+// The two-phase plain scoring pipeline:
+//   k_hist_vol -> k_vscan_* (segment bases) -> k_rows
+//   -> k_rows_classify -> k_count_* -> k_score_terms -> k_score_fin
+// or, for the half-edge and binned gathers, members in community order:
 //   k_hist -> scan (sizes) -> k_scatter_deg -> scan (member degrees = arc offsets)
-//   -> k_expand -> k_classify -> k_count -> k_score_terms -> k_score_fin
+//   -> k_expand_half / k_expand_bin -> k_classify -> ...
 int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh,
                   const PerCommDev *pc, int num_sms, cudaStream_t s, TraceFn tr, int shard_r, int shard_p,
                   bool sizes_ready)
@@ -1884,32 +1959,33 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     int launches = 0;
     const Shard own{shard_r, shard_p};
     const long long n = g.n;
-    if (!sizes_ready) {
-        const int hist_smem = (K <= 12288) ? K * 4 : 0;
-        TRACE("k_hist");
-        k_hist<<<grid_for(n, 512, num_sms, 4), 512, hist_smem, s>>>(labels, K, ws.size, nullptr, 0, nullptr, n,
-                                                                    ws.status, hist_smem ? 1 : 0);
+    const bool rows = score_rows(g, sh.algo, shard_p);
+    // without per-community Qds terms each unordered pair of communities is
+    // counted by its smaller id only, so only the labels above c are packed
+    const bool hi = !(pc && pc->qds) && !g.wt;
+    const int *packed_len = ws.inter;  // entries of each community's packed run (member order)
+    const bool half = !rows && sh.algo == ALGO_HALF;
+    if (rows) {
+        launches += launch_phase_rows(g, labels, K, ws, sh, hi, num_sms, s, tr, own, sizes_ready);
+        if (g.wt) return launch_weighted_tail(g, K, ws, pc, num_sms, s, tr, own, launches);
+    } else {
+        if (!sizes_ready) {
+            const int hist_smem = (K <= 12288) ? K * 4 : 0;
+            TRACE("k_hist");
+            k_hist<<<grid_for(n, 512, num_sms, 4), 512, hist_smem, s>>>(labels, K, ws.size, nullptr, 0, nullptr, n,
+                                                                        ws.status, hist_smem ? 1 : 0);
+            ++launches;
+        }
+        launches += launch_scan(ws.size, K, ws.start, ws.cursor, ws.recip, INT_MAX, nullptr, ws.counters,
+                                ws.scan_tmp, ws.status, s, tr);
+        TRACE("k_scatter_deg");
+        k_scatter_deg<<<grid_for(n, 512, num_sms, 8), 512, 0, s>>>(labels, g.row_ptr, n, ws.cursor, ws.members,
+                                                                   (int *)ws.aoff, ws.status);
         ++launches;
+        // exclusive prefix of the member degrees, in place: aoff[p] = arcs before member position p
+        launches += launch_scan((const int *)ws.aoff, (int)n, (int *)ws.aoff, nullptr, nullptr, INT_MAX, nullptr,
+                                ws.counters, ws.scan_tmp, ws.status, s, tr);
     }
-    launches += launch_scan(ws.size, K, ws.start, ws.cursor, ws.recip, INT_MAX, nullptr, ws.counters,
-                            ws.scan_tmp, ws.status, s, tr);
-    TRACE("k_scatter_deg");
-    k_scatter_deg<<<grid_for(n, 512, num_sms, 8), 512, 0, s>>>(labels, g.row_ptr, n, ws.cursor, ws.members,
-                                                               (int *)ws.aoff, ws.status);
-    ++launches;
-    // exclusive prefix of the member degrees, in place: aoff[p] = arcs before member position p
-    launches += launch_scan((const int *)ws.aoff, (int)n, (int *)ws.aoff, nullptr, nullptr, INT_MAX, nullptr,
-                            ws.counters, ws.scan_tmp, ws.status, s, tr);
-    if (g.wt) {
-        TRACE("k_expand");
-        k_expand<true, LAB_PLAIN, false><<<expand_grid(n, num_sms), EXPAND_THREADS, 0, s>>>(g.row_ptr, g.col, labels, nullptr, ws.members, ws.aoff,
-                                                              ws.start, n, ws.inter, nullptr, ws.nbr, ws.status, own, g.wt,
-                                                              ws.nbrw, ws.wl);
-        ++launches;
-        return launch_weighted_tail(g, K, ws, pc, num_sms, s, tr, own, launches);
-    }
-    const int *packed_len = ws.inter;  // entries of each community's packed run
-    const bool half = sh.algo == ALGO_HALF && g.up_ptr && shard_p == 1 && !ws.bin_pool;
     if (half) {
         // each undirected edge gathered once, from its lower end; the scatter
         // cursors are free now and take the segment bases
@@ -1939,7 +2015,7 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
                                                           ws.inter, ws.inter_hi, ws.nbr, ws.status);
         ++launches;
         packed_len = ws.inter_hi;
-    } else if (ws.bin_pool) {
+    } else if (!rows) {
         BinArgs ba;
         ba.pool = ws.bin_pool;
         ba.list = ws.bin_list;
@@ -1959,64 +2035,6 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
         TRACE("k_resolve");
         k_resolve<<<num_sms * 8, RESOLVE_THREADS, 0, s>>>(ba, labels, ws.inter, ws.nbr, ws.status);
         launches += 3;
-    } else {
-        // without per-community Qds terms each unordered pair of communities is
-        // counted by its smaller id only, so only the labels above c are packed
-        const bool hi = !(pc && pc->qds);
-        const dim3 eg(expand_grid(n, num_sms)), eb(EXPAND_THREADS);
-        // on a renumbered graph above BLOCKS_MIN_NODES nodes (any size with
-        // algorithm 4) the block encoding is tried first (the packed copy, in
-        // the same buffer, only when it does not fit)
-        const bool blocks = ws.plab && g.inv && label_blocks(sh.algo, n);
-        int *const bx_bad = blocks ? &ws.counters[C_BX_BAD] : nullptr;
-        if (blocks) {
-            TRACE("k_pack_blocks");
-            const long long nb = (n + BLK_NODES - 1) / BLK_NODES;
-            k_pack_blocks<<<grid_for((nb + 2 * PACKB_UNROLL - 1) / (2 * PACKB_UNROLL) * 32, 256, num_sms, 8), 256, 0,
-                            s>>>(
-                labels, n, ws.plab, blocks_xcap(n), &ws.counters[C_BX_COUNT], bx_bad, ws.status);
-            ++launches;
-        }
-        if (ws.plab) {
-            TRACE("k_pack3");
-            k_pack3<<<grid_for((n + 2) / 3, 256, num_sms, 8), 256, 0, s>>>(labels, n, ws.plab, ws.status, bx_bad);
-            ++launches;
-        }
-        TRACE("k_expand");
-        if (blocks) {
-            if (hi)
-                k_expand<false, LAB_BLOCKS, true><<<expand_grid(n, num_sms, expand_per_sm<false, LAB_BLOCKS, true>()),
-                                                    eb, 0, s>>>(g.row_ptr, g.col, labels, ws.plab, ws.members,
-                                                                    ws.aoff, ws.start, n, ws.inter, ws.inter_hi,
-                                                                    ws.nbr, ws.status, own, nullptr, nullptr,
-                                                                    nullptr, bx_bad);
-            else
-                k_expand<false, LAB_BLOCKS, false><<<expand_grid(n, num_sms,
-                                                                 expand_per_sm<false, LAB_BLOCKS, false>()),
-                                                     eb, 0, s>>>(g.row_ptr, g.col, labels, ws.plab, ws.members,
-                                                                     ws.aoff, ws.start, n, ws.inter, nullptr, ws.nbr,
-                                                                     ws.status, own, nullptr, nullptr, nullptr,
-                                                                     bx_bad);
-            ++launches;
-        }
-        if (ws.plab && hi)
-            k_expand<false, LAB_PACK3, true><<<eg, eb, 0, s>>>(g.row_ptr, g.col, labels, ws.plab, ws.members,
-                                                               ws.aoff, ws.start, n, ws.inter, ws.inter_hi, ws.nbr,
-                                                               ws.status, own, nullptr, nullptr, nullptr, bx_bad);
-        else if (ws.plab)
-            k_expand<false, LAB_PACK3, false><<<eg, eb, 0, s>>>(g.row_ptr, g.col, labels, ws.plab, ws.members,
-                                                                ws.aoff, ws.start, n, ws.inter, nullptr, ws.nbr,
-                                                                ws.status, own, nullptr, nullptr, nullptr, bx_bad);
-        else if (hi)
-            k_expand<false, LAB_PLAIN, true><<<eg, eb, 0, s>>>(g.row_ptr, g.col, labels, nullptr, ws.members, ws.aoff,
-                                                           ws.start, n, ws.inter, ws.inter_hi, ws.nbr, ws.status,
-                                                           own, nullptr, nullptr, nullptr);
-        else
-            k_expand<false, LAB_PLAIN, false><<<eg, eb, 0, s>>>(g.row_ptr, g.col, labels, nullptr, ws.members,
-                                                            ws.aoff, ws.start, n, ws.inter, nullptr, ws.nbr,
-                                                            ws.status, own, nullptr, nullptr, nullptr);
-        ++launches;
-        packed_len = hi ? ws.inter_hi : ws.inter;
     }
     const CountPlan cp = plan_count(sh.threads, sh.smem_bytes);
     const bool sorted = sh.algo == ALGO_SORT;
@@ -2027,7 +2045,15 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     const int cb = ct_count_bits(K);
     const int most = tab ? (int)std::min<long long>(INT_MAX, (1LL << cb) - 1) : 0;
     TRACE("k_classify");
-    if (tab)
+    if (rows) {
+        // run classes: the count's tables, or (sorted) SORT_WARP_CAP and the blocks' buffers
+        const int wf = tab ? std::min(CT_FILL_WARP, most) : sorted ? SORT_WARP_CAP : cp.fill_w;
+        const int gf = tab ? std::min(CT_FILL_GROUP, most) : sorted ? SORT_WARP_CAP : cp.fill_g;
+        const int bf = tab ? std::min(CB_FILL, most) : sorted ? sp.cap : cp.fill;
+        k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
+            ws.cv, (const unsigned *)ws.cursor, ws.curs, K, wf, gf, bf, ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid,
+            ws.inter, ws.counters, ws.status, own);
+    } else if (tab)
         k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
             ws.start, ws.aoff, packed_len, K, std::min(CT_FILL_WARP, most), std::min(CT_FILL_GROUP, most),
             std::min(CB_FILL, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
@@ -2118,7 +2144,7 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     PerCommDev pcd{};
     if (pc) pcd = *pc;
     TRACE("k_score_terms");
-    k_score_terms<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(ws.start, ws.rec, K, g.n_arcs / 2, pcd, ws.gacc,
+    k_score_terms<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(ws.start, rows ? ws.cv : nullptr, ws.rec, K, g.n_arcs / 2, pcd, ws.gacc,
                                                                ws.status, own);
     ++launches;
     if (shard_p == 1) {  // a shard's caller reads the partial sums instead

@@ -525,7 +525,8 @@ __global__ void k_pb_tile(const int *__restrict__ labels, const unsigned short *
                           int ntiles, int K, int *__restrict__ tmp, int *status);
 template <int B, bool V4>
 __global__ void k_pb_window(const int *__restrict__ tmp, const unsigned short *__restrict__ dloc, long long n, int wb,
-                            int nw, int *__restrict__ out, int *size, int K);
+                            int nw, int *__restrict__ out, int *size, int K, const long long *__restrict__ row_ptr,
+                            unsigned long long *cv);
 
 template <int B, bool V4>
 static cudaError_t pb_set_smem_v(size_t smem_max)
@@ -729,11 +730,13 @@ __global__ void __launch_bounds__(PB_THREADS, 2) k_pb_tile(const int *__restrict
 
 // Pass 2, one window per block step: slots into shared memory at their new
 // ids, then the window out in order.  With `size`, the labels are counted as
-// k_hist does (pass 1 has checked them).
+// k_hist does, with `cv` as k_hist_vol does (pass 1 has checked them).
 template <int B, bool V4>
-__global__ void __launch_bounds__(PB_THREADS, 2) k_pb_window(const int *__restrict__ tmp,
+__global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restrict__ tmp,
                                                           const unsigned short *__restrict__ dloc, long long n,
-                                                          int wb, int nw, int *__restrict__ out, int *size, int K)
+                                                          int wb, int nw, int *__restrict__ out, int *size, int K,
+                                                          const long long *__restrict__ row_ptr,
+                                                          unsigned long long *cv)
 {
     extern __shared__ __align__(16) unsigned char smb[];
     const int T = blockDim.x, tid = threadIdx.x;
@@ -743,16 +746,27 @@ __global__ void __launch_bounds__(PB_THREADS, 2) k_pb_window(const int *__restri
         bool unused = false;
         pb_stage<B, V4>(tmp + base, dloc + base, len, smb, INT_MAX, unused);
         __syncthreads();
-        for (int i = tid; i - (tid & 31) < len; i += T) {  // warp-uniform trip count
-            const bool in = i < len;
-            const int l = in ? pb_get<B>(smb, i) : 0;
-            if (in) out[base + i] = l;
-            if (size) {
-                const bool ok = in && (unsigned)l < (unsigned)K;
-                const unsigned act = __ballot_sync(0xffffffffu, ok);
-                if (ok) {
-                    const unsigned peers = __match_any_sync(act, l);
-                    if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&size[l], __popc(peers));
+        for (int i0 = tid; i0 - (tid & 31) < len; i0 += T * PB_UNROLL) {  // warp-uniform trip count
+            int l[PB_UNROLL];
+            unsigned d[PB_UNROLL];
+#pragma unroll
+            for (int q = 0; q < PB_UNROLL; ++q) {
+                const int i = i0 + q * T;
+                l[q] = i < len ? pb_get<B>(smb, i) : -1;
+                d[q] = cv && i < len ? (unsigned)(__ldg(&row_ptr[base + i + 1]) - __ldg(&row_ptr[base + i])) : 0u;
+                if (i < len) out[base + i] = l[q];
+            }
+#pragma unroll
+            for (int q = 0; q < PB_UNROLL; ++q) {
+                const bool ok = (unsigned)l[q] < (unsigned)K;
+                if (cv) {
+                    vol_add_warp(cv, l[q], d[q], ok);
+                } else if (size) {
+                    const unsigned act = __ballot_sync(0xffffffffu, ok);
+                    if (ok) {
+                        const unsigned peers = __match_any_sync(act, l[q]);
+                        if ((threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&size[l[q]], __popc(peers));
+                    }
                 }
             }
         }
@@ -760,8 +774,8 @@ __global__ void __launch_bounds__(PB_THREADS, 2) k_pb_window(const int *__restri
     }
 }
 
-int launch_permute_buckets(const int *labels, const PermBuckets &pb, long long n, int *tmp, int *out, int *size,
-                           int K, int *status, int num_sms, cudaStream_t s, void (*tr)(const char *, cudaStream_t))
+int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long long *row_ptr, long long n, int *tmp,
+                           int *out, int *size, unsigned long long *cv, int K, int *status, int num_sms, cudaStream_t s, void (*tr)(const char *, cudaStream_t))
 {
     const bool narrow = K <= (1 << 24);
     const int B = narrow ? 3 : 4;
@@ -775,7 +789,7 @@ int launch_permute_buckets(const int *labels, const PermBuckets &pb, long long n
     auto pass1 = [&](auto kern) {
         kern<<<g1, PB_THREADS, p1, s>>>(labels, pb.lpos, pb.toff, pb.tlb, n, pb.tb, pb.nw, pb.ntiles, K, tmp, status);
     };
-    auto pass2 = [&](auto kern) { kern<<<g2, PB_THREADS, p2, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K); };
+    auto pass2 = [&](auto kern) { kern<<<g2, PB_THREADS, p2, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K, row_ptr, cv); };
     if (tr) tr("k_pb_tile", s);
     if (narrow)
         v1 ? pass1(k_pb_tile<3, true>) : pass1(k_pb_tile<3, false>);

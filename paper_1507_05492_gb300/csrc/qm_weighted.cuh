@@ -9,7 +9,7 @@
 //                    - sum_{cj != ci} W_ci,cj / (2W) d_ci,cj ]
 // Weights are float32 (0 or in [2^-20, 2^20)); each is an exact fixed-point
 // integer w * 2^43, so every weight sum below is exact:
-//   - k_expand<true> sums each community's intra-arc weights (2 W_c^in) and
+//   - k_rows<true> sums each community's intra-arc weights (2 W_c^in) and
 //     cut-arc weights (W_c^out) into three-limb integers, and packs the cut
 //     arcs' weights beside their labels;
 //   - k_count_w counts each community's run in the shared-memory table
@@ -198,7 +198,8 @@ __device__ __forceinline__ void count_run_weighted(const CountCtx &x, const floa
 
 // One block per owned non-empty community (grid-stride), whole-block table.
 __global__ void __launch_bounds__(1024) k_count_w(CountCtx x, const float *nbrw, unsigned long long *recw,
-                                                   SmemPlan p, const int *status, Shard own)
+                                                   const unsigned long long *cv, const unsigned *base,
+                                                   const unsigned long long *curs, SmemPlan p, const int *status, Shard own)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     if (*status) return;
@@ -211,17 +212,16 @@ __global__ void __launch_bounds__(1024) k_count_w(CountCtx x, const float *nbrw,
     block_sync();
     const SmemTable tb{slot, used, &ctl[0], &ctl[1], p.cap, p.max_used};
     for (int c = blockIdx.x; c < x.K; c += gridDim.x) {
-        const int s0 = __ldcg(&x.start[c]), s1 = __ldcg(&x.start[c + 1]);
-        if (s1 == s0 || !own.owns(c)) continue;
-        const unsigned a0 = __ldcg(&x.aoff[s0]), vol = __ldcg(&x.aoff[s1]) - a0;
-        const unsigned m = (unsigned)__ldcg(&x.inter[c]);
+        const unsigned long long v = __ldcg(&cv[c]);
+        if ((v >> VOL_BITS) == 0ull || !own.owns(c)) continue;
+        const unsigned a0 = __ldcg(&base[c]), vol = (unsigned)(v & VOL_MASK), m = (unsigned)__ldcg(&curs[c]);
         count_run_weighted(x, nbrw, recw, c, a0, m, vol, tb, threadIdx.x, blockDim.x, red);
     }
 }
 
 // FP64 terms of every owned community from its integers (weighted Eqs. 8-9,
 // unweighted Sec. II-B.3), added in fixed point; Q_w goes to GS_QW.
-__global__ void k_score_terms_w(const int *start, const unsigned long long *rec, const unsigned long long *recw,
+__global__ void k_score_terms_w(const unsigned long long *cv, const unsigned long long *rec, const unsigned long long *recw,
                                 const unsigned long long *wl, int K, long long E, unsigned long long w_lo,
                                 unsigned long long w_hi, PerCommDev pc, unsigned long long *g, const int *status,
                                 Shard own)
@@ -233,7 +233,7 @@ __global__ void k_score_terms_w(const int *start, const unsigned long long *rec,
     i128 qw = 0;
     const double W2 = __dmul_rn(2.0, u128_to_double(((u128)w_hi << 64) | (u128)w_lo));  // 2W * 2^43
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < K; c += gridDim.x * blockDim.x) {
-        const long long size = start[c + 1] - start[c];
+        const long long size = (long long)(cv[c] >> VOL_BITS);
         if (size == 0 || !own.owns(c)) continue;
         const unsigned long long *rc = rec + (size_t)c * REC_WORDS;
         const unsigned long long same = rc[REC_SAME], vol = rc[REC_VOL];
