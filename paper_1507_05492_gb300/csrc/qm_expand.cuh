@@ -144,14 +144,23 @@ __device__ __forceinline__ void expand_range(unsigned e_lo, unsigned e_hi, int c
     }
 }
 
+// Warp total of a value below 2^76 (a lane's sum of a few fixed-point weights
+// below 2^63): three 27-bit chunks, each added by one redux.
+__device__ __forceinline__ u128 warp_sum_u81(u128 v)
+{
+    constexpr unsigned M = (1u << 27) - 1u;
+    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)v & M);
+    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 27) & M);
+    const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 54) & M);
+    return (u128)a + ((u128)b << 27) + ((u128)c << 54);
+}
+
 // Adds a warp's intra and cut weight sums of community c to its limbs (wl:
 // six words per community, intra then cut).
 __device__ __forceinline__ void flush_weights(unsigned long long *wl, int c, u128 w_in, u128 w_out, int lane)
 {
-    for (int d = 16; d > 0; d >>= 1) {
-        w_in += shfl_down_u128(w_in, d);
-        w_out += shfl_down_u128(w_out, d);
-    }
+    w_in = warp_sum_u81(w_in);
+    w_out = warp_sum_u81(w_out);
     if (lane == 0) {
         if (w_in) limbs_add(wl + (size_t)c * 6, (i128)w_in);
         if (w_out) limbs_add(wl + (size_t)c * 6 + 3, (i128)w_out);

@@ -1544,10 +1544,6 @@ __global__ void k_score_terms(const int *start, const unsigned long long *cv, co
 
 #include "qm_weighted.cuh"
 
-// Launch shape of k_count_w (weighted graphs) and its occupancy.
-constexpr int COUNT_W_THREADS = 256, COUNT_W_SMEM = 48 * 1024;
-static int g_count_w_blocks_per_sm = 1;  // set by prepare_kernels
-
 void prepare_kernels()
 {
     cudaFuncSetAttribute(k_score_cm, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
@@ -1562,12 +1558,9 @@ void prepare_kernels()
     cudaFuncSetAttribute(k_count_long, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
-    cudaFuncSetAttribute(k_count_w, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
+    cudaFuncSetAttribute(k_count_w_big, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM);
     cudaFuncSetAttribute(k_expand_bin, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          bin_smem_bytes_per_warp(BIN_MAX) * (EXPAND_THREADS / 32));
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_count_w, COUNT_W_THREADS, COUNT_W_SMEM);
-    g_count_w_blocks_per_sm = nb > 0 ? nb : 1;
     k_fill_log_int<<<(LOGT_MAX + 256) / 256, 256>>>();
     cudaDeviceSynchronize();
 }
@@ -1828,6 +1821,12 @@ static void launch_rows(const RowsArgs &a, int num_sms, cudaStream_t s)
     k_rows<WT, LAB, HI><<<expand_grid(a.n, num_sms, nb), ROWS_THREADS, 0, s>>>(a);
 }
 
+// Longest run of a single warp of k_count_tab: when every community can have a
+// resident block to itself, all but the shortest runs go to blocks, whose four
+// warps share a run's latency (10^4 nodes, 209 communities: k_count_tab 14.3 ->
+// 10.2 us, k_count_w_tab 18.4 -> 12.3 us).
+static int ct_fill_warp(int K, int num_sms) { return K <= num_sms * CT_BLOCKS ? 96 : CT_FILL_WARP; }
+
 // Weighted graphs after k_rows<true>: one block per community counts and
 // forms the weighted pair sums, then the weighted terms and the result.
 
@@ -1844,11 +1843,30 @@ static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, con
     x.K = K;
     x.err = ws.status;
     x.full = 0;
-    TRACE("k_count_w");
-    k_count_w<<<(int)std::min<long long>((long long)num_sms * g_count_w_blocks_per_sm, K), COUNT_W_THREADS,
-                COUNT_W_SMEM, s>>>(
-        x, ws.nbrw, ws.recw, ws.cv, (const unsigned *)ws.cursor, ws.curs, plan_smem(COUNT_W_THREADS, COUNT_W_SMEM),
+    // runs classed as for k_count_tab; from 2^20 label ids on all go to hash classes
+    const int cb = ct_count_bits(K), most = K < CT_MAX_K ? (int)std::min<long long>(INT_MAX, (1LL << cb) - 1) : 0;
+    TRACE("k_classify");
+    k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
+        ws.cv, (const unsigned *)ws.cursor, ws.curs, K, std::min(ct_fill_warp(K, num_sms), most),
+        std::min(CT_FILL_GROUP, most), std::min(CB_FILL_LONG, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.inter, ws.counters,
         ws.status, own);
+    CountWArgs a;
+    a.x = x;
+    a.nbrw = ws.nbrw;
+    a.recw = ws.recw;
+    a.big = ws.hdr_big;
+    a.small = ws.hdr_small;
+    a.lng = ws.hdr_long;
+    a.mid = ws.hdr_mid;
+    a.counters = ws.counters;
+    a.status = ws.status;
+    a.cb = cb;
+    a.plan = plan_smem(CB_THREADS, CB_SMEM);
+    TRACE("k_count_w_tab");
+    k_count_w_tab<<<(int)std::min<long long>((long long)num_sms * 6, K), CT_THREADS, 0, s>>>(a);
+    TRACE("k_count_w_big");
+    k_count_w_big<<<std::min(2 * num_sms, K), CB_THREADS, CB_SMEM, s>>>(a);
+    launches += 2;
     PerCommDev pcd{};
     if (pc) pcd = *pc;
     TRACE("k_score_terms_w");
@@ -2047,7 +2065,7 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     TRACE("k_classify");
     if (rows) {
         // run classes: the count's tables, or (sorted) SORT_WARP_CAP and the blocks' buffers
-        const int wf = tab ? std::min(CT_FILL_WARP, most) : sorted ? SORT_WARP_CAP : cp.fill_w;
+        const int wf = tab ? std::min(ct_fill_warp(K, num_sms), most) : sorted ? SORT_WARP_CAP : cp.fill_w;
         const int gf = tab ? std::min(CT_FILL_GROUP, most) : sorted ? SORT_WARP_CAP : cp.fill_g;
         const int bf = tab ? std::min(CB_FILL, most) : sorted ? sp.cap : cp.fill;
         k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
@@ -2055,8 +2073,8 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
             ws.inter, ws.counters, ws.status, own);
     } else if (tab)
         k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
-            ws.start, ws.aoff, packed_len, K, std::min(CT_FILL_WARP, most), std::min(CT_FILL_GROUP, most),
-            std::min(CB_FILL, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
+            ws.start, ws.aoff, packed_len, K, std::min(ct_fill_warp(K, num_sms), most),
+            std::min(CT_FILL_GROUP, most), std::min(CB_FILL, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
             half ? ws.inter : nullptr);
     else if (sorted)  // warps sort runs up to SORT_WARP_CAP, blocks up to their buffers
         k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(ws.start, ws.aoff, packed_len, K, SORT_WARP_CAP,

@@ -312,26 +312,34 @@ __device__ __forceinline__ void rows_one(const RowsArgs &a, const int *col, cons
 
 // The arcs [0, total) of a chunk whose nodes belong to many communities: each
 // arc's node is tabulated (own), and the lanes of one community take their
-// places with one atomic.
-template <int LAB, bool HI>
-__device__ __forceinline__ void rows_mixed(const RowsArgs &a, const int *col, unsigned total, const unsigned char *own,
-                                           const int *cw, const unsigned *bw, unsigned long long keep, int lane)
+// places with one atomic.  On a weighted graph an arc's table entry is marked
+// when it is cut, for rows_mixed_weights.
+constexpr unsigned char ROWS_CUT = 0x80;
+
+template <bool WT, int LAB, bool HI>
+__device__ __forceinline__ void rows_mixed(const RowsArgs &a, const int *col, const float *wt, unsigned total,
+                                           unsigned char *own, const int *cw, const unsigned *bw,
+                                           unsigned long long keep, int lane)
 {
     const unsigned lt = (1u << lane) - 1u;
     for (unsigned e0 = 0; e0 < total; e0 += 32u * ROWS_MIX_UNROLL) {
         int lab[ROWS_MIX_UNROLL], o[ROWS_MIX_UNROLL];
+        float wv[ROWS_MIX_UNROLL];
         unsigned peers[ROWS_MIX_UNROLL], hm[ROWS_MIX_UNROLL], at[ROWS_MIX_UNROLL];
 #pragma unroll
         for (int k = 0; k < ROWS_MIX_UNROLL; ++k) {
             const unsigned e = e0 + lane + 32u * k;
             lab[k] = e < total ? __ldcs(&col[e]) : -1;
+            if (WT) wv[k] = e < total ? __ldg(&wt[e]) : 0.0f;
             o[k] = e < total ? own[e] : 0;
         }
         far_labels<LAB, ROWS_MIX_UNROLL, true>(a, lab, keep);
 #pragma unroll
         for (int k = 0; k < ROWS_MIX_UNROLL; ++k) {
             const int c = cw[o[k]];
-            const bool cut = lab[k] >= 0 && lab[k] != c && a.own.owns(c), pack = cut && (!HI || lab[k] > c);
+            const bool out = lab[k] >= 0 && lab[k] != c;
+            if (WT && out) own[e0 + lane + 32u * k] |= ROWS_CUT;
+            const bool cut = out && a.own.owns(c), pack = cut && (!HI || lab[k] > c);
             const unsigned cm = __ballot_sync(0xffffffffu, cut);
             hm[k] = __ballot_sync(0xffffffffu, pack);
             peers[k] = __match_any_sync(0xffffffffu, c) & cm;
@@ -344,9 +352,29 @@ __device__ __forceinline__ void rows_mixed(const RowsArgs &a, const int *col, un
 #pragma unroll
         for (int k = 0; k < ROWS_MIX_UNROLL; ++k) {
             const unsigned b = __shfl_sync(0xffffffffu, at[k], peers[k] ? __ffs(peers[k]) - 1 : 0);
-            if (peers[k] && ((hm[k] >> lane) & 1u)) __stcs(&a.nbr[b + __popc(peers[k] & hm[k] & lt)], lab[k]);
+            if (peers[k] && ((hm[k] >> lane) & 1u)) {
+                const unsigned q = b + __popc(peers[k] & hm[k] & lt);
+                __stcs(&a.nbr[q], lab[k]);
+                if (WT) __stcs(&a.nbrw[q], wv[k]);
+            }
         }
     }
+}
+
+// Intra and cut weight sums of a mixed chunk, a lane per node over its arcs
+// [rel, end) (the chunk's weights are in L1 by then), added to its community's
+// limbs.
+__device__ __forceinline__ void rows_mixed_weights(const RowsArgs &a, const float *wt, const unsigned char *own,
+                                                   unsigned rel, unsigned end, int c, bool node)
+{
+    if (!node || rel == end || !a.own.owns(c)) return;
+    u128 w_in = 0, w_out = 0;
+    for (unsigned e = rel; e < end; ++e) {
+        const unsigned long long f = w_fixed(__ldg(&wt[e]));
+        if (own[e] & ROWS_CUT) w_out += f; else w_in += f;
+    }
+    if (w_in) limbs_add(a.wl + (size_t)c * 6, (i128)w_in);
+    if (w_out) limbs_add(a.wl + (size_t)c * 6 + 3, (i128)w_out);
 }
 
 template <bool WT, int LAB, bool HI>
@@ -354,7 +382,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
 {
     __shared__ int cw_s[ROWS_THREADS / 32][32];
     __shared__ unsigned bw_s[ROWS_THREADS / 32][32];
-    __shared__ unsigned char own_s[WT ? 1 : ROWS_THREADS / 32][WT ? 1 : ROWS_OWN_CAP];
+    __shared__ unsigned char own_s[ROWS_THREADS / 32][ROWS_OWN_CAP];
     if (*a.status) return;
     if (a.bx_bad && (LAB == LAB_BLOCKS) == (*a.bx_bad != 0)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -372,7 +400,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
         if (total == 0u) continue;
         const unsigned bs = __ldg(&a.base[c]);
         const int *col = a.col + r0;
-        if (WT || __popc(heads) <= ROWS_MAX_RUNS || total > (unsigned)ROWS_OWN_CAP) {
+        if (__popc(heads) <= ROWS_MAX_RUNS || total > (unsigned)ROWS_OWN_CAP) {
             unsigned rem = heads;
             while (rem) {
                 const int lo = __ffs(rem) - 1;
@@ -394,10 +422,14 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
             const unsigned nxt = __shfl_down_sync(0xffffffffu, rel, 1);
             const unsigned end = lane == 31 ? total : nxt;
             if (lane < nm)
-                for (unsigned e = rel; e < end; ++e) own_s[WT ? 0 : w][WT ? 0 : e] = (unsigned char)lane;
+                for (unsigned e = rel; e < end; ++e) own_s[w][e] = (unsigned char)lane;
             __syncwarp();
-            rows_mixed<LAB, HI>(a, col, total, own_s[WT ? 0 : w], cw_s[w], bw_s[w], keep, lane);
+            rows_mixed<WT, LAB, HI>(a, col, WT ? a.wt + r0 : nullptr, total, own_s[w], cw_s[w], bw_s[w], keep, lane);
             __syncwarp();
+            if (WT) {
+                rows_mixed_weights(a, a.wt + r0, own_s[w], rel, end, c, lane < nm);
+                __syncwarp();
+            }
         }
     }
 }

@@ -12,11 +12,11 @@
 //   - k_rows<true> sums each community's intra-arc weights (2 W_c^in) and
 //     cut-arc weights (W_c^out) into three-limb integers, and packs the cut
 //     arcs' weights beside their labels;
-//   - k_count_w counts each community's run in the shared-memory table
-//     (|E_ci,cj| for every neighbour cj) and then, in a second pass over the
-//     run, adds for every cut arc (weight w, neighbour cj) the exact product
-//     w * |E_ci,cj| * Rcp_cj, so that P_i = sum_j W_ij |E_ij| / |c_j| is a
-//     256-bit integer (scale 2^171);
+//   - k_count_w_tab and k_count_w_big count each community's run in a
+//     shared-memory table (|E_ci,cj| for every neighbour cj) and then, in a
+//     second pass over the run, add for every cut arc (weight w, neighbour cj)
+//     the exact product w * |E_ci,cj| * Rcp_cj, so that
+//     P_i = sum_j W_ij |E_ij| / |c_j| is a 256-bit integer (scale 2^171);
 //   - k_score_terms_w forms the FP64 terms of each community once from these
 //     integers and adds them in fixed point (Q_w into its own accumulator).
 // The six measures of Sec. II-B.3 keep their unweighted counts.
@@ -196,26 +196,248 @@ __device__ __forceinline__ void count_run_weighted(const CountCtx &x, const floa
     }
 }
 
-// One block per owned non-empty community (grid-stride), whole-block table.
-__global__ void __launch_bounds__(1024) k_count_w(CountCtx x, const float *nbrw, unsigned long long *recw,
-                                                   const unsigned long long *cv, const unsigned *base,
-                                                   const unsigned long long *curs, SmemPlan p, const int *status, Shard own)
+// a += x * r for x < 2^64.
+__device__ __forceinline__ void u256_mac64(U256 &a, unsigned long long x, const Rcp &r)
+{
+    const u128 p0 = (u128)x * r.lo, p1 = (u128)x * r.hi;
+    const u128 t = p1 + (unsigned long long)(p0 >> 64);  // below 2^128: (2^64 - 1)^2 + 2^64 - 1
+    asm("add.cc.u64 %0, %0, %4;\n\taddc.cc.u64 %1, %1, %5;\n\taddc.cc.u64 %2, %2, %6;\n\taddc.u64 %3, %3, 0;"
+        : "+l"(a.w[0]), "+l"(a.w[1]), "+l"(a.w[2]), "+l"(a.w[3])
+        : "l"((unsigned long long)p0), "l"((unsigned long long)t), "l"((unsigned long long)(t >> 64)));
+}
+
+// Warp total of a 256-bit sum (valid in every lane): ten 27-bit chunks, each
+// added by one redux.
+__device__ __forceinline__ U256 ct_warp_sum256(const U256 &a)
+{
+    U256 r;
+    u256_zero(r);
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        const int at = 27 * k, w = at / 64, s = at % 64;
+        unsigned long long v = a.w[w] >> s;
+        if (s > 37 && w < 3) v |= a.w[w + 1] << (64 - s);
+        const unsigned long long sum = __reduce_add_sync(0xffffffffu, (unsigned)v & ((1u << 27) - 1u));
+        U256 t;
+        u256_zero(t);
+        t.w[w] = sum << s;
+        if (s > 32 && w < 3) t.w[w + 1] = sum >> (64 - s);
+        u256_add(r, t);
+    }
+    return r;
+}
+
+// Counts community h.c's run (labels nbr[a0 ..), weights nbrw[a0 ..), m entries)
+// with a group of GS threads and the one-word tables of qm_count.cuh: every
+// label's occurrences in a first pass over the run, then every entry's exact
+// share w |E_cj| Rcp_j in a second (the same integer whatever the order).
+// Bound by the instructions of the two passes.  6.5*10^7 cut arcs of 10^7
+// nodes: 2.71 ms for whole blocks on 64-bit tables with a pass to clear them,
+// 1.23 ms so (k_count_w_tab 0.59, k_count_w_big 0.64).
+template <int GS>
+__device__ __forceinline__ void ct_count_run_weighted(const CountCtx &x, const RunHdr &h, const float *nbrw,
+                                                      unsigned long long *recw, unsigned *slot, int cb, int gtid,
+                                                      unsigned *late, unsigned long long *red)
+{
+    constexpr unsigned ALL = 0xffffffffu;
+    const int m = (int)h.m, c = h.c, lane = threadIdx.x & 31;
+    const int *src = x.nbr + h.a0;
+    const float *wsrc = nbrw + h.a0;
+    const unsigned lt = (1u << lane) - 1u, one = 1u << cb;
+    const unsigned lg = ct_slots_log2(h.m), mask = (1u << lg) - 1u, shift = 32u - lg;
+    unsigned counts[3] = {0u, 0u, 0u};  // above c: repeats, twice the occurrences before them, entries
+    unsigned nl = 0;
+    auto follow = [&](unsigned n) {
+        nl -= n;
+        const unsigned key = (unsigned)lane < n ? late[nl + lane] : 0u;
+        const unsigned before = ct_follow(slot, key, mask, shift, cb);
+        if (before && (int)(key - 1u) > c) {
+            counts[0] += 1u;
+            counts[1] += 2u * before;
+        }
+        __syncwarp();
+    };
+    for (int e0 = gtid & ~31; e0 < m; e0 += GS * CT_UNROLL) {
+        int lv[CT_UNROLL];
+        unsigned cur[CT_UNROLL];
+#pragma unroll
+        for (int k = 0; k < CT_UNROLL; ++k) {
+            const int e = e0 + lane + GS * k;
+            lv[k] = e < m ? __ldg(&src[e]) : -1;
+            if (lv[k] >= 0 && !QM_CHK(lv[k], x.K, 6)) lv[k] = -1;
+            counts[2] += lv[k] > c ? 1u : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < CT_UNROLL; ++k) {
+            const unsigned hs = ((unsigned)lv[k] * 0x9E3779B1u) >> shift;
+            cur[k] = lv[k] >= 0 ? atomicCAS(&slot[hs], 0u, (unsigned)lv[k] * one + one) : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < CT_UNROLL; ++k) {
+            const unsigned taken = __ballot_sync(ALL, cur[k] != 0u);
+            if (cur[k] != 0u) late[nl + __popc(taken & lt)] = (unsigned)lv[k] + 1u;
+            nl += __popc(taken);
+        }
+        __syncwarp();
+        while (nl >= 32u) follow(32u);
+    }
+    if (nl) follow(nl);
+    ct_sync<GS>();
+    U256 P;
+    u256_zero(P);
+    for (int e0 = gtid & ~31; e0 < m; e0 += GS * CT_UNROLL) {
+        int lv[CT_UNROLL];
+        float wv[CT_UNROLL];
+        unsigned cnt[CT_UNROLL], hs[CT_UNROLL];
+        Rcp rj[CT_UNROLL];
+#pragma unroll
+        for (int k = 0; k < CT_UNROLL; ++k) {
+            const int e = e0 + lane + GS * k;
+            lv[k] = e < m ? __ldg(&src[e]) : -1;
+            wv[k] = e < m ? __ldcs(&wsrc[e]) : 0.0f;
+            if (lv[k] >= 0 && !QM_CHK(lv[k], x.K, 6)) lv[k] = -1;
+            rj[k] = Rcp{0ull, 0ull};
+            if (lv[k] >= 0) rj[k] = ld_rcp(&x.recip[lv[k]]);
+            hs[k] = ((unsigned)lv[k] * 0x9E3779B1u) >> shift;
+            cnt[k] = 0u;
+        }
+        // every key is in the table: each lane steps on until it meets its own
+        for (unsigned step = 0; step <= mask; ++step) {
+            bool pend = false;
+#pragma unroll
+            for (int k = 0; k < CT_UNROLL; ++k) {
+                if (lv[k] < 0 || cnt[k]) continue;
+                const unsigned v = ((volatile unsigned *)slot)[hs[k]];
+                if ((v >> cb) == (unsigned)lv[k] + 1u) cnt[k] = (v & (one - 1u)) + 1u;
+                else pend = true;
+                hs[k] = (hs[k] + 1u) & mask;
+            }
+            if (!__any_sync(ALL, pend)) break;
+        }
+#pragma unroll
+        for (int k = 0; k < CT_UNROLL; ++k) {
+            const u128 q = (u128)w_fixed(wv[k]) * cnt[k];  // 0 where there is no entry
+            const bool wide = (unsigned long long)(q >> 64) != 0ull;
+            u256_mac64(P, wide ? 0ull : (unsigned long long)q, rj[k]);
+            if (__any_sync(ALL, wide)) {
+                if (wide) u256_mac(P, q, rj[k]);
+                __syncwarp();
+            }
+        }
+    }
+    ct_sync<GS>();
+    for (unsigned i = (unsigned)gtid; i < (1u << lg) / 4u; i += (unsigned)GS)
+        reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) counts[k] = __reduce_add_sync(ALL, counts[k]);
+    P = ct_warp_sum256(P);
+    if (GS > 32) {
+        const int wid = threadIdx.x >> 5;
+        if (lane == 0) {
+            unsigned long long *r = red + 6 * wid;
+            r[0] = ((unsigned long long)counts[2] << 32) | counts[0];
+            r[1] = counts[1];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r[2 + k] = P.w[k];
+        }
+        ct_sync<GS>();
+        if (threadIdx.x == 0)
+            for (int v = 1; v < GS / 32; ++v) {
+                const unsigned long long *r = red + 6 * v;
+                counts[0] += (unsigned)r[0];
+                counts[2] += (unsigned)(r[0] >> 32);
+                counts[1] += (unsigned)r[1];
+                u256_add(P, U256{{r[2], r[3], r[4], r[5]}});
+            }
+    }
+    if (gtid == 0) {
+        unsigned long long *rc = x.rec + (size_t)c * REC_WORDS;
+        rc[REC_SAME] = (unsigned long long)(h.vol - h.m);
+        rc[REC_VOL] = (unsigned long long)h.vol;
+        rc[REC_SLOTS] = (unsigned long long)(counts[2] - counts[0]);
+        rc[REC_CNT2] = (unsigned long long)counts[2] + counts[1];
+        rc[REC_INNER_LO] = rc[REC_INNER_HI] = rc[REC_FULL_LO] = rc[REC_FULL_HI] = 0ull;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) recw[(size_t)c * 4 + k] = P.w[k];
+    }
+    ct_sync<GS>();
+}
+
+struct CountWArgs {
+    CountCtx x;
+    const float *nbrw;
+    unsigned long long *recw;
+    const RunHdr *big, *small, *lng, *mid;
+    int *counters;
+    const int *status;
+    int cb;
+    SmemPlan plan;  // hash-class tables of k_count_w_big
+};
+
+// As k_count_tab.  (The block's second pass re-reads the run from L1 / L2.)
+__global__ void __launch_bounds__(CT_THREADS, 6) k_count_w_tab(CountWArgs a)
+{
+    __shared__ __align__(16) unsigned slot[CT_WORDS];
+    __shared__ unsigned late[CT_THREADS / 32][CT_LATE];
+    __shared__ unsigned long long red[6 * (CT_THREADS / 32)];
+    __shared__ int s_i;
+    if (*a.status) return;
+    constexpr int W = CT_THREADS / 32;
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < CT_WORDS / 4; i += CT_THREADS)
+        reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const int nmid = a.counters[C_MID_COUNT];
+    for (;;) {
+        if (tid == 0) s_i = atomicAdd(&a.counters[C_MID_NEXT], 1);
+        block_sync();
+        const int i = s_i;
+        if (i >= nmid) break;
+        ct_count_run_weighted<CT_THREADS>(a.x, a.mid[i], a.nbrw, a.recw, slot, a.cb, tid, late[wid], red);
+    }
+    const int nsmall = a.counters[C_SMALL_COUNT];
+    const int chunk = claim_chunk(nsmall, (long long)gridDim.x * W);
+    unsigned *const ws = slot + wid * (CT_WORDS / W);
+    for (;;) {
+        int base = 0;
+        if (lane == 0) base = atomicAdd(&a.counters[C_SMALL_NEXT], chunk);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (base >= nsmall) break;
+        const int top = min(nsmall, base + chunk);
+        for (int i = base; i < top; ++i)
+            ct_count_run_weighted<32>(a.x, a.small[i], a.nbrw, a.recw, ws, a.cb, lane, late[wid], red);
+    }
+}
+
+// The longer runs: one table in the block's shared memory up to CB_FILL_LONG
+// entries (and below 2^cb), then hash classes.
+__global__ void __launch_bounds__(CB_THREADS, 2) k_count_w_big(CountWArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
-    if (*status) return;
-    unsigned long long *red = (unsigned long long *)(sm + p.red_off);
-    int *ctl = (int *)(sm + p.ctl_off);
-    unsigned long long *slot = (unsigned long long *)(sm + p.slot_off);
-    int *used = (int *)(sm + p.used_off);
-    for (int i = threadIdx.x; i < p.cap; i += blockDim.x) slot[i] = 0ull;
-    if (threadIdx.x < 2) ctl[threadIdx.x] = 0;
+    __shared__ unsigned late[CB_THREADS / 32][CT_LATE];
+    __shared__ unsigned long long red[6 * (CB_THREADS / 32)];
+    if (*a.status) return;
+    const int nbig = a.counters[C_BIG_COUNT], nlong = a.counters[C_LONG_COUNT], tid = threadIdx.x;
+    const int G = gridDim.x, b = blockIdx.x;
+    if (b >= nbig && b >= nlong) return;
+    unsigned *slot = (unsigned *)sm;
+    for (int i = tid; i < CB_WORDS_LONG / 4; i += CB_THREADS)
+        reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
     block_sync();
-    const SmemTable tb{slot, used, &ctl[0], &ctl[1], p.cap, p.max_used};
-    for (int c = blockIdx.x; c < x.K; c += gridDim.x) {
-        const unsigned long long v = __ldcg(&cv[c]);
-        if ((v >> VOL_BITS) == 0ull || !own.owns(c)) continue;
-        const unsigned a0 = __ldcg(&base[c]), vol = (unsigned)(v & VOL_MASK), m = (unsigned)__ldcg(&curs[c]);
-        count_run_weighted(x, nbrw, recw, c, a0, m, vol, tb, threadIdx.x, blockDim.x, red);
+    for (int i = b; i < nbig; i += G)
+        ct_count_run_weighted<CB_THREADS>(a.x, a.big[i], a.nbrw, a.recw, slot, a.cb, tid, late[tid >> 5], red);
+    if (b >= nlong) return;
+    const SmemPlan &p = a.plan;
+    int *ctl = (int *)(sm + p.ctl_off);
+    unsigned long long *lslot = (unsigned long long *)(sm + p.slot_off);
+    int *used = (int *)(sm + p.used_off);
+    for (int i = tid; i < p.cap; i += CB_THREADS) lslot[i] = 0ull;
+    if (tid < 2) ctl[tid] = 0;
+    block_sync();
+    const SmemTable tb{lslot, used, &ctl[0], &ctl[1], p.cap, p.max_used};
+    for (int i = b; i < nlong; i += G) {
+        const RunHdr h = a.lng[i];
+        count_run_weighted(a.x, a.nbrw, a.recw, h.c, h.a0, h.m, h.vol, tb, tid, CB_THREADS,
+                           (unsigned long long *)(sm + p.red_off));
     }
 }
 

@@ -52,3 +52,25 @@ def test_many_label_ids(qm, oracle_mod, K, m):
         lab[1:] = ids[np.arange(m) % keys]
         check_quality(qm.score(graph, torch.from_numpy(lab).cuda(), K), oracle_mod.score(rp, col, lab, K),
                       f"K={K} m={m} keys={keys}")
+
+
+@pytest.mark.parametrize("m", [1, 33, 96, 97, 768, 769, 3072, 3073, 12288, 12289])
+def test_weighted_hub_run_lengths(qm, oracle_mod, m):
+    """The weighted count's classes, with weights over the whole accepted range
+    (products beyond 64 bits among them)."""
+    rp, col = star(m)
+    rng = np.random.default_rng(m)
+    leaf = np.exp2(rng.uniform(-20, 19.9, m)).astype(np.float32)
+    leaf[rng.random(m) < 0.1] = 0.0
+    leaf[0] = 1.0
+    w = np.concatenate([leaf, leaf])  # the hub's row, then one arc a leaf
+    graph = qm.Graph(torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda(), weights=w, validate=True)
+    for keys in sorted({1, min(m, 3), max(1, m // 2), m}):
+        lab = np.zeros(m + 1, np.int32)
+        lab[1:] = 1 + np.arange(m) % keys
+        o = oracle_mod.score_weighted(rp, col, w.astype(np.float64), lab, keys + 1)
+        q = qm.score(graph, torch.from_numpy(lab).cuda(), keys + 1)
+        for name, cond in (("modularity", "cond_modularity"), ("modularity_density", "cond_modularity_density")):
+            assert abs(q[name] - o[name]) <= 1e-12 * max(abs(o[name]), abs(o[cond])), (m, keys, name)
+        u = oracle_mod.score(rp, col, lab, keys + 1)
+        assert q["n_community_pairs"] == u["n_community_pairs"] and q["pair_count_sq_sum"] == u["pair_count_sq_sum"]
