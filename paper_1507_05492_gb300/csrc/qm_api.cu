@@ -1687,6 +1687,7 @@ static qm_status cover_status(int st)
 {
     if (st & 1) return fail(QM_EINVAL, "a cover's offsets or lists are malformed (lists must be strictly increasing ids in [0, K))");
     if (st & 2) return fail(QM_EOVERFLOW, "a community borders too many distinct communities");
+    if (st & 4) return fail(QM_ETIMEOUT, "a staging copy did not complete within its wait limit");
     if (st) return fail(QM_ECUDA, "device status " + std::to_string(st));
     return QM_OK;
 }
@@ -1707,10 +1708,15 @@ qm_status qm_score_cover(const qm_graph *gc, const int64_t *mptr, const int32_t 
     long long m = 0;
     qm_status st = stage_cover(g->device, mptr, memb, g->n, where, s, stage, &dptr, &dmemb, &m);
     if (st != QM_OK) return st;
-    Lease ws(g_pool.acquire(cover_score_ws_bytes(g->n, m, K), g->device, false));
+    long long runs = cover_run_entries(g->n, g->n_arcs, m, K);
+    Lease ws(g_pool.acquire(cover_score_ws_bytes(g->n, m, K, runs), g->device, false));
+    if (!ws.b && runs) {  // no room for the packed runs: the member lists need less
+        runs = 0;
+        ws.b = g_pool.acquire(cover_score_ws_bytes(g->n, m, K, 0), g->device, false);
+    }
     Lease pin(g_pool.acquire(512, g->device, true));
     if (!ws.b || !pin.b) return fail(QM_ENOMEM, "scratch allocation failed");
-    const CoverWs w = carve_cover_score_ws(ws.ptr(), g->n, m, K);
+    const CoverWs w = carve_cover_score_ws(ws.ptr(), g->n, m, K, runs);
     CK(cudaMemsetAsync(ws.ptr(), 0, w.zero_bytes, s));
     const int L = launch_cover_score(g->d, dptr, dmemb, m, K, w, num_sms_of(g->device), s);
     if (L < 0) return cuda_fail(cudaGetLastError(), "launch_cover_score");

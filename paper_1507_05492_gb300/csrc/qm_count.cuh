@@ -217,7 +217,7 @@ __device__ __forceinline__ void ct_count_run(const CountCtx &x, const RunHdr &h,
     auto label = [&](int e) { return SMEM ? src[e] : __ldcs(&src[e]); };
     int nx[CT_UNROLL];
 #pragma unroll
-    for (int k = 0; k < CT_UNROLL; ++k) nx[k] = label(min(gtid + GS * k, m - 1));
+    for (int k = 0; k < CT_UNROLL; ++k) nx[k] = label(max(0, min(gtid + GS * k, m - 1)));  // (an empty run reads the slack)
     // one step of CT_UNROLL entries a lane from e0 (warp-uniform) on
     auto step = [&](int e0, auto last) {
         constexpr bool LAST = decltype(last)::value;

@@ -8,13 +8,20 @@
 // and a pair of nodes "in the same community" when the two share one.
 //
 // Scoring (Eqs. 8-9, Sec. II-B.3): the cover is brought to the graph's stored
-// order, transposed into member lists, and one block per community walks its
-// members' arcs, testing the far end's list for c, counting the boundary arcs,
-// and counting in a shared-memory table the communities j > c of the far end
-// that the near end is not in (each unordered pair is charged to its smaller
-// id, as in the partition path).  The terms are formed and summed exactly as
-// there (qm_finalize.cuh), so a cover with one community per node gives the
-// partition's bits.
+// order and scored by the partition path's two phases.  k_cover_walk takes the
+// rows in node order; for every arc and every community c of its near end it
+// tests the far end's list for c, counts the arc as cut, and packs into c's run
+// the communities j > c of the far end that the near end is not in (each
+// unordered pair is charged to its smaller id).  A run's segment is sized by
+// the list lengths of its members' neighbours (k_cover_cap).  The counting,
+// the terms and the sums are the partition path's, so a cover with one
+// community per node gives the partition's bits.  Covers whose segments do not
+// fit the scratch (long lists), and ones of 2^20 ids or more, are transposed
+// into member lists and scored by one block per community (k_cover_score).
+// Measured, 10^6 nodes, a tenth of them in two communities: 2.46 ms by member
+// lists, 0.60 by runs (k_cover_walk 0.27, k_cover_cap 0.14, counting 0.07); the
+// walk is bound by the instructions of its rounds (two for most warps), the
+// segment sizes by their atomics.
 //
 // Comparison (Eqs. 1-7): one block per truth community counts the cells
 // |a n b| over its members' found lists; rows and columns add the entropy, F
@@ -26,6 +33,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "qm_batched.h"
 #include "qm_cover.h"
 #include "qm_community.cuh"
 #include "qm_finalize.cuh"
@@ -41,7 +49,8 @@ constexpr int OVL_CAP = 2048;  // overlapping members of one community paired in
 
 // extra accumulator words after the GC_* words of a comparison
 enum { GC_SAME_A_CORR = GC_COUNT, GC_SAME_B_CORR = GC_COUNT + 1, GC_A11_CORR = GC_COUNT + 2, GC_WORDS = GC_COUNT + 3 };
-enum { CC_NEXT_A = 0, CC_NEXT_B = 1, CC_NEXT_C = 2, CC_SCAN = 8 };
+enum { CC_NEXT_A = 0, CC_NEXT_B = 1, CC_NEXT_C = 2, CC_GATE = 3, CC_OLD = 4, CC_LONG = 5, CC_TOTAL = 6 /* two words */,
+       CC_SCAN = 8, CC_RUNS = 16 };
 
 size_t al(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -62,12 +71,23 @@ void carve_side(char *&p, CoverSide &c, long long n, long long m, int K)
 
 }  // namespace
 
-size_t cover_score_ws_bytes(long long n, long long m, int K)
+// Entries of the packed runs' scratch: what covers whose memberships do not
+// follow the degrees need (every arc once per pair of its ends' communities),
+// and a quarter more.
+long long cover_run_entries(long long n, long long n_arcs, long long m, int K)
 {
-    return carve_cover_score_ws(reinterpret_cast<void *>(4096), n, m, K).bytes;
+    if (!cover_runs_ok(K)) return 0;
+    const double r = std::max(1.0, (double)m / (double)n);
+    const double e = 1.25 * (double)n_arcs * r * r + 4096.0;
+    return e < 4.0e9 ? (long long)e : 0;
 }
 
-CoverWs carve_cover_score_ws(void *base, long long n, long long m, int K)
+size_t cover_score_ws_bytes(long long n, long long m, int K, long long run_entries)
+{
+    return carve_cover_score_ws(reinterpret_cast<void *>(4096), n, m, K, run_entries).bytes;
+}
+
+CoverWs carve_cover_score_ws(void *base, long long n, long long m, int K, long long run_entries)
 {
     CoverWs w{};
     char *p = (char *)base;
@@ -82,10 +102,35 @@ CoverWs carve_cover_score_ws(void *base, long long n, long long m, int K)
     p += al((size_t)K * 4);
     w.a.cur = (int *)p;
     p += al((size_t)K * 4);
+    if (run_entries) {
+        w.cv = (unsigned long long *)p;
+        p += al((size_t)K * 8);
+        w.capw = (unsigned long long *)p;
+        p += al((size_t)K * 8);
+        w.curs = (unsigned long long *)p;
+        p += al((size_t)K * 8);
+    }
     w.zero_bytes = (size_t)(p - (char *)base);
     carve_side(p, w.a, n, m, K);
     w.recip = (Rcp *)p;
     p += al((size_t)K * 16);
+    w.run_entries = run_entries;
+    if (run_entries) {
+        w.head = (int *)p;
+        p += al((size_t)n * 4);
+        w.base = (unsigned *)p;
+        p += al((size_t)K * 4);
+        w.inter = (int *)p;
+        p += al((size_t)K * 4);
+        w.rec = (unsigned long long *)p;
+        p += al((size_t)K * REC_WORDS * 8);
+        for (int k = 0; k < 4; ++k) {
+            w.hdr[k] = (RunHdr *)p;
+            p += al((size_t)K * sizeof(RunHdr));
+        }
+        w.nbr = (int *)p;
+        p += al((size_t)run_entries * 4) + 256;
+    }
     w.scan_tmp = (int *)p;
     p += al((scan_tmp_elems(std::max<long long>(n + 1, K)) + 64) * 4);
     w.bytes = (size_t)(p - (char *)base);
@@ -125,6 +170,8 @@ CoverWs carve_cover_compare_ws(void *base, long long n, long long ma, int ka, lo
     p += al((size_t)ka * 4);
     w.rowbest = (unsigned long long *)p;
     p += al((size_t)ka * 8);
+    w.logt = (double *)p;
+    p += al((size_t)LOGT_WORDS * 8);
     w.scan_tmp = (int *)p;
     p += al((scan_tmp_elems(std::max<long long>(n + 1, std::max(ka, kb))) + 64) * 4);
     w.bytes = (size_t)(p - (char *)base);
@@ -155,8 +202,10 @@ __global__ void k_cover_len(const long long *mptr, long long n, long long m, con
 
 // Copies every stored node's list to its new offset, checks it (ids in [0, K),
 // strictly increasing) and counts the community sizes.
+// head[j] (when wanted): the id of a list of one, -1 for an empty list, else the
+// list's offset with the sign bit set.
 __global__ void k_cover_copy(const long long *mptr, const int *memb, long long n, const int *inv, int K,
-                             const int *off, int *out, int *size, int *status)
+                             const int *off, int *out, int *size, int *status, int *head)
 {
     if (*(volatile int *)status) return;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -176,15 +225,17 @@ __global__ void k_cover_copy(const long long *mptr, const int *memb, long long n
             out[o + k] = c;
             atomicAdd(&size[c], 1);
         }
+        if (head) head[j] = len == 1 ? prev : len == 0 ? -1 : (int)(0x80000000u | (unsigned)o);
     }
     if (bad) atomicOr(status, 1);
 }
 
 // Members of every community: node j into its communities' lists.
+// (run_if: only when that flag is set.)
 __global__ void k_cover_scatter(const int *off, const int *memb, long long n, const int *cstart, int *cur, int *cmem,
-                                const int *status)
+                                const int *status, const int *run_if)
 {
-    if (*status) return;
+    if (*status || (run_if && !*run_if)) return;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride)
         for (int k = __ldg(&off[j]); k < __ldg(&off[j + 1]); ++k) {
@@ -193,9 +244,9 @@ __global__ void k_cover_scatter(const int *off, const int *memb, long long n, co
         }
 }
 
-__global__ void k_cover_rcp(const int *size, int K, Rcp *recip, const int *status)
+__global__ void k_cover_rcp(const int *size, int K, Rcp *recip, const int *status, const int *run_if)
 {
-    if (*status) return;
+    if (*status || (run_if && !*run_if)) return;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < K; c += gridDim.x * blockDim.x)
         recip[c] = size[c] > 0 ? rcp_of(size[c]) : Rcp{0ull, 0ull};
 }
@@ -242,7 +293,203 @@ __device__ __forceinline__ int claim_next(int *counter, int *slot)
     return *slot;
 }
 
-// ------------------------------------------------------------------ scoring
+// ------------------------------------------------------------------ scoring in node order
+
+constexpr int COVER_LIST_MAX = 1 << 20;  // longer lists are scored by k_cover_score
+
+// Length of node v's list from its head word.
+__device__ __forceinline__ int head_len(int h, const int *off, int v)
+{
+    if (h >= 0) return 1;
+    return h == -1 ? 0 : __ldg(&off[v + 1]) - (h & 0x7FFFFFFF);
+}
+
+// Members and arcs (cv) of every community, and members and segment size
+// (capw): for each of its members the list lengths of the neighbours, summed.
+// A warp takes 32 nodes, a lane per arc of one node at a time.  The segments'
+// total goes to *total.
+__global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__ row_ptr, const int *__restrict__ col,
+                                                   const int *__restrict__ off, const int *__restrict__ memb,
+                                                   const int *__restrict__ head, long long n, unsigned long long *cv,
+                                                   unsigned long long *capw, unsigned long long *total, int *too_long,
+                                                   const int *status)
+{
+    if (*status) return;
+    const int lane = threadIdx.x & 31;
+    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
+    unsigned long long sum = 0;
+    for (long long u0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; u0 < n; u0 += nw * 32) {
+        const long long u = min(u0 + lane, n - 1);
+        const long long r = __ldg(&row_ptr[u]);
+        const unsigned deg = (unsigned)(__ldg(&row_ptr[u + 1]) - r);
+        unsigned long long mine = 0;
+        const int cnt = (int)min(32LL, n - u0);
+        for (int i0 = 0; i0 < cnt; i0 += 4) {
+            unsigned s[4] = {0u, 0u, 0u, 0u};
+            bool more = false;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const long long ri = __shfl_sync(0xffffffffu, r, i0 + q);
+                const unsigned d = i0 + q < cnt ? __shfl_sync(0xffffffffu, deg, i0 + q) : 0u;
+                if ((unsigned)lane < d) {
+                    const int v = __ldg(&col[ri + lane]);
+                    const int l = head_len(__ldg(&head[v]), off, v);
+                    if (l > COVER_LIST_MAX) *too_long = 1;
+                    s[q] = (unsigned)min(l, COVER_LIST_MAX);
+                }
+                more |= d > 32u;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned t = __reduce_add_sync(0xffffffffu, s[q]);
+                if (lane == i0 + q) mine = t;
+            }
+            if (more)  // rows of more than 32 arcs: the rest
+                for (int q = 0; q < 4 && i0 + q < cnt; ++q) {
+                    const long long ri = __shfl_sync(0xffffffffu, r, i0 + q);
+                    const unsigned d = __shfl_sync(0xffffffffu, deg, i0 + q);
+                    for (unsigned e0 = 32u; e0 < d; e0 += 32u) {
+                        unsigned x = 0u;
+                        if (e0 + lane < d) {
+                            const int v = __ldg(&col[ri + e0 + lane]);
+                            const int l = head_len(__ldg(&head[v]), off, v);
+                            if (l > COVER_LIST_MAX) *too_long = 1;
+                            x = (unsigned)min(l, COVER_LIST_MAX);
+                        }
+                        const unsigned t = __reduce_add_sync(0xffffffffu, x);
+                        if (lane == i0 + q) mine += t;
+                    }
+                }
+        }
+        if (lane < cnt) {
+            const int b = __ldg(&off[u]), e = __ldg(&off[u + 1]);
+            for (int k = b; k < e; ++k) {
+                const int c = __ldg(&memb[k]);
+                atomicAdd(&cv[c], (1ull << VOL_BITS) | deg);
+                atomicAdd(&capw[c], (1ull << VOL_BITS) | mine);  // (a sum beyond 33 bits is beyond the scratch too)
+            }
+            sum += mine * (unsigned long long)(e - b);
+        }
+    }
+    sum = warp_sum_u64(sum);
+    if (lane == 0 && sum) atomicAdd(total, sum);
+}
+
+// gate: nonzero keeps the kernels over runs from working; old_path: set when
+// the cover is to be scored by member lists instead.
+__global__ void k_cover_gate(const int *status, const unsigned long long *total, long long entries, const int *too_long,
+                             int *gate, int *old_path)
+{
+    const bool fits = entries > 0 && *total <= (unsigned long long)entries && !*too_long;
+    *gate = *status | (fits ? 0 : 256);
+    *old_path = *status || fits ? 0 : 1;
+}
+
+struct CoverWalkArgs {
+    const long long *row_ptr;
+    const int *col, *off, *memb, *head;
+    long long n;
+    const unsigned *base;
+    unsigned long long *curs;  // cut arcs << 32 | packed entries of each community
+    int *nbr;
+    const int *gate;
+};
+
+constexpr int CW_THREADS = 256;
+constexpr int CW_UNROLL = 4;
+constexpr int CW_OWN_CAP = 2048;
+
+// The arcs col[0 .. total) of a warp's nodes, node_of(e) the owner of arc e
+// (0 .. 31), aoff the owners' list offsets (33).  Every arc is taken once per
+// community c of its owner; each such visit adds one to c's cut arcs unless the
+// far end is in c, and packs the far end's communities above c that the owner
+// is not in.  The loops over the lists are warp-uniform (one turn each where
+// all lists hold one id); the lanes of one community take their places with
+// one atomic.
+template <class OWN>
+__device__ __forceinline__ void cover_arcs(const CoverWalkArgs &a, const int *col, unsigned total, const int *aoff,
+                                           OWN node_of, int lane)
+{
+    constexpr unsigned ALL = 0xffffffffu;
+    const unsigned lt = (1u << lane) - 1u;
+    for (unsigned e0 = 0; e0 < total; e0 += 32u * CW_UNROLL) {
+        int v[CW_UNROLL], hv[CW_UNROLL], o[CW_UNROLL];
+#pragma unroll
+        for (int k = 0; k < CW_UNROLL; ++k) {
+            const unsigned e = e0 + lane + 32u * k;
+            v[k] = e < total ? __ldcs(&col[e]) : -1;
+            o[k] = e < total ? node_of(e) : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < CW_UNROLL; ++k) hv[k] = v[k] >= 0 ? __ldg(&a.head[v[k]]) : -1;
+#pragma unroll
+        for (int k = 0; k < CW_UNROLL; ++k) {
+            const int ab = aoff[o[k]], la = v[k] >= 0 ? aoff[o[k] + 1] - ab : 0;
+            const int h = hv[k], lb = v[k] >= 0 ? head_len(h, a.off, v[k]) : 0;
+            const int *A = a.memb + ab, *B = a.memb + (h & 0x7FFFFFFF);
+            const unsigned xa = __reduce_max_sync(ALL, (unsigned)la), yb = max(1u, __reduce_max_sync(ALL, (unsigned)lb));
+            for (unsigned x = 0; x < xa; ++x) {
+                const int c = (int)x < la ? __ldg(&A[x]) : -1;
+                bool cut = c >= 0 && (lb == 1 ? h != c : !list_has(B, lb, c));
+                __syncwarp();
+                for (unsigned y = 0; y < yb; ++y) {
+                    int j = -1;
+                    if (cut && (int)y < lb) j = lb == 1 ? h : __ldg(&B[y]);
+                    bool pack = j > c;
+                    if (pack && la > 1) pack = !list_has(A, la, j);
+                    __syncwarp();
+                    const unsigned pm = __ballot_sync(ALL, pack), cm = y == 0 ? __ballot_sync(ALL, cut) : 0u;
+                    if (!(pm | cm)) continue;
+                    const unsigned same = __match_any_sync(ALL, c);
+                    const unsigned peers = same & (pm | cm);
+                    unsigned at = 0;
+                    if ((peers >> lane) & 1u) {
+                        if (lane == __ffs(peers) - 1)
+                            at = __ldg(&a.base[c]) +
+                                 (unsigned)atomicAdd(&a.curs[c], ((unsigned long long)__popc(same & cm) << 32) |
+                                                                      (unsigned)__popc(same & pm));
+                    }
+                    at = __shfl_sync(ALL, at, peers ? __ffs(peers) - 1 : 0);
+                    if (pack) __stcs(&a.nbr[at + __popc(same & pm & lt)], j);
+                }
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(CW_THREADS) k_cover_walk(CoverWalkArgs a)
+{
+    __shared__ int aoff_s[CW_THREADS / 32][33];
+    __shared__ unsigned char own_s[CW_THREADS / 32][CW_OWN_CAP];
+    if (*a.gate) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long nwarps = (long long)gridDim.x * (CW_THREADS / 32);
+    for (long long u0 = ((long long)blockIdx.x * (CW_THREADS / 32) + w) * 32; u0 < a.n; u0 += nwarps * 32) {
+        const int nm = (int)min(32LL, a.n - u0);
+        const long long u = u0 + min(lane, nm - 1);
+        const long long r = __ldg(&a.row_ptr[u]), r0 = __shfl_sync(0xffffffffu, r, 0);
+        const unsigned total = (unsigned)(__ldg(&a.row_ptr[u0 + nm]) - r0);
+        const unsigned rel = lane < nm ? (unsigned)(r - r0) : total;
+        const unsigned nxt = __shfl_down_sync(0xffffffffu, rel, 1), end = lane == 31 ? total : nxt;
+        aoff_s[w][lane] = __ldg(&a.off[u0 + min(lane, nm)]);
+        if (lane == 0) aoff_s[w][32] = __ldg(&a.off[u0 + nm]);
+        __syncwarp();
+        if (total <= (unsigned)CW_OWN_CAP) {
+            for (unsigned e = rel; e < end; ++e) own_s[w][e] = (unsigned char)lane;
+            __syncwarp();
+            const unsigned char *own = own_s[w];
+            cover_arcs(a, a.col + r0, total, aoff_s[w], [own](unsigned e) { return (int)own[e]; }, lane);
+        } else {
+            for (int i = 0; i < nm; ++i) {
+                const unsigned b = __shfl_sync(0xffffffffu, rel, i), z = __shfl_sync(0xffffffffu, end, i);
+                cover_arcs(a, a.col + r0 + b, z - b, aoff_s[w], [i](unsigned) { return i; }, lane);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// ------------------------------------------------------------------ scoring by member lists
 
 struct CoverScoreArgs {
     const long long *row_ptr;
@@ -255,6 +502,7 @@ struct CoverScoreArgs {
     int *next;                 // claim counter
     unsigned long long *g;     // GS_* accumulators
     int *status;
+    const int *run_if;         // only when this flag is set (null: always)
     SmemPlan plan;             // shared-memory layout of the block
 };
 
@@ -262,7 +510,7 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_score(CoverScoreArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_c;
-    if (*a.status) return;
+    if (*a.status || (a.run_if && !*a.run_if)) return;
     const SmemPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);
@@ -419,6 +667,7 @@ struct CoverCmpArgs {
     int *next_a, *next_b, *next_c;
     unsigned long long *g;
     int *status;
+    const double *logt;  // log(N / n), then n / N, 1 <= n <= LOGT_MAX
     SmemPlan plan;
 };
 
@@ -439,6 +688,14 @@ __device__ __forceinline__ void flush_compare_acc(const CompareAcc &acc, unsigne
         const unsigned long long u = group_sum_u64(*src[k], T, red);
         if (threadIdx.x == 0 && u) atomicAdd(g + dst[k], u);
     }
+}
+
+// The larger of two fractions n << 32 | d (0: none), compared exactly.
+__device__ __forceinline__ unsigned long long larger_fraction(unsigned long long x, unsigned long long y)
+{
+    if (!y) return x;
+    if (!x) return y;
+    return (y >> 32) * (x & 0xFFFFFFFFull) > (x >> 32) * (y & 0xFFFFFFFFull) ? y : x;
 }
 
 // The cells of every truth community a: counts |a n b| over a's members' found
@@ -470,16 +727,26 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_cells(CoverCmpArgs a)
         unsigned R = 1;
         for (;;) {
             unsigned rmax = 0;
-            unsigned long long rbest = 0;
+            unsigned long long rbest = 0;  // the largest n / (n_a + n_b) as n << 32 | n_a + n_b
             CompareAcc part;
             compare_acc_zero(part);
             bool ok = true;
             for (unsigned r = 0; r < R && ok; ++r) {
-                for (int idx = mb + tid; idx < me; idx += T) {
-                    const int i = __ldg(&a.acmem[idx]);
-                    for (int k = __ldg(&a.boff[i]); k < __ldg(&a.boff[i + 1]); ++k) {
-                        const int b = __ldg(&a.bmemb[k]);
-                        if (R == 1 || tab_split((unsigned)b, R) == r) tab_insert(tab, (unsigned)b);
+                // (warp-uniform: the members of a community mostly share a found id,
+                // so a warp's equal ids are merged into one update)
+                for (int i0 = mb + (tid & ~31); i0 < me; i0 += T) {
+                    const int idx = i0 + (tid & 31);
+                    int k = 0, ke = 0;
+                    if (idx < me) {
+                        const int i = __ldg(&a.acmem[idx]);
+                        k = __ldg(&a.boff[i]);
+                        ke = __ldg(&a.boff[i + 1]);
+                    }
+                    while (__any_sync(0xffffffffu, k < ke)) {
+                        const int b = k < ke ? __ldg(&a.bmemb[k]) : 0;
+                        tab_insert_warp(tab, (unsigned)b, k < ke && (R == 1 || tab_split((unsigned)b, R) == r));
+                        __syncwarp();
+                        ++k;
                     }
                 }
                 block_sync();
@@ -494,9 +761,12 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_cells(CoverCmpArgs a)
                     part.cells += 1;
                     const double l1 = cell_log(n, na, nb);
                     part.vi += fp_from_double(vi_term_l(n, l1), SC_VI);
-                    part.hnum += fp_from_double(nmi_num_term_l(n, a.N, l1, log_ratio(a.N, n)), SC_H);
+                    const bool tb = n <= LOGT_MAX;
+                    part.hnum += fp_from_double(nmi_num_term_q(tb ? __ldg(&a.logt[LOGT_MAX + 1 + n]) : nmi_over(n, a.N), l1,
+                                                               tb ? __ldg(&a.logt[n]) : log_ratio(a.N, n)),
+                                                SC_H);
                     rmax = max(rmax, (unsigned)n);
-                    rbest = max(rbest, (unsigned long long)__double_as_longlong(f_ratio(n, na, nb)));
+                    rbest = larger_fraction(rbest, ((unsigned long long)n << 32) | (unsigned long long)(na + nb));
                     atomicMax(&a.colmax[b], (unsigned)n);
                 });
                 block_sync();
@@ -519,18 +789,20 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_cells(CoverCmpArgs a)
                 continue;
             }
             compare_acc_add(acc, part);
-            // the row's largest cell and ratio (non-negative doubles order as their bits)
+            // the row's largest cell and ratio (divided once: rounding is monotone,
+            // so the largest rounded ratio is the rounded largest ratio)
             const unsigned m = group_max_u32(rmax, T, red);
             unsigned long long bb = rbest;
-            for (int d = 16; d > 0; d >>= 1) bb = max(bb, __shfl_down_sync(0xffffffffu, bb, d));
+            for (int d = 16; d > 0; d >>= 1) bb = larger_fraction(bb, __shfl_down_sync(0xffffffffu, bb, d));
             block_sync();
             if ((tid & 31) == 0) red[tid >> 5] = bb;
             block_sync();
             if (tid == 0) {
                 unsigned long long best = 0;
-                for (int w = 0; w < (T >> 5); ++w) best = max(best, red[w]);
+                for (int w = 0; w < (T >> 5); ++w) best = larger_fraction(best, red[w]);
                 a.rowmax[c] = m;
-                a.rowbest[c] = best;
+                const long long bn = (long long)(best >> 32), bd = (long long)(best & 0xFFFFFFFFull);
+                a.rowbest[c] = bn ? (unsigned long long)__double_as_longlong(f_ratio(bn, na, bd - na)) : 0ull;
             }
             break;
         }
@@ -575,16 +847,6 @@ __global__ void k_cover_cols(CoverCmpArgs a)
     flush_compare_acc(acc, a.g, red);
 }
 
-// Pair index k < L(L-1)/2 -> (p, q), p < q < L.
-__device__ __forceinline__ void pair_of(long long k, long long *p, long long *q)
-{
-    long long b = (long long)((1.0 + sqrt(1.0 + 8.0 * (double)k)) * 0.5);
-    while (b * (b - 1) / 2 > k) --b;
-    while ((b + 1) * b / 2 <= k) ++b;
-    *q = b;
-    *p = k - b * (b - 1) / 2;
-}
-
 // Pair-count corrections for pairs of nodes sharing two or more communities on
 // side X (the other side is Y).  For community c of X, its members with two or
 // more memberships are paired up; a pair is taken by the smallest community
@@ -626,11 +888,10 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_pairs(CoverCmpArgs a)
         const bool in_smem = L <= OVL_CAP;
         // pairs of overlapping members (from shared memory, or the whole member
         // list filtered again when there are too many to hold)
-        const long long Lp = in_smem ? L : (long long)(me - mb);
-        const long long npairs = Lp * (Lp - 1) / 2;
-        for (long long k = tid; k < npairs; k += T) {
-            long long pp, qq;
-            pair_of(k, &pp, &qq);
+        // a warp per first member, its lanes over the later ones
+        const int Lp = in_smem ? L : me - mb;
+        for (int pp = tid >> 5; pp < Lp - 1; pp += T >> 5)
+        for (int qq = pp + 1 + (tid & 31); qq < Lp; qq += 32) {
             const int i = in_smem ? ovl[pp] : __ldg(&xcmem[mb + pp]);
             const int j = in_smem ? ovl[qq] : __ldg(&xcmem[mb + qq]);
             const int li = __ldg(&xoff[i + 1]) - __ldg(&xoff[i]), lj = __ldg(&xoff[j + 1]) - __ldg(&xoff[j]);
@@ -685,9 +946,20 @@ int grid_of(long long n, int threads, int num_sms, int per_sm)
     return (int)std::max<long long>(g, 1);
 }
 
-// Brings one cover to the stored order and builds its member lists.
+// Member lists of a cover's communities (run_if: only when that flag is set).
+int members_of_side(const CoverSide &c, long long n, const CoverWs &w, int num_sms, cudaStream_t s, const int *run_if)
+{
+    const int l2 = scan_offsets(c.size, c.K, c.cstart, w.scan_tmp, w.counters + CC_SCAN, w.status, s);
+    if (l2 < 0) return -1;
+    k_cover_scatter<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(c.off, c.memb, n, c.cstart, c.cur, c.cmem, w.status,
+                                                               run_if);
+    return l2 + 1;
+}
+
+// Brings one cover to the stored order and builds its member lists (members).
 int prepare_side(const long long *mptr, const int *memb, long long m, long long n, const int *inv,
-                 const CoverSide &c, const CoverWs &w, int num_sms, cudaStream_t s)
+                 const CoverSide &c, const CoverWs &w, int num_sms, cudaStream_t s, int *head = nullptr,
+                 bool members = true)
 {
     int L = 0;
     k_cover_len<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(mptr, n, m, inv, c.len, w.status);
@@ -696,15 +968,11 @@ int prepare_side(const long long *mptr, const int *memb, long long m, long long 
     if (l1 < 0) return -1;
     L += l1;
     k_cover_copy<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(mptr, memb, n, inv, c.K, c.off, c.memb, c.size,
-                                                            w.status);
+                                                            w.status, head);
     ++L;
-    const int l2 = scan_offsets(c.size, c.K, c.cstart, w.scan_tmp, w.counters + CC_SCAN, w.status, s);
-    if (l2 < 0) return -1;
-    L += l2;
-    k_cover_scatter<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(c.off, c.memb, n, c.cstart, c.cur, c.cmem,
-                                                               w.status);
-    ++L;
-    return L;
+    if (!members) return L;
+    const int l2 = members_of_side(c, n, w, num_sms, s, nullptr);
+    return l2 < 0 ? -1 : L + l2;
 }
 
 }  // namespace
@@ -721,9 +989,50 @@ int launch_cover_score(const GraphDev &g, const long long *mptr, const int *memb
                        const CoverWs &w, int num_sms, cudaStream_t s)
 {
     const long long n = g.n;
-    int L = prepare_side(mptr, memb, m, n, g.inv, w.a, w, num_sms, s);
+    const bool runs = w.run_entries > 0;
+    int L = prepare_side(mptr, memb, m, n, g.inv, w.a, w, num_sms, s, runs ? w.head : nullptr, !runs);
     if (L < 0) return -1;
-    k_cover_rcp<<<grid_of(K, 256, num_sms, 4), 256, 0, s>>>(w.a.size, K, w.recip, w.status);
+    const int *run_if = nullptr;
+    if (runs) {
+        int *const gate = w.counters + CC_GATE, *const old_path = w.counters + CC_OLD;
+        unsigned long long *const total = (unsigned long long *)(w.counters + CC_TOTAL);
+        k_cover_cap<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(g.row_ptr, g.col, w.a.off, w.a.memb, w.head, n, w.cv, w.capw,
+                                                               total, w.counters + CC_LONG, w.status);
+        k_cover_gate<<<1, 1, 0, s>>>(w.status, total, w.run_entries, w.counters + CC_LONG, gate, old_path);
+        L += 2 + launch_segment_bases(w.capw, K, w.base, w.recip, (unsigned *)w.scan_tmp, gate, s);
+        CoverWalkArgs a;
+        a.row_ptr = g.row_ptr;
+        a.col = g.col;
+        a.off = w.a.off;
+        a.memb = w.a.memb;
+        a.head = w.head;
+        a.n = n;
+        a.base = w.base;
+        a.curs = w.curs;
+        a.nbr = w.nbr;
+        a.gate = gate;
+        k_cover_walk<<<grid_of(n, CW_THREADS, num_sms, 5), CW_THREADS, 0, s>>>(a);
+        CoverRuns r;
+        r.cv = w.cv;
+        r.curs = w.curs;
+        r.base = w.base;
+        r.nbr = w.nbr;
+        r.recip = w.recip;
+        r.inter = w.inter;
+        r.rec = w.rec;
+        for (int k = 0; k < 4; ++k) r.hdr[k] = w.hdr[k];
+        r.counters = w.counters + CC_RUNS;
+        r.gate = gate;
+        r.err = w.status;
+        const int lr = launch_cover_runs(r, K, g.n_arcs / 2, w.gacc, num_sms, s);
+        if (lr < 0) return -1;
+        L += 1 + lr;
+        run_if = old_path;  // the kernels below work only when the runs did not fit
+        const int lm = members_of_side(w.a, n, w, num_sms, s, run_if);
+        if (lm < 0) return -1;
+        L += lm;
+    }
+    k_cover_rcp<<<grid_of(K, 256, num_sms, 4), 256, 0, s>>>(w.a.size, K, w.recip, w.status, run_if);
     CoverScoreArgs a;
     a.row_ptr = g.row_ptr;
     a.col = g.col;
@@ -737,6 +1046,7 @@ int launch_cover_score(const GraphDev &g, const long long *mptr, const int *memb
     a.next = w.counters + CC_NEXT_C;
     a.g = w.gacc;
     a.status = w.status;
+    a.run_if = run_if;
     a.plan = plan_smem(COVER_THREADS, COVER_SMEM);
     k_cover_score<<<std::min(num_sms * 4, std::max(K, 1)), COVER_THREADS, COVER_SMEM, s>>>(a);
     k_cover_score_fin<<<1, 32, 0, s>>>(w.gacc, w.status, n, g.n_arcs / 2, (qm_quality *)w.result);
@@ -774,14 +1084,16 @@ int launch_cover_compare(const long long *aptr, const int *amemb, long long ma, 
     a.next_c = w.counters + CC_NEXT_C;
     a.g = w.gacc;
     a.status = w.status;
+    a.logt = w.logt;
     a.plan = plan_smem(COVER_THREADS, COVER_SMEM);
+    launch_batch_logt(w.logt, n, s);
     k_cover_cells<<<std::min(num_sms * 4, std::max(ka, 1)), COVER_THREADS, COVER_SMEM, s>>>(a);
     k_cover_rows<<<grid_of(ka, 256, num_sms, 2), 256, 0, s>>>(a);
     k_cover_cols<<<grid_of(kb, 256, num_sms, 2), 256, 0, s>>>(a);
     k_cover_pairs<true><<<std::min(num_sms * 4, std::max(ka, 1)), COVER_THREADS, 0, s>>>(a);
     k_cover_pairs<false><<<std::min(num_sms * 4, std::max(kb, 1)), COVER_THREADS, 0, s>>>(a);
     k_cover_compare_fin<<<1, 32, 0, s>>>(w.gacc, w.status, n, (qm_compare *)w.result);
-    return cudaGetLastError() == cudaSuccess ? L1 + L2 + 6 : -1;
+    return cudaGetLastError() == cudaSuccess ? L1 + L2 + 7 : -1;
 }
 
 }  // namespace qm

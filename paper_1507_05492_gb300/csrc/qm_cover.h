@@ -35,6 +35,17 @@ struct CoverWs {
     unsigned *rowmax;          // [ka] comparison: largest cell of each truth community
     unsigned long long *rowbest; // [ka] comparison: largest F ratio of each row (as double bits)
     unsigned *colmax;          // [kb] comparison: largest cell of each found community (zeroed)
+    double *logt;              // [LOGT_WORDS] comparison: log(N / n), then n / N
+    // scoring by runs in node order (run_entries > 0)
+    unsigned long long *cv, *capw;  // [K] members << 33 | arcs, members << 33 | segment size (zeroed)
+    unsigned long long *curs;  // [K] cut arcs << 32 | packed entries (zeroed)
+    int *head;                 // [n] each node's list: its id, -1, or its offset with the sign bit
+    unsigned *base;            // [K] segment bases
+    int *inter;                // [K] cut arcs
+    unsigned long long *rec;   // [K][8] count records
+    qmk::RunHdr *hdr[4];       // [K] each: run headers by class
+    int *nbr;                  // [run_entries] packed runs
+    long long run_entries;
     int *scan_tmp;
     size_t zero_bytes;
     size_t bytes;
@@ -42,8 +53,11 @@ struct CoverWs {
 
 // Scratch of a cover scoring call (n nodes, m memberships, K ids) and of a
 // comparison of two covers (ma, mb memberships; ka, kb ids).
-size_t cover_score_ws_bytes(long long n, long long m, int K);
-CoverWs carve_cover_score_ws(void *base, long long n, long long m, int K);
+// run_entries: entries of the packed runs (cover_run_entries), or 0 to score by
+// member lists only.
+long long cover_run_entries(long long n, long long n_arcs, long long m, int K);
+size_t cover_score_ws_bytes(long long n, long long m, int K, long long run_entries);
+CoverWs carve_cover_score_ws(void *base, long long n, long long m, int K, long long run_entries);
 size_t cover_compare_ws_bytes(long long n, long long ma, int ka, long long mb, int kb);
 CoverWs carve_cover_compare_ws(void *base, long long n, long long ma, int ka, long long mb, int kb);
 

@@ -195,6 +195,28 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
 // (algorithms 1, 4, 5 and 6, weighted graphs, and 7 where the half-edge pass does
 // not apply) rather than the members in community order.
 bool score_rows(const GraphDev &g, int algo, int shard_p);
+// Segment bases (exclusive prefix of the low 33 bits) and reciprocals of the
+// sizes (the bits above) of K words; sums: scratch of K / 4096 + 1 words.
+// Returns its launches.
+int launch_segment_bases(const unsigned long long *words, int K, unsigned *base, qmk::Rcp *recip, unsigned *sums,
+                         const int *status, cudaStream_t s, TraceFn tr = nullptr);
+// Counting and terms of the packed runs of a cover (qm_cover.cu): members and
+// volumes in cv, runs nbr[base[c] ..) with curs[c] = cut arcs << 32 | length;
+// nothing is done when *gate is set.  Sums go to gacc (GS_* words).
+struct CoverRuns {
+    const unsigned long long *cv, *curs;
+    const unsigned *base;
+    const int *nbr;
+    const qmk::Rcp *recip;
+    int *inter;                // [K]
+    unsigned long long *rec;   // [K][8]
+    qmk::RunHdr *hdr[4];       // [K] each
+    int *counters;             // [16] zeroed
+    const int *gate;
+    int *err;
+};
+bool cover_runs_ok(int K);
+int launch_cover_runs(const CoverRuns &r, int K, long long E, unsigned long long *gacc, int num_sms, cudaStream_t s);
 // For a renumbered graph: out[j] = labels[inv[j]] and the community sizes into
 // ws.size, or (rows) members and arcs into ws.cv (zeroed), with the label range
 // check of k_hist.  Returns 1 or -1.

@@ -1888,6 +1888,19 @@ bool score_rows(const GraphDev &g, int algo, int shard_p)
     return algo != 0 && !bin_mode_of(algo, false) && !(algo == ALGO_HALF && g.up_ptr && shard_p == 1);
 }
 
+int launch_segment_bases(const unsigned long long *words, int K, unsigned *base, Rcp *recip, unsigned *sums,
+                         const int *status, cudaStream_t s, TraceFn tr)
+{
+    const int tiles = (K + VSCAN_TILE - 1) / VSCAN_TILE;
+    if (tiles > 1) {
+        TRACE("k_vscan_tiles");
+        k_vscan_tiles<<<tiles, VSCAN_THREADS, 0, s>>>(words, K, sums, status);
+    }
+    TRACE("k_vscan_apply");
+    k_vscan_apply<<<tiles, VSCAN_THREADS, 0, s>>>(words, K, sums, base, recip, status);
+    return tiles > 1 ? 2 : 1;
+}
+
 // Phase A in stored node order: volumes (unless the label permutation has
 // counted them), segment bases, the walk.  Returns its launches.
 static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh, bool hi,
@@ -1902,16 +1915,8 @@ static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const 
             labels, g.row_ptr, n, K, ws.cv, ws.status, smem ? 1 : 0);
         ++launches;
     }
-    const int tiles = (K + VSCAN_TILE - 1) / VSCAN_TILE;
-    unsigned *base = (unsigned *)ws.cursor, *sums = (unsigned *)ws.scan_tmp;
-    if (tiles > 1) {
-        TRACE("k_vscan_tiles");
-        k_vscan_tiles<<<tiles, VSCAN_THREADS, 0, s>>>(ws.cv, K, sums, ws.status);
-        ++launches;
-    }
-    TRACE("k_vscan_apply");
-    k_vscan_apply<<<tiles, VSCAN_THREADS, 0, s>>>(ws.cv, K, sums, base, ws.recip, ws.status);
-    ++launches;
+    unsigned *base = (unsigned *)ws.cursor;
+    launches += launch_segment_bases(ws.cv, K, base, ws.recip, (unsigned *)ws.scan_tmp, ws.status, s, tr);
     RowsArgs a;
     a.row_ptr = g.row_ptr;
     a.col = g.col;
@@ -2172,6 +2177,41 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     }
     TRACE(nullptr);
     return cudaGetLastError() == cudaSuccess ? launches : -1;
+}
+
+bool cover_runs_ok(int K) { return K < CT_MAX_K; }
+
+int launch_cover_runs(const CoverRuns &r, int K, long long E, unsigned long long *gacc, int num_sms, cudaStream_t s)
+{
+    const int cb = ct_count_bits(K), most = (int)std::min<long long>(INT_MAX, (1LL << cb) - 1);
+    const Shard own{0, 1};
+    k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
+        r.cv, r.base, r.curs, K, std::min(ct_fill_warp(K, num_sms), most), std::min(CT_FILL_GROUP, most),
+        std::min(CB_FILL, most), r.hdr[0], r.hdr[1], r.hdr[2], r.hdr[3], r.inter, r.counters, r.gate, own);
+    CountTabArgs t;
+    t.x.nbr = r.nbr;
+    t.x.aoff = nullptr;
+    t.x.start = nullptr;
+    t.x.inter = r.inter;
+    t.x.recip = r.recip;
+    t.x.rec = r.rec;
+    t.x.K = K;
+    t.x.err = r.err;
+    t.x.full = 0;
+    t.big = r.hdr[0];
+    t.small = r.hdr[1];
+    t.lng = r.hdr[2];
+    t.mid = r.hdr[3];
+    t.counters = r.counters;
+    t.status = r.gate;
+    t.cb = cb;
+    t.stage_wait = g_stage_wait.load();
+    t.plan = plan_smem(CB_THREADS, CB_SMEM);
+    k_count_tab<CT_ABOVE><<<(int)std::min<long long>((long long)num_sms * CT_BLOCKS, K), CT_THREADS, 0, s>>>(t);
+    k_count_big<CT_ABOVE><<<std::min(2 * num_sms, K), CB_THREADS, CB_SMEM, s>>>(t);
+    k_score_terms<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(nullptr, r.cv, r.rec, K, E, PerCommDev{}, gacc, r.gate,
+                                                               own);
+    return cudaGetLastError() == cudaSuccess ? 4 : -1;
 }
 
 int launch_score_fin(const unsigned long long *gacc, const int *status, long long n, long long E, qm_quality *out,
