@@ -1110,6 +1110,7 @@ constexpr int BU_CELLS_SMEM = 48 * 1024;  // shared memory of a k_bu_cells block
 __global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *items, int count, BatchUnits b)
 {
     __shared__ unsigned long long red[72];
+    __shared__ unsigned late[BU_FIN_THREADS / 32][LATE_CELL_WORDS];
     const int tid = threadIdx.x, T = blockDim.x;
     for (int it = blockIdx.x; it < count; it += gridDim.x) {
         const BatchItem I = items[it];
@@ -1157,21 +1158,23 @@ __global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *item
             CompareAcc acc;
             compare_acc_zero(acc);
             const int nc = __ldcg(&b.ncells[it]);
-            for (int i = tid; i < nc; i += T) {
-                const Cell cl = S.cells[i];
-                if (!QM_CHK(cl.a, x.ka, 30) || !QM_CHK(cl.b, x.kb, 31)) continue;
-                const long long n = cl.n, na = __ldcg(&S.size_a[cl.a]);
-                const long long nb = __ldcg(&S.start[cl.b + 1]) - __ldcg(&S.start[cl.b]);
-                acc.a11 += (unsigned long long)(n * (n - 1) / 2);
-                atomicMax(&S.rowmax_n[cl.a], (unsigned)n);
-                rowmax_ratio_update(&S.rowmax_r[cl.a], (unsigned long long)n, (unsigned long long)(na + nb));
-                const double l1 = cell_log(n, na, nb);
-                acc.vi += fp_from_double(vi_term_l(n, l1), SC_VI);
-                const bool tab = logt && n <= LOGT_MAX;
-                const double lr = tab ? __ldg(&logt[n]) : log_ratio(x.N, n);
-                const double q = tab ? __ldg(&logt[LOGT_MAX + 1 + n]) : nmi_over(n, x.N);
-                acc.hnum += fp_from_double(nmi_num_term_q(q, l1, lr), SC_H);
+            LateCells lc{late[tid >> 5], 0u};
+            for (int i0 = tid & ~31; i0 < nc; i0 += T) {
+                const int i = i0 + (tid & 31);
+                Cell cl{0, 0, 0u, 0u};
+                if (i < nc) cl = S.cells[i];
+                const bool in = i < nc && QM_CHK(cl.a, x.ka, 30) && QM_CHK(cl.b, x.kb, 31);
+                unsigned na = 0, nb = 0;
+                if (in) {
+                    na = (unsigned)__ldcg(&S.size_a[cl.a]);
+                    nb = (unsigned)(__ldcg(&S.start[cl.b + 1]) - __ldcg(&S.start[cl.b]));
+                    acc.a11 += (unsigned long long)cl.n * (cl.n - 1u) / 2ull;
+                    if (cl.n > *(volatile unsigned *)&S.rowmax_n[cl.a]) atomicMax(&S.rowmax_n[cl.a], cl.n);
+                    rowmax_ratio_update(&S.rowmax_r[cl.a], cl.n, (unsigned long long)na + nb);
+                }
+                cell_terms_warp(cl.n, na, nb, in, x.N, logt, acc, lc);
             }
+            late_cells_flush(x.N, logt, acc, lc);
             for (int c = tid; c < I.K; c += T) {
                 const long long nb = __ldcg(&S.start[c + 1]) - __ldcg(&S.start[c]);
                 if (nb == 0) continue;

@@ -380,14 +380,18 @@ static __global__ void k_fill_log_int()
 // units of 2^-52 * 18, so the relative error stays below 1e-14); otherwise,
 // and in particular near a ratio of 1 where the terms would cancel, one
 // logarithm of the ratio is taken.
+// The comparisons are made on the integers (products below 2^26, exact as
+// doubles too): GB300 issues FP64 at a small fraction of the integer rate.
 __device__ __forceinline__ double cell_log(long long n, long long na, long long nb)
 {
-    const double x = __dmul_rn((double)n, (double)n), y = __dmul_rn((double)na, (double)nb);
-    if (n <= LOGT_MAX && na <= LOGT_MAX && nb <= LOGT_MAX && (__dmul_rn(4.0, x) < y || x > __dmul_rn(4.0, y))) {
-        const double ln = __ldg(&qm_log_int[n]), la = __ldg(&qm_log_int[na]), lb = __ldg(&qm_log_int[nb]);
-        return __dsub_rn(__dsub_rn(__dmul_rn(2.0, ln), la), lb);
+    if (n <= LOGT_MAX && na <= LOGT_MAX && nb <= LOGT_MAX) {
+        const unsigned x = (unsigned)n * (unsigned)n, y = (unsigned)na * (unsigned)nb;
+        if (4u * x < y || x > 4u * y) {
+            const double ln = __ldg(&qm_log_int[n]), la = __ldg(&qm_log_int[na]), lb = __ldg(&qm_log_int[nb]);
+            return __dsub_rn(__dsub_rn(__dadd_rn(ln, ln), la), lb);
+        }
     }
-    return log(__ddiv_rn(x, y));
+    return log(__ddiv_rn(__dmul_rn((double)n, (double)n), __dmul_rn((double)na, (double)nb)));
 }
 
 // log(N / n); every caller evaluates this same expression (directly, or via

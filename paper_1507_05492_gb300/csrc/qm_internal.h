@@ -129,6 +129,7 @@ struct CompareWs {
     int *big_list;              // [kb]
     int *members;               // [n]
     qmk::Cell *cells;  // contingency cells of the counting pass ([n])
+    int *cell_off;              // bucketed cells (qm_cells.cuh): places of the (bucket, tile) groups
     int *scan_tmp;
     double *logt;               // [LOGT_WORDS] log(N / n), then n / N (LOGT_MAX + 1 each)
     size_t zero_bytes;

@@ -28,7 +28,7 @@ enum { C_BIG_COUNT = 0, C_BIG_NEXT = 1, C_SMALL_NEXT = 2, C_OVF_COUNT = 3, C_OVF
        C_BX_COUNT = 12 /* two words */ };
 
 constexpr int SCAN_TILE = 4096;   // elements per block in the multi-block scan
-constexpr int SCAN_SINGLE_MAX = 1 << 16;
+constexpr int SCAN_SINGLE_MAX = 1 << 13;  // beyond that one block is slower than three launches (4*10^4: 100 against 18 us)
 
 SmemPlan plan_smem(int T, int S)
 {
@@ -134,6 +134,8 @@ ScoreWs carve_score_ws(void *base, long long n, int K)
     return w;
 }
 
+#include "qm_cells.cuh"
+
 size_t compare_ws_bytes(long long n, int ka, int kb)
 {
     return carve_compare_ws(reinterpret_cast<void *>(4096), n, ka, kb).bytes;
@@ -169,8 +171,12 @@ CompareWs carve_compare_ws(void *base, long long n, int ka, int kb)
     p += align_up((size_t)n * 4, 256);
     w.cells = (Cell *)p;  // at most one new cell per node
     p += align_up((size_t)n * sizeof(Cell), 256);
+    const CellPlan cp = cell_plan(n, ka, kb);
+    const long long groups = cp.ok ? (long long)cp.nb * cp.ntiles : 0;
+    w.cell_off = (int *)p;
+    if (groups) p += align_up((size_t)(groups + 1) * 4, 256);
     w.scan_tmp = (int *)p;
-    p += align_up((size_t)(scan_tiles(kb) + 1) * 4, 256);
+    p += align_up((size_t)(scan_tiles((int)std::max<long long>(kb, groups)) + 1) * 4, 256);
     w.logt = (double *)p;
     p += align_up((size_t)LOGT_WORDS * 8, 256);
     w.bytes = (size_t)(p - (char *)base);
@@ -622,24 +628,28 @@ __global__ void k_compare_cells(CompareCtx x, const Cell *cells, const int *coun
                                 unsigned long long *g, const int *status)
 {
     __shared__ unsigned long long red[72];
+    __shared__ unsigned late[8][LATE_CELL_WORDS];  // blocks of 256 threads
     if (*status) return;
     CompareAcc acc;
     compare_acc_zero(acc);
+    LateCells lc{late[threadIdx.x >> 5], 0u};
     const int nc = counters[C_NCELLS];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
-        const Cell c = cells[i];
-        if (!QM_CHK(c.a, x.ka, 30) || !QM_CHK(c.b, x.kb, 31)) continue;
-        const long long n = c.n, na = __ldg(&x.size_a[c.a]), nb = __ldg(&size_b[c.b]);
-        acc.a11 += (unsigned long long)(n * (n - 1) / 2);
-        atomicMax(&x.rowmax_n[c.a], (unsigned)n);
-        rowmax_ratio_update(&x.rowmax_r[c.a], (unsigned long long)n, (unsigned long long)(na + nb));
-        const double l1 = cell_log(n, na, nb);
-        acc.vi += fp_from_double(vi_term_l(n, l1), SC_VI);
-        const bool tab = n <= LOGT_MAX;
-        acc.hnum += fp_from_double(nmi_num_term_q(tab ? __ldg(&x.logt[LOGT_MAX + 1 + n]) : nmi_over(n, x.N), l1,
-                                                  tab ? __ldg(&x.logt[n]) : log_ratio(x.N, n)),
-                                   SC_H);
+    for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < nc; i0 += gridDim.x * blockDim.x) {
+        const int i = i0 + (threadIdx.x & 31);
+        Cell c{0, 0, 0u, 0u};
+        if (i < nc) c = cells[i];
+        const bool in = i < nc && QM_CHK(c.a, x.ka, 30) && QM_CHK(c.b, x.kb, 31);
+        unsigned na = 0, nb = 0;
+        if (in) {
+            na = (unsigned)__ldg(&x.size_a[c.a]);
+            nb = (unsigned)__ldg(&size_b[c.b]);
+            acc.a11 += (unsigned long long)c.n * (c.n - 1u) / 2ull;
+            if (c.n > *(volatile unsigned *)&x.rowmax_n[c.a]) atomicMax(&x.rowmax_n[c.a], c.n);
+            rowmax_ratio_update(&x.rowmax_r[c.a], c.n, (unsigned long long)na + nb);
+        }
+        cell_terms_warp(c.n, na, nb, in, x.N, x.logt, acc, lc);
     }
+    late_cells_flush(x.N, x.logt, acc, lc);
     flush_compare(acc, g, red);
 }
 
@@ -1558,6 +1568,8 @@ void prepare_kernels()
     cudaFuncSetAttribute(k_count_long, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
+    cudaFuncSetAttribute(k_cells_split, cudaFuncAttributeMaxDynamicSharedMemorySize, CELL_SPLIT_SMEM);
+    cudaFuncSetAttribute(k_cells_table, cudaFuncAttributeMaxDynamicSharedMemorySize, CELL_TAB_SMEM);
     cudaFuncSetAttribute(k_count_w_big, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM);
     cudaFuncSetAttribute(k_expand_bin, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          bin_smem_bytes_per_warp(BIN_MAX) * (EXPAND_THREADS / 32));
@@ -2233,6 +2245,39 @@ int launch_compare(const int *truth, const int *found, long long n, int ka, int 
                    const CompareWs &ws, const Shape &sh, int num_sms, cudaStream_t s, TraceFn tr)
 {
     int launches = 0;
+    const CellPlan cells = cell_plan(n, ka, kb);
+    const bool bucketed = cells.ok;
+    const SmemPlan plan = plan_smem(sh.threads, sh.smem_bytes);
+    if (bucketed) {
+        CellArgs c;
+        c.truth = truth;
+        c.found = found;
+        c.n = n;
+        c.ka = ka;
+        c.kb = kb;
+        c.sh = cells.sh;
+        c.nb = cells.nb;
+        c.ntiles = cells.ntiles;
+        c.off = ws.cell_off;
+        c.pairs = (unsigned *)ws.members;
+        c.abits = bits_of(ka);
+        c.cells = ws.cells;
+        c.ncells = &ws.counters[C_NCELLS];
+        c.size_a = ws.size_a;
+        c.size_b = ws.size_b;
+        c.gacc = ws.gacc;
+        c.next = &ws.counters[C_BIG_NEXT];
+        c.status = ws.status;
+        TRACE("k_cells_count");
+        k_cells_count<<<std::min(cells.ntiles, num_sms * 2), CELL_THREADS, 0, s>>>(c);
+        launches += 1 + launch_scan(ws.cell_off, cells.nb * cells.ntiles, ws.cell_off, nullptr, nullptr, INT_MAX, nullptr,
+                                    ws.counters, ws.scan_tmp, ws.status, s, tr);
+        TRACE("k_cells_split");
+        k_cells_split<<<std::min(cells.ntiles, num_sms), CELL_THREADS, CELL_SPLIT_SMEM, s>>>(c);
+        TRACE("k_cells_table");
+        k_cells_table<<<std::min(cells.nb, num_sms), CELL_TAB_THREADS, CELL_TAB_SMEM, s>>>(c);
+        launches += 2;
+    } else {
     // sizes of the detected communities (the truth sizes are summed from the
     // contingency cells by k_compare_cm, far fewer updates than one per node)
     const int hist_smem = (kb <= 12288) ? kb * 4 : 0;
@@ -2240,12 +2285,12 @@ int launch_compare(const int *truth, const int *found, long long n, int ka, int 
     k_hist<<<grid_for(n, 512, num_sms, 4), 512, hist_smem, s>>>(found, kb, ws.size_b, nullptr, 0, nullptr, n,
                                                                 ws.status, hist_smem ? 1 : 0);
     ++launches;
-    const SmemPlan plan = plan_smem(sh.threads, sh.smem_bytes);
     launches += launch_scan(ws.size_b, kb, ws.start, ws.cursor, nullptr, plan.max_used_w, ws.big_list,
                             ws.counters, ws.scan_tmp, ws.status, s, tr);
     TRACE("k_scatter");
     k_scatter<<<grid_for(n, 512, num_sms, 8), 512, 0, s>>>(found, truth, n, ws.cursor, ws.members, ws.status, ka);
     ++launches;
+    }
     CompareKArgs a;
     a.x.truth = truth;
     a.x.tl = ws.members;  // truth labels in detected-community order (k_scatter with vals)
@@ -2269,8 +2314,11 @@ int launch_compare(const int *truth, const int *found, long long n, int ka, int 
     TRACE("k_log_table");
     k_log_table<<<(LOGT_MAX + 256) / 256, 256, 0, s>>>(ws.logt, n);
     ++launches;
-    TRACE("k_compare_cm");  // sh.blocks_per_sm: occupancy resolved by the caller
-    k_compare_cm<<<community_grid(kb, num_sms, sh), sh.threads, sh.smem_bytes, s>>>(a);
+    if (!bucketed) {
+        TRACE("k_compare_cm");  // sh.blocks_per_sm: occupancy resolved by the caller
+        k_compare_cm<<<community_grid(kb, num_sms, sh), sh.threads, sh.smem_bytes, s>>>(a);
+        ++launches;
+    }
     TRACE("k_compare_cells");
     k_compare_cells<<<grid_for(n, 256, num_sms, 8), 256, 0, s>>>(a.x, ws.cells, ws.counters, ws.size_b, ws.gacc,
                                                                  ws.status);
@@ -2281,7 +2329,7 @@ int launch_compare(const int *truth, const int *found, long long n, int ka, int 
     TRACE("k_compare_fin");
     k_compare_fin<<<1, 32, 0, s>>>(ws.gacc, ws.status, n, ws.result);
     TRACE(nullptr);
-    launches += 5;
+    launches += 4;
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
