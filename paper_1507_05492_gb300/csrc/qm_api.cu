@@ -1061,6 +1061,18 @@ qm_status qm_compare_partitions(const int32_t *truth, const int32_t *found, int6
         CK(cudaMemcpyAsync((void *)dt, truth, (size_t)n * 4, cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync((void *)df, found, (size_t)n * 4, cudaMemcpyHostToDevice, s));
     }
+    if (compare_small_ok(n, ka, kb)) {
+        num_sms_of(dev);  // kernel set-up
+        const int L = launch_compare_small(dt, df, n, ka, kb, w, (qm_compare *)(pin.ptr() + 256), (int *)pin.ptr(), s,
+                                           trace_begin());
+        if (L < 0) return cuda_fail(cudaGetLastError(), "launch_compare_small");
+        g_launches += L;
+        CK(cudaStreamSynchronize(s));
+        trace_collect();
+        if (*(volatile int *)pin.ptr() & 1) return fail(QM_EINVAL, "a label lies outside its range");
+        std::memcpy(out, pin.ptr() + 256, sizeof(qm_compare));
+        return QM_OK;
+    }
     CK(cudaMemsetAsync(ws.ptr(), 0, w.zero_bytes, s));
     // Comparison runs are the detected communities' member lists (a few hundred
     // entries with few distinct truth labels): small blocks with large warp

@@ -1158,7 +1158,7 @@ __global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *item
             CompareAcc acc;
             compare_acc_zero(acc);
             const int nc = __ldcg(&b.ncells[it]);
-            LateCells lc{late[tid >> 5], 0u};
+            LateCells lc = late_cells(late[tid >> 5], logt);
             for (int i0 = tid & ~31; i0 < nc; i0 += T) {
                 const int i = i0 + (tid & 31);
                 Cell cl{0, 0, 0u, 0u};
@@ -1174,7 +1174,7 @@ __global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *item
                 }
                 cell_terms_warp(cl.n, na, nb, in, x.N, logt, acc, lc);
             }
-            late_cells_flush(x.N, logt, acc, lc);
+            late_cells_flush_block(late[0], (unsigned *)red, x.N, logt, acc, lc);
             for (int c = tid; c < I.K; c += T) {
                 const long long nb = __ldcg(&S.start[c + 1]) - __ldcg(&S.start[c]);
                 if (nb == 0) continue;

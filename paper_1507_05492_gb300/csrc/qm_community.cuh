@@ -1143,37 +1143,39 @@ __device__ __forceinline__ void rowmax_ratio_settle(unsigned long long *slot, lo
 constexpr int LATE_CELL_WORDS = 3 * 64;
 
 struct LateCells {
-    unsigned *late;  // the warp's LATE_CELL_WORDS words of shared memory
-    unsigned n;      // cells waiting, the same in every lane
+    unsigned *late;   // the warp's LATE_CELL_WORDS words of shared memory
+    bool ones;        // whether q1 and lr1 are given (else every cell waits)
+    double q1, lr1;   // 1 / N and log(N / 1)
+    unsigned n = 0u;  // cells waiting, the same in every lane
 };
 
-// The VI and NMI-numerator terms of the last m <= 32 waiting cells.
-__device__ __forceinline__ void late_cells_take(unsigned m, long long N, const double *logt, CompareAcc &acc, LateCells &lc)
+// With the tables of log(N / i) and i / N, or without (logt null).
+__device__ __forceinline__ LateCells late_cells(unsigned *late, const double *logt)
 {
-    lc.n -= m;
-    const unsigned lane = threadIdx.x & 31u;
-    if (lane < m) {
-        const unsigned *w = lc.late + 3u * (lc.n + lane);
-        const long long n = w[0], na = w[1], nb = w[2];
-        const double l1 = cell_log(n, na, nb);
-        const bool tab = logt && n <= LOGT_MAX;
-        acc.vi += fp_from_double(vi_term_l(n, l1), SC_VI);
-        acc.hnum += fp_from_double(nmi_num_term_q(tab ? __ldg(&logt[LOGT_MAX + 1 + n]) : nmi_over(n, N), l1,
-                                                  tab ? __ldg(&logt[n]) : log_ratio(N, n)),
-                                   SC_H);
-    }
-    __syncwarp();
+    return LateCells{late, logt != nullptr, logt ? __ldg(&logt[LOGT_MAX + 2]) : 0.0, logt ? __ldg(&logt[1]) : 0.0};
+}
+
+// The VI and NMI-numerator terms of one waiting cell (three words at w).
+__device__ __forceinline__ void late_cell(const unsigned *w, long long N, const double *logt, CompareAcc &acc)
+{
+    const long long n = w[0], na = w[1], nb = w[2];
+    const double l1 = cell_log(n, na, nb);
+    const bool tab = logt && n <= LOGT_MAX;
+    acc.vi += fp_from_double(vi_term_l(n, l1), SC_VI);
+    acc.hnum += fp_from_double(nmi_num_term_q(tab ? __ldg(&logt[LOGT_MAX + 1 + n]) : nmi_over(n, N), l1,
+                                              tab ? __ldg(&logt[n]) : log_ratio(N, n)),
+                               SC_H);
 }
 
 // Adds the terms of one cell per lane (valid lanes); all 32 lanes call this.
 __device__ __forceinline__ void cell_terms_warp(unsigned n, unsigned na, unsigned nb, bool valid, long long N,
                                                 const double *logt, CompareAcc &acc, LateCells &lc)
 {
-    const bool one = valid && n == 1u && logt && na <= (unsigned)LOGT_MAX && nb <= (unsigned)LOGT_MAX && na * nb > 4u;
+    const bool one = valid && n == 1u && lc.ones && na <= (unsigned)LOGT_MAX && nb <= (unsigned)LOGT_MAX && na * nb > 4u;
     if (one) {
         const double s = __dadd_rn(__ldg(&qm_log_int[na]), __ldg(&qm_log_int[nb]));  // minus the cell's logarithm
         acc.vi += fp_from_double(-s, SC_VI);
-        acc.hnum += fp_from_double(nmi_num_term_q(__ldg(&logt[LOGT_MAX + 2]), -s, __ldg(&logt[1])), SC_H);
+        acc.hnum += fp_from_double(nmi_num_term_q(lc.q1, -s, lc.lr1), SC_H);
     }
     __syncwarp();
     const unsigned wait = __ballot_sync(0xffffffffu, valid && !one);
@@ -1185,12 +1187,31 @@ __device__ __forceinline__ void cell_terms_warp(unsigned n, unsigned na, unsigne
     }
     lc.n += (unsigned)__popc(wait);
     __syncwarp();
-    if (lc.n >= 32u) late_cells_take(32u, N, logt, acc, lc);
+    if (lc.n >= 32u) {
+        lc.n -= 32u;
+        late_cell(lc.late + 3u * (lc.n + (threadIdx.x & 31u)), N, logt, acc);
+        __syncwarp();
+    }
 }
 
-__device__ __forceinline__ void late_cells_flush(long long N, const double *logt, CompareAcc &acc, LateCells &lc)
+// The cells still waiting in the block's warps (fewer than 32 each, in buffers
+// LATE_CELL_WORDS apart from `late` on), gathered so that few warps take them.
+// All threads of the block call this; counts: one word per warp.
+__device__ __forceinline__ void late_cells_flush_block(const unsigned *late, unsigned *counts, long long N,
+                                                       const double *logt, CompareAcc &acc, LateCells &lc)
 {
-    if (lc.n) late_cells_take(lc.n, N, logt, acc, lc);
+    const unsigned wid = threadIdx.x >> 5, lane = threadIdx.x & 31u, W = blockDim.x >> 5;
+    if (lane == 0) counts[wid] = lc.n;
+    block_sync();
+    unsigned total = 0;
+    for (unsigned w = 0; w < W; ++w) total += counts[w];
+    for (unsigned i0 = 32u * wid; i0 < total; i0 += 32u * W) {
+        unsigned i = i0 + lane, w = 0;
+        while (w + 1u < W && i >= counts[w]) i -= counts[w++];
+        if (i0 + lane < total) late_cell(late + w * (unsigned)LATE_CELL_WORDS + 3u * i, N, logt, acc);
+        __syncwarp();
+    }
+    lc.n = 0u;  // (the caller's next block barrier comes before the buffers' next use)
 }
 
 // Row side of the contingency table for truth community a (Eqs. 2-4).

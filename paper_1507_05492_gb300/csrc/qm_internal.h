@@ -232,6 +232,11 @@ int launch_score_fin(const unsigned long long *gacc, const int *status, long lon
 // caller); status bit 1: weight out of range, bit 2: asymmetric.
 int launch_weight_check(const GraphDev &g, const float *wt, int full, int *status, unsigned long long *lim,
                         int num_sms, cudaStream_t s);
+// Comparisons of a few thousand nodes in one kernel: nothing in ws need be
+// zeroed, and the result and status go straight to (pinned) out and out_status.
+bool compare_small_ok(long long n, int ka, int kb);
+int launch_compare_small(const int *truth, const int *found, long long n, int ka, int kb, const CompareWs &ws,
+                         qm_compare *out, int *out_status, cudaStream_t s, TraceFn tr);
 int launch_compare(const int *truth, const int *found, long long n, int ka, int kb,
                    const CompareWs &ws, const Shape &sh, int num_sms, cudaStream_t s, TraceFn tr);
 int count_blocks_per_sm(const Shape &sh);

@@ -632,7 +632,7 @@ __global__ void k_compare_cells(CompareCtx x, const Cell *cells, const int *coun
     if (*status) return;
     CompareAcc acc;
     compare_acc_zero(acc);
-    LateCells lc{late[threadIdx.x >> 5], 0u};
+    LateCells lc = late_cells(late[threadIdx.x >> 5], x.logt);
     const int nc = counters[C_NCELLS];
     for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < nc; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + (threadIdx.x & 31);
@@ -649,7 +649,7 @@ __global__ void k_compare_cells(CompareCtx x, const Cell *cells, const int *coun
         }
         cell_terms_warp(c.n, na, nb, in, x.N, x.logt, acc, lc);
     }
-    late_cells_flush(x.N, x.logt, acc, lc);
+    late_cells_flush_block(late[0], (unsigned *)red, x.N, x.logt, acc, lc);
     flush_compare(acc, g, red);
 }
 
@@ -698,6 +698,8 @@ __global__ void k_compare_fin(const unsigned long long *g, const int *status, lo
     t.kb = g[GC_KB];
     make_compare(t, n, out);
 }
+
+#include "qm_small.cuh"
 
 // ------------------------------------------------------------------ graph validation
 
@@ -1568,6 +1570,7 @@ void prepare_kernels()
     cudaFuncSetAttribute(k_count_long, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
     cudaFuncSetAttribute(k_count_sort<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_DYN_SMEM);
+    cudaFuncSetAttribute(k_compare_small, cudaFuncAttributeMaxDynamicSharedMemorySize, CS_MAX_SLOTS * 10);
     cudaFuncSetAttribute(k_cells_split, cudaFuncAttributeMaxDynamicSharedMemorySize, CELL_SPLIT_SMEM);
     cudaFuncSetAttribute(k_cells_table, cudaFuncAttributeMaxDynamicSharedMemorySize, CELL_TAB_SMEM);
     cudaFuncSetAttribute(k_count_w_big, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM);
@@ -2239,6 +2242,37 @@ int launch_weight_check(const GraphDev &g, const float *wt, int full, int *statu
     k_wcheck<<<grid_for(g.n_arcs, 256, num_sms, 8), 256, 0, s>>>(wt, g.n_arcs, status, lim);
     if (full) k_wsym<<<grid_for(g.n, 256, num_sms, 8), 256, 0, s>>>(g.row_ptr, g.col, wt, g.n, status);
     return cudaGetLastError() == cudaSuccess ? (full ? 2 : 1) : -1;
+}
+
+bool compare_small_ok(long long n, int ka, int kb)
+{
+    return n <= CS_MAX_NODES && ka <= CS_MAX_K && kb <= CS_MAX_K && bits_of(ka) + bits_of(kb) <= 31;
+}
+
+int launch_compare_small(const int *truth, const int *found, long long n, int ka, int kb, const CompareWs &ws,
+                         qm_compare *out, int *out_status, cudaStream_t s, TraceFn tr)
+{
+    CompareSmallArgs a;
+    a.truth = truth;
+    a.found = found;
+    a.n = (int)n;
+    a.ka = ka;
+    a.kb = kb;
+    a.abits = bits_of(ka);
+    a.slots = std::min(CS_MAX_SLOTS, ((int)(4 * n / 3) + 1027) / 4 * 4);
+    a.size_a = ws.size_a;
+    a.rowmax_n = ws.rowmax_n;
+    a.rowmax_r = ws.rowmax_r;
+    a.size_b = ws.size_b;
+    a.colmax = (unsigned *)ws.cursor;
+    a.g = ws.gacc;
+    a.status = ws.status;
+    a.out = out;
+    a.out_status = out_status;
+    TRACE("k_compare_small");
+    k_compare_small<<<CS_CTAS, CS_THREADS, (size_t)a.slots * 10, s>>>(a);
+    TRACE(nullptr);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
 int launch_compare(const int *truth, const int *found, long long n, int ka, int kb,

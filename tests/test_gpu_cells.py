@@ -81,3 +81,26 @@ def test_cells_of_one_node(qm, oracle_mod, n, ka, kb):
     c = qm.compare(da, db, ka, kb)
     check_compare(c, oracle_mod.compare(a, b, ka, kb), f"n={n}")
     assert qm.compare_batched(da, db[None], ka, kb)[0] == c
+
+
+# 16,128 nodes: the largest comparison of the one-kernel path
+@pytest.mark.parametrize("n", [2, 31, 513, 16_127, 16_128, 16_129])
+@pytest.mark.parametrize("kind", ["few", "one found", "distinct", "many ids"])
+def test_small_comparisons(qm, oracle_mod, n, kind):
+    rng = np.random.default_rng(n)
+    ka, kb = {"few": (20, 30), "one found": (9, 1), "distinct": (n, n), "many ids": (1 << 16, (1 << 15) - 1)}[kind]
+    a, b = rng.integers(0, ka, n).astype(np.int32), rng.integers(0, kb, n).astype(np.int32)
+    if kind == "distinct":
+        a, b = rng.permutation(n).astype(np.int32), rng.permutation(n).astype(np.int32)
+    da, db = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+    c, o = qm.compare(da, db, ka, kb), oracle_mod.compare(a, b, ka, kb)
+    assert qm.compare(a, b, ka, kb) == c                            # host labels
+    assert qm.compare_batched(da, db[None], ka, kb)[0] == c         # the other path's bits
+    if min(c["k_truth"], c["k_found"]) > 1:
+        check_compare(c, o, f"{kind} n={n}")
+    for bad in (-1, kb):
+        x = db.clone()
+        x[n - 1] = bad
+        with pytest.raises(qm.QmError) as e:
+            qm.compare(da, x, ka, kb)
+        assert e.value.status == qm.QM_EINVAL
