@@ -236,23 +236,14 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) k_batched(BatchKArgs a)
             const int novf = s_novf;
             for (int i = 0; i < novf; ++i) score_community(x, __ldcg(&ovf[i]), tb, offs, rs, &sacc[0], tid, T, red);
             block_sync();
-            if (tid == 0) {
-                ScoreAcc t = sacc[0];
-                for (int w = 1; w < W; ++w) score_acc_add(t, sacc[w]);
-                ScoreTotals tt;
-                tt.qds_self = t.qds_self;
-                tt.qds_pair = t.qds_pair;
-                tt.dens = t.dens;
-                tt.contr = t.contr;
-                tt.expn = t.expn;
-                tt.cond = t.cond;
-                tt.vol2 = (i128)t.vol2;
-                tt.ein = t.ein;
-                tt.eout = t.eout;
-                tt.nonempty = t.nonempty;
-                tt.slots = t.slots;
-                tt.cnt2 = t.cnt2;
-                make_quality(tt, n, I.n_arcs / 2, I.out_q);
+            if (tid < 32) {
+                if (tid == 0) {
+                    ScoreAcc t = sacc[0];
+                    for (int w = 1; w < W; ++w) score_acc_add(t, sacc[w]);
+                    score_words(t, red);
+                }
+                __syncwarp();
+                quality_warp(red, n, I.n_arcs / 2, false, I.out_q);
             }
         }
 
@@ -296,27 +287,23 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) k_batched(BatchKArgs a)
             CompareAcc racc;
             compare_acc_zero(racc);
             for (int r = tid; r < kt; r += T) compare_row(x, r, racc);
-            CompareTotals t;
-            t.hden = group_sum_i128(racc.hden, T, red);
-            t.f = group_sum_i128(racc.f, T, red);
-            t.sa = group_sum_u64(racc.sa, T, red);
-            t.nvd = group_sum_u64(racc.nvd, T, red);
-            t.ka = group_sum_u64(racc.ka, T, red);
-            if (tid == 0) {
-                CompareAcc c = cacc[0];
-                for (int w = 1; w < W; ++w) compare_acc_add(c, cacc[w]);
-                t.vi = c.vi;
-                t.hnum = c.hnum;
-                t.hden += c.hden;
-                t.f += c.f;
-                t.a11 = c.a11;
-                t.sa += c.sa;
-                t.sb = c.sb;
-                t.nvd += c.nvd;
-                t.cells = c.cells;
-                t.ka += c.ka;
-                t.kb = c.kb;
-                make_compare(t, n, I.out_c);
+            const i128 hden = group_sum_i128(racc.hden, T, red), f = group_sum_i128(racc.f, T, red);
+            const unsigned long long sa = group_sum_u64(racc.sa, T, red), nvd = group_sum_u64(racc.nvd, T, red),
+                                     ka = group_sum_u64(racc.ka, T, red);
+            block_sync();
+            if (tid < 32) {
+                if (tid == 0) {
+                    CompareAcc t = cacc[0];
+                    for (int w = 1; w < W; ++w) compare_acc_add(t, cacc[w]);
+                    t.hden += hden;
+                    t.f += f;
+                    t.sa += sa;
+                    t.nvd += nvd;
+                    t.ka += ka;
+                    compare_words(t, red);
+                }
+                __syncwarp();
+                compare_warp(red, n, I.out_c);
             }
         }
         block_sync();
@@ -1104,45 +1091,61 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 1) k_bu_cells(BuArgs a)
 constexpr int BU_FIN_THREADS = 256;
 constexpr int BU_CELLS_SMEM = 48 * 1024;  // shared memory of a k_bu_cells block at most
 
-// One block per candidate: the FP64 terms of every community record (Eq. (9),
-// Sec. II-B.3) and of every contingency cell, column and row (Eqs. 1-7), all
-// lanes busy, summed in fixed point; then the final results.
-__global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *items, int count, BatchUnits b)
+// Word w of rank r's copy of a shared array (r a rank of this cluster).
+__device__ __forceinline__ unsigned long long cluster_word(const unsigned long long *w, int r)
 {
-    __shared__ unsigned long long red[72];
+    unsigned a;
+    unsigned long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(w)), "r"(r));
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// One cluster of cl blocks per candidate: the FP64 terms of every community
+// record (Eq. (9), Sec. II-B.3) and of every contingency cell, column and row
+// (Eqs. 1-7), all lanes busy, summed in fixed point; then the final results.
+// Bound by FP64, of which an SM issues two operations a cycle, so the candidates
+// are spread over the SMs (32 candidates on graphs of 10^4 nodes, one block each:
+// 63 us; eight blocks each: the whole call 420 -> 381 us.  256 candidates on a graph
+// of 10^5 nodes, four blocks each: the call 7.23 -> 7.06 ms).  No kernel from here on
+// writes a status, so all blocks of a cluster skip the same candidates.
+__global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *items, int count, BatchUnits b, int cl)
+{
     __shared__ unsigned late[BU_FIN_THREADS / 32][LATE_CELL_WORDS];
-    const int tid = threadIdx.x, T = blockDim.x;
-    for (int it = blockIdx.x; it < count; it += gridDim.x) {
+    __shared__ unsigned wait[64];
+    __shared__ unsigned long long part[BU_FIN_THREADS / 32][GS_COUNT], sum_s[GS_COUNT], sum_c[GC_COUNT];
+    static_assert(GC_COUNT <= GS_COUNT && GS_COUNT <= 32, "one warp adds the words");
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, W = BU_FIN_THREADS / 32;
+    const int rank = (int)blockIdx.x % cl, T = cl * BU_FIN_THREADS, gt = rank * BU_FIN_THREADS + tid;
+    for (int it = blockIdx.x / cl; it < count; it += gridDim.x / cl) {
         const BatchItem I = items[it];
         if (bu_dead(I)) continue;
         const BuSlice S = bu_slice(b, it);
         const long long E = I.n_arcs / 2;
-        if (I.flags & 1) {
+        const bool score = I.flags & 1, cmp = (I.flags & 2) && I.truth && S.cells;
+        if (score) {
             ScoreAcc acc;
             score_acc_zero(acc);
-            for (int c = tid; c < I.K; c += T) {
+            for (int c = gt; c < I.K; c += T) {
                 const long long size = __ldcg(&S.start[c + 1]) - __ldcg(&S.start[c]);
                 if (size <= 0) continue;
-                double pen, qs, dens, contr, expn, cond;
-                terms_from_record(S.rec + (size_t)c * REC_WORDS, size, E, acc, &pen, &qs, &dens, &contr, &expn, &cond);
+                double qs, dens, contr, expn, cond;
+                terms_from_record(S.rec + (size_t)c * REC_WORDS, size, E, acc, nullptr, &qs, &dens, &contr, &expn, &cond);
             }
-            ScoreTotals t;
-            t.qds_self = group_sum_i128(acc.qds_self, T, red);
-            t.qds_pair = group_sum_i128(acc.qds_pair, T, red);
-            t.dens = group_sum_i128(acc.dens, T, red);
-            t.contr = group_sum_i128(acc.contr, T, red);
-            t.expn = group_sum_i128(acc.expn, T, red);
-            t.cond = group_sum_i128(acc.cond, T, red);
-            t.vol2 = group_sum_i128((i128)acc.vol2, T, red);
-            t.ein = group_sum_u64(acc.ein, T, red);
-            t.eout = group_sum_u64(acc.eout, T, red);
-            t.nonempty = group_sum_u64(acc.nonempty, T, red);
-            t.slots = group_sum_u64(acc.slots, T, red);
-            t.cnt2 = group_sum_u64(acc.cnt2, T, red);
-            if (tid == 0) make_quality(t, I.n, E, I.out_q);
+            __syncwarp();
+            score_words_warp(acc, 0, part[wid]);
+            block_sync();
+            if (tid < GS_COUNT) {
+                unsigned long long t = 0;
+                for (int w = 0; w < W; ++w) t += part[w][tid];
+                sum_s[tid] = t;
+            }
+            block_sync();
         }
-        if ((I.flags & 2) && I.truth && S.cells) {
-            CompareCtx x;
+        CompareCtx x;
+        CompareAcc acc;
+        compare_acc_zero(acc);
+        if (cmp) {
             x.truth = I.truth;
             x.tl = nullptr;
             x.members = S.members;
@@ -1155,12 +1158,10 @@ __global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *item
             x.kb = I.K;
             x.err = I.status;
             const double *logt = I.n == b.logt_n ? b.logt : nullptr;
-            CompareAcc acc;
-            compare_acc_zero(acc);
             const int nc = __ldcg(&b.ncells[it]);
-            LateCells lc = late_cells(late[tid >> 5], logt);
-            for (int i0 = tid & ~31; i0 < nc; i0 += T) {
-                const int i = i0 + (tid & 31);
+            LateCells lc = late_cells(late[wid], logt);
+            for (int i0 = gt & ~31; i0 < nc; i0 += T) {
+                const int i = i0 + lane;
                 Cell cl{0, 0, 0u, 0u};
                 if (i < nc) cl = S.cells[i];
                 const bool in = i < nc && QM_CHK(cl.a, x.ka, 30) && QM_CHK(cl.b, x.kb, 31);
@@ -1174,39 +1175,58 @@ __global__ void __launch_bounds__(BU_FIN_THREADS) k_bu_fin(const BatchItem *item
                 }
                 cell_terms_warp(cl.n, na, nb, in, x.N, logt, acc, lc);
             }
-            late_cells_flush_block(late[0], (unsigned *)red, x.N, logt, acc, lc);
-            for (int c = tid; c < I.K; c += T) {
+            late_cells_flush_block(late[0], wait, x.N, logt, acc, lc);
+            for (int c = gt; c < I.K; c += T) {
                 const long long nb = __ldcg(&S.start[c + 1]) - __ldcg(&S.start[c]);
                 if (nb == 0) continue;
                 acc.sb += (unsigned long long)(nb * (nb - 1) / 2);
                 acc.hden += fp_from_double(entropy_term(nb, x.N), SC_H);
                 acc.kb += 1;
             }
-            __threadfence();
-            block_sync();  // this candidate's row maxima are complete
-            for (int r = tid; r < x.ka; r += T) {
-                rowmax_ratio_settle(&S.rowmax_r[r], __ldcg(&S.size_a[r]));
-                compare_row(x, r, acc);
-            }
-            CompareTotals t;
-            t.vi = group_sum_i128(acc.vi, T, red);
-            t.hnum = group_sum_i128(acc.hnum, T, red);
-            t.hden = group_sum_i128(acc.hden, T, red);
-            t.f = group_sum_i128(acc.f, T, red);
-            t.a11 = group_sum_u64(acc.a11, T, red);
-            t.sa = group_sum_u64(acc.sa, T, red);
-            t.sb = group_sum_u64(acc.sb, T, red);
-            t.nvd = group_sum_u64(acc.nvd, T, red);
-            t.ka = group_sum_u64(acc.ka, T, red);
-            t.kb = group_sum_u64(acc.kb, T, red);
-            if (tid == 0) {
-                t.nvd += __ldcg(&b.gcell[2 * (size_t)it]);
-                t.cells = __ldcg(&b.gcell[2 * (size_t)it + 1]);
-                make_compare(t, x.N, I.out_c);
-            }
         }
+        __threadfence();
+        cluster_sync();  // this candidate's row maxima and score sums are complete
+        if (score && rank == 0 && wid == 0) {
+            unsigned long long t = 0;
+            if (lane < GS_COUNT)
+                for (int r = 0; r < cl; ++r) t += cluster_word(&sum_s[lane], r);
+            if (lane < GS_COUNT) part[0][lane] = t;
+            __syncwarp();
+            quality_warp(part[0], I.n, E, false, I.out_q);
+            __syncwarp();
+        }
+        if (!cmp) {
+            // (the sums of the next candidate wait until these were read)
+            cluster_sync();
+            continue;
+        }
+        for (int r = gt; r < x.ka; r += T) {
+            rowmax_ratio_settle(&S.rowmax_r[r], __ldcg(&S.size_a[r]));
+            compare_row(x, r, acc);
+        }
+        __syncwarp();
+        compare_words_warp(acc, part[wid]);
         block_sync();
+        if (tid < GC_COUNT) {
+            unsigned long long t = 0;
+            for (int w = 0; w < W; ++w) t += part[w][tid];
+            sum_c[tid] = t;
+        }
+        cluster_sync();
+        if (rank == 0 && wid == 0) {
+            unsigned long long t = 0;
+            if (lane < GC_COUNT)
+                for (int r = 0; r < cl; ++r) t += cluster_word(&sum_c[lane], r);
+            if (lane == GC_NVD) t += __ldcg(&b.gcell[2 * (size_t)it]);
+            if (lane == GC_CELLS) t = __ldcg(&b.gcell[2 * (size_t)it + 1]);
+            if (lane < GC_COUNT) part[0][lane] = t;
+            __syncwarp();
+            compare_warp(part[0], x.N, I.out_c);
+            __syncwarp();
+        }
+        block_sync();  // part is free again
     }
+    cluster_sync();  // no block leaves while its sums are read
 }
 
 int batch_units_blocks_per_sm(const Shape &sh)
@@ -1261,7 +1281,20 @@ int launch_batch_units(const BatchItem *items_dev, int count, const BatchUnits &
             ++L;
         }
     }
-    k_bu_fin<<<std::min(count, num_sms * 8), BU_FIN_THREADS, 0, s>>>(items_dev, count, bb);
+    // blocks per candidate: enough for four blocks an SM when there are few candidates
+    int cl = 1;
+    while (cl < 8 && (long long)count * cl < 4LL * num_sms) cl *= 2;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)(std::min(count, num_sms * 8) * cl));
+    lc.blockDim = dim3(BU_FIN_THREADS);
+    lc.stream = s;
+    cudaLaunchAttribute la{};
+    la.id = cudaLaunchAttributeClusterDimension;
+    la.val.clusterDim.x = (unsigned)cl;
+    la.val.clusterDim.y = la.val.clusterDim.z = 1;
+    lc.attrs = &la;
+    lc.numAttrs = 1;
+    cudaLaunchKernelEx(&lc, k_bu_fin, (const BatchItem *)items_dev, count, bb, cl);
     ++L;
     return cudaGetLastError() == cudaSuccess ? L : -1;
 }

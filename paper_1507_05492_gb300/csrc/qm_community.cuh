@@ -1097,7 +1097,7 @@ __device__ __forceinline__ void terms_from_record(const unsigned long long *rc, 
     acc.ein += (unsigned long long)ein;
     acc.eout += (unsigned long long)eout;
     acc.nonempty += 1;
-    *pen_out = pair_penalty_own(full, size, E);
+    if (pen_out) *pen_out = pair_penalty_own(full, size, E);
     *qs_out = qs;
     *dens_o = dens;
     *contr_o = contr;

@@ -633,24 +633,10 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_score(CoverScoreArgs a)
 __global__ void k_cover_score_fin(const unsigned long long *g, const int *status, long long n, long long E,
                                   qm_quality *out)
 {
-    if (threadIdx.x != 0 || *status) return;
-    ScoreTotals t;
-    t.qds_self = limbs_get(g + GS_QDS_SELF);
-    t.qds_pair = limbs_get(g + GS_QDS_PAIR);
-    t.dens = limbs_get(g + GS_DENS);
-    t.contr = limbs_get(g + GS_CONTR);
-    t.expn = limbs_get(g + GS_EXPN);
-    t.cond = limbs_get(g + GS_COND);
-    t.vol2 = limbs_get(g + GS_VOL2);
-    t.ein = g[GS_EIN];
-    t.eout = g[GS_EOUT];
-    t.nonempty = g[GS_NONEMPTY];
-    t.slots = g[GS_SLOTS];
-    t.cnt2 = g[GS_CNT2];
-    qm_quality r;
-    make_quality(t, n, E, &r);
-    r.cut_edges_total = (long long)t.eout;
-    *out = r;
+    if (*status) return;
+    quality_warp(g, n, E, false, out);
+    __syncwarp();
+    if (threadIdx.x == 0) out->cut_edges_total = (long long)g[GS_EOUT];
 }
 
 // ------------------------------------------------------------------ comparison
@@ -919,20 +905,14 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_pairs(CoverCmpArgs a)
 
 __global__ void k_cover_compare_fin(const unsigned long long *g, const int *status, long long n, qm_compare *out)
 {
-    if (threadIdx.x != 0 || *status) return;
-    CompareTotals t;
-    t.vi = limbs_get(g + GC_VI);
-    t.hnum = limbs_get(g + GC_HNUM);
-    t.hden = limbs_get(g + GC_HDEN);
-    t.f = limbs_get(g + GC_F);
-    t.a11 = g[GC_A11] - g[GC_A11_CORR];
-    t.sa = g[GC_SA] - g[GC_SAME_A_CORR];
-    t.sb = g[GC_SB] - g[GC_SAME_B_CORR];
-    t.nvd = g[GC_NVD];
-    t.cells = g[GC_CELLS];
-    t.ka = g[GC_KA];
-    t.kb = g[GC_KB];
-    make_compare(t, n, out);
+    __shared__ unsigned long long w[GC_COUNT];
+    if (*status) return;
+    const int lane = threadIdx.x;
+    if (lane < GC_COUNT)
+        w[lane] = g[lane] - (lane == GC_A11 ? g[GC_A11_CORR] : lane == GC_SA ? g[GC_SAME_A_CORR]
+                             : lane == GC_SB ? g[GC_SAME_B_CORR] : 0ull);
+    __syncwarp();
+    compare_warp(w, n, out);
 }
 
 // ------------------------------------------------------------------ launchers

@@ -140,6 +140,36 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
     return v;
 }
 
+// Warp totals (modulo 2^128 and 2^64, valid in every lane): 27-bit chunks, each
+// added by one redux, instead of five rounds of shuffles and carries.
+__device__ __forceinline__ i128 warp_sum_i128_redux(i128 v)
+{
+    constexpr unsigned M = (1u << 27) - 1u;
+    const u128 u = (u128)v;
+    u128 r = 0;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) r += (u128)__reduce_add_sync(0xffffffffu, (unsigned)(u >> (27 * k)) & M) << (27 * k);
+    return (i128)r;
+}
+
+__device__ __forceinline__ unsigned long long warp_sum_u64_redux(unsigned long long v)
+{
+    constexpr unsigned M = (1u << 27) - 1u;
+    unsigned long long r = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        r += (unsigned long long)__reduce_add_sync(0xffffffffu, (unsigned)(v >> (27 * k)) & M) << (27 * k);
+    return r;
+}
+
+// Every thread of the cluster has arrived, and sees the others' global and
+// shared writes from before.  (A hardware barrier of the resident cluster.)
+__device__ __forceinline__ void cluster_sync()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- exact pair sums
 //
 // The split penalty of Eq. (9) for community i needs S_i = sum_j |E_ij|^2 / |c_j|

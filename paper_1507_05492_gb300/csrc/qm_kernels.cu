@@ -24,7 +24,7 @@ namespace qm {
 using namespace qmk;
 
 enum { C_BIG_COUNT = 0, C_BIG_NEXT = 1, C_SMALL_NEXT = 2, C_OVF_COUNT = 3, C_OVF_NEXT = 4, C_SMALL_COUNT = 5,
-       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_BAD = 9, C_MID_NEXT = 10,
+       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_BAD = 9, C_MID_NEXT = 10, C_TERMS_DONE = 11,
        C_BX_COUNT = 12 /* two words */ };
 
 constexpr int SCAN_TILE = 4096;   // elements per block in the multi-block scan
@@ -481,25 +481,12 @@ __global__ void __launch_bounds__(1024) k_score_cm(ScoreKArgs a)
     if (threadIdx.x == 0) flush_score(sacc, W, a.gacc);
 }
 
+// One warp (see quality_warp).
 __global__ void k_score_fin(const unsigned long long *g, const int *status, long long n, long long E,
                             qm_quality *out, int weighted)
 {
-    if (threadIdx.x != 0 || *status) return;
-    ScoreTotals t;
-    t.qds_self = limbs_get(g + GS_QDS_SELF);
-    t.qds_pair = limbs_get(g + GS_QDS_PAIR);
-    t.dens = limbs_get(g + GS_DENS);
-    t.contr = limbs_get(g + GS_CONTR);
-    t.expn = limbs_get(g + GS_EXPN);
-    t.cond = limbs_get(g + GS_COND);
-    t.vol2 = limbs_get(g + GS_VOL2);
-    t.ein = g[GS_EIN];
-    t.eout = g[GS_EOUT];
-    t.nonempty = g[GS_NONEMPTY];
-    t.slots = g[GS_SLOTS];
-    t.cnt2 = g[GS_CNT2];
-    make_quality(t, n, E, out);
-    if (weighted) out->modularity = fp_to_double(limbs_get(g + GS_QW), SC_QDS);
+    if (*status) return;
+    quality_warp(g, n, E, weighted != 0, out);
 }
 
 // ------------------------------------------------------------------ compare
@@ -514,25 +501,16 @@ struct CompareKArgs {
     SmemPlan plan;
 };
 
-__device__ __forceinline__ void flush_compare(const CompareAcc &acc, unsigned long long *g,
-                                              unsigned long long *red)
+// A block's sums (blocks of up to 256 threads) into the comparison's words.
+__device__ __forceinline__ void flush_compare(const CompareAcc &acc, unsigned long long *g)
 {
-    const int T = blockDim.x;
-    i128 v;
-    v = group_sum_i128(acc.vi, T, red);
-    if (threadIdx.x == 0) limbs_add(g + GC_VI, v);
-    v = group_sum_i128(acc.hnum, T, red);
-    if (threadIdx.x == 0) limbs_add(g + GC_HNUM, v);
-    v = group_sum_i128(acc.hden, T, red);
-    if (threadIdx.x == 0) limbs_add(g + GC_HDEN, v);
-    v = group_sum_i128(acc.f, T, red);
-    if (threadIdx.x == 0) limbs_add(g + GC_F, v);
-    const unsigned long long *src[7] = {&acc.a11, &acc.sa, &acc.sb, &acc.nvd, &acc.cells, &acc.ka, &acc.kb};
-    const int dst[7] = {GC_A11, GC_SA, GC_SB, GC_NVD, GC_CELLS, GC_KA, GC_KB};
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        const unsigned long long u = group_sum_u64(*src[k], T, red);
-        if (threadIdx.x == 0 && u) atomicAdd(g + dst[k], u);
+    __shared__ unsigned long long part[8][GC_COUNT];
+    compare_words_warp(acc, part[threadIdx.x >> 5]);
+    block_sync();
+    if (threadIdx.x < GC_COUNT) {
+        unsigned long long t = 0;
+        for (unsigned w = 0; w < blockDim.x / 32; ++w) t += part[w][threadIdx.x];
+        if (t) atomicAdd(g + threadIdx.x, t);
     }
 }
 
@@ -609,7 +587,6 @@ __global__ void __launch_bounds__(1024) k_compare_cm(CompareKArgs a)
 
 __global__ void k_compare_rows(CompareCtx x, unsigned long long *g, const int *status)
 {
-    __shared__ unsigned long long red[72];
     if (*status) return;
     CompareAcc acc;
     compare_acc_zero(acc);
@@ -617,7 +594,7 @@ __global__ void k_compare_rows(CompareCtx x, unsigned long long *g, const int *s
         rowmax_ratio_settle(&x.rowmax_r[a], __ldcg(&x.size_a[a]));
         compare_row(x, a, acc);
     }
-    flush_compare(acc, g, red);
+    flush_compare(acc, g);
 }
 
 // Terms of every contingency cell (Eqs. 1-4), in parallel over the cell list:
@@ -650,7 +627,7 @@ __global__ void k_compare_cells(CompareCtx x, const Cell *cells, const int *coun
         cell_terms_warp(c.n, na, nb, in, x.N, x.logt, acc, lc);
     }
     late_cells_flush_block(late[0], (unsigned *)red, x.N, x.logt, acc, lc);
-    flush_compare(acc, g, red);
+    flush_compare(acc, g);
 }
 
 // log(N / n) and n / N for n = 1 .. LOGT_MAX (contingency cells and community
@@ -667,7 +644,6 @@ __global__ void k_log_table(double *logt, long long N)
 // Column side of every found community b: C(|b|, 2), its entropy term, the count.
 __global__ void k_compare_cols(const int *size_b, int kb, long long N, unsigned long long *g, const int *status)
 {
-    __shared__ unsigned long long red[72];
     if (*status) return;
     CompareAcc acc;
     compare_acc_zero(acc);
@@ -678,25 +654,14 @@ __global__ void k_compare_cols(const int *size_b, int kb, long long N, unsigned 
         acc.hden += fp_from_double(entropy_term(nb, N), SC_H);
         acc.kb += 1;
     }
-    flush_compare(acc, g, red);
+    flush_compare(acc, g);
 }
 
+// One warp (see compare_warp).
 __global__ void k_compare_fin(const unsigned long long *g, const int *status, long long n, qm_compare *out)
 {
-    if (threadIdx.x != 0 || *status) return;
-    CompareTotals t;
-    t.vi = limbs_get(g + GC_VI);
-    t.hnum = limbs_get(g + GC_HNUM);
-    t.hden = limbs_get(g + GC_HDEN);
-    t.f = limbs_get(g + GC_F);
-    t.a11 = g[GC_A11];
-    t.sa = g[GC_SA];
-    t.sb = g[GC_SB];
-    t.nvd = g[GC_NVD];
-    t.cells = g[GC_CELLS];
-    t.ka = g[GC_KA];
-    t.kb = g[GC_KB];
-    make_compare(t, n, out);
+    if (*status) return;
+    compare_warp(g, n, out);
 }
 
 #include "qm_small.cuh"
@@ -1507,41 +1472,66 @@ int sort_blocks_per_sm(const Shape &sh)
     return nb;
 }
 
-// Block reduction of per-thread sums into the partition's global limbs.
-__device__ __forceinline__ void flush_score_threads(const ScoreAcc &acc, unsigned long long *g,
-                                                    unsigned long long *red)
+// Where the terms' last block puts the results (done null: no results are asked
+// for, as for one shard's sums).
+struct ScoreOut {
+    int *done;  // blocks finished, zero at the start
+    long long n, E;
+    qm_quality *out;
+    int weighted;
+};
+
+// Block sums (blocks of up to 256 threads) into the partition's words; the last
+// block to finish forms the results from them, which saves a launch.
+__device__ __forceinline__ void flush_terms(const ScoreAcc &acc, i128 qw, unsigned long long *g, const ScoreOut &o)
 {
-    const int T = blockDim.x;
-    const i128 v[7] = {acc.qds_self, acc.qds_pair, acc.dens, acc.contr, acc.expn, acc.cond, (i128)acc.vol2};
-    const int at[7] = {GS_QDS_SELF, GS_QDS_PAIR, GS_DENS, GS_CONTR, GS_EXPN, GS_COND, GS_VOL2};
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        const i128 t = group_sum_i128(v[k], T, red);
-        if (threadIdx.x == 0) limbs_add(g + at[k], t);
+    __shared__ unsigned long long part[8][GS_COUNT];
+    const int tid = threadIdx.x;
+    score_words_warp(acc, qw, part[tid >> 5]);
+    block_sync();
+    if (tid >= 32) return;
+    if (tid < GS_COUNT) {
+        unsigned long long t = 0;
+        for (unsigned w = 0; w < blockDim.x / 32; ++w) t += part[w][tid];
+        if (t) atomicAdd(g + tid, t);
     }
-    const unsigned long long u[5] = {acc.ein, acc.eout, acc.nonempty, acc.slots, acc.cnt2};
-    const int au[5] = {GS_EIN, GS_EOUT, GS_NONEMPTY, GS_SLOTS, GS_CNT2};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const unsigned long long t = group_sum_u64(u[k], T, red);
-        if (threadIdx.x == 0 && t) atomicAdd(g + au[k], t);
-    }
+    if (!o.done) return;
+    __threadfence();
+    __syncwarp();
+    int at = 0;
+    if (tid == 0) at = atomicAdd(o.done, 1);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (at != (int)gridDim.x - 1) return;
+    __threadfence();
+    if (tid < GS_COUNT) part[0][tid] = __ldcg(&g[tid]);
+    __syncwarp();
+    quality_warp(part[0], o.n, o.E, o.weighted != 0, o.out);
+}
+
+// Threads of a terms block: small enough that few communities still spread over
+// every SM.  A community's eight divisions are FP64, of which an SM issues two a
+// cycle, so 256 communities on one SM take 14 us and 32 take 2 (10^4 nodes, 400
+// communities: the call 80 -> 75 us, with the results formed by the last block).
+static int terms_threads(long long K, int num_sms)
+{
+    int T = 32;
+    while (T < 256 && K > (long long)T * num_sms) T *= 2;
+    return T;
 }
 
 // FP64 terms of every community from the phase-B records, all in parallel.
 __global__ void k_score_terms(const int *start, const unsigned long long *cv, const unsigned long long *rec, int K, long long E, PerCommDev pc,
-                              unsigned long long *g, const int *status, Shard own)
+                              unsigned long long *g, const int *status, Shard own, ScoreOut o)
 {
-    __shared__ unsigned long long red[72];
     if (*status) return;
     ScoreAcc acc;
     score_acc_zero(acc);
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < K; c += gridDim.x * blockDim.x) {
         const long long size = cv ? (long long)(cv[c] >> VOL_BITS) : start[c + 1] - start[c];
         if (size == 0 || !own.owns(c)) continue;
-        double pen, qs, dens, contr, expn, cond;
+        double pen = 0.0, qs, dens, contr, expn, cond;
         const unsigned long long *rc = rec + (size_t)c * REC_WORDS;
-        terms_from_record(rc, size, E, acc, &pen, &qs, &dens, &contr, &expn, &cond);
+        terms_from_record(rc, size, E, acc, pc.qds ? &pen : nullptr, &qs, &dens, &contr, &expn, &cond);
         if (pc.size) pc.size[c] = size;
         if (pc.ein) pc.ein[c] = (long long)(rc[REC_SAME] / 2);
         if (pc.eout) pc.eout[c] = (long long)(rc[REC_VOL] - rc[REC_SAME]);
@@ -1551,7 +1541,7 @@ __global__ void k_score_terms(const int *start, const unsigned long long *cv, co
         if (pc.cond) pc.cond[c] = cond;
         if (pc.qds) pc.qds[c] = __dsub_rn(qs, pen);
     }
-    flush_score_threads(acc, g, red);
+    flush_terms(acc, 0, g, o);
 }
 
 #include "qm_weighted.cuh"
@@ -1885,14 +1875,11 @@ static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, con
     PerCommDev pcd{};
     if (pc) pcd = *pc;
     TRACE("k_score_terms_w");
-    k_score_terms_w<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(ws.cv, ws.rec, ws.recw, ws.wl, K, g.n_arcs / 2,
-                                                                 g.w_lo, g.w_hi, pcd, ws.gacc, ws.status, own);
-    launches += 2;
-    if (own.p == 1) {
-        TRACE("k_score_fin");
-        k_score_fin<<<1, 32, 0, s>>>(ws.gacc, ws.status, g.n, g.n_arcs / 2, ws.result, 1);
-        ++launches;
-    }
+    const ScoreOut so{own.p == 1 ? ws.counters + C_TERMS_DONE : nullptr, g.n, g.n_arcs / 2, ws.result, 1};
+    const int tt = terms_threads(K, num_sms);
+    k_score_terms_w<<<grid_for(K, tt, num_sms, 2), tt, 0, s>>>(ws.cv, ws.rec, ws.recw, ws.wl, K, g.n_arcs / 2, g.w_lo,
+                                                               g.w_hi, pcd, ws.gacc, ws.status, own, so);
+    ++launches;
     TRACE(nullptr);
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
@@ -1986,7 +1973,7 @@ static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const 
 
 // The two-phase plain scoring pipeline:
 //   k_hist_vol -> k_vscan_* (segment bases) -> k_rows
-//   -> k_rows_classify -> k_count_* -> k_score_terms -> k_score_fin
+//   -> k_rows_classify -> k_count_* -> k_score_terms (and the results)
 // or, for the half-edge and binned gathers, members in community order:
 //   k_hist -> scan (sizes) -> k_scatter_deg -> scan (member degrees = arc offsets)
 //   -> k_expand_half / k_expand_bin -> k_classify -> ...
@@ -2182,14 +2169,12 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     PerCommDev pcd{};
     if (pc) pcd = *pc;
     TRACE("k_score_terms");
-    k_score_terms<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(ws.start, rows ? ws.cv : nullptr, ws.rec, K, g.n_arcs / 2, pcd, ws.gacc,
-                                                               ws.status, own);
+    // (a shard's caller reads the partial sums instead of the results)
+    const ScoreOut so{shard_p == 1 ? ws.counters + C_TERMS_DONE : nullptr, n, g.n_arcs / 2, ws.result, 0};
+    const int tt = terms_threads(K, num_sms);
+    k_score_terms<<<grid_for(K, tt, num_sms, 2), tt, 0, s>>>(ws.start, rows ? ws.cv : nullptr, ws.rec, K,
+                                                             g.n_arcs / 2, pcd, ws.gacc, ws.status, own, so);
     ++launches;
-    if (shard_p == 1) {  // a shard's caller reads the partial sums instead
-        TRACE("k_score_fin");
-        k_score_fin<<<1, 32, 0, s>>>(ws.gacc, ws.status, n, g.n_arcs / 2, ws.result, 0);
-        ++launches;
-    }
     TRACE(nullptr);
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
@@ -2224,8 +2209,9 @@ int launch_cover_runs(const CoverRuns &r, int K, long long E, unsigned long long
     t.plan = plan_smem(CB_THREADS, CB_SMEM);
     k_count_tab<CT_ABOVE><<<(int)std::min<long long>((long long)num_sms * CT_BLOCKS, K), CT_THREADS, 0, s>>>(t);
     k_count_big<CT_ABOVE><<<std::min(2 * num_sms, K), CB_THREADS, CB_SMEM, s>>>(t);
-    k_score_terms<<<grid_for(K, 256, num_sms, 2), 256, 0, s>>>(nullptr, r.cv, r.rec, K, E, PerCommDev{}, gacc, r.gate,
-                                                               own);
+    const int tt = terms_threads(K, num_sms);
+    k_score_terms<<<grid_for(K, tt, num_sms, 2), tt, 0, s>>>(nullptr, r.cv, r.rec, K, E, PerCommDev{}, gacc, r.gate, own,
+                                                             ScoreOut{});
     return cudaGetLastError() == cudaSuccess ? 4 : -1;
 }
 

@@ -10,9 +10,8 @@
 // memory, with a cluster barrier between the phases; and the result is written
 // straight to the caller's pinned memory.  The terms are the other path's
 // functions and every sum is exact, so the results are the same bits.
-// 10^4 nodes: 109 -> 69 us a call (the kernel 37 us, bound by its chains of
-// dependent FP64 operations: a division, a logarithm and a barrier after
-// another); beyond CS_MAX_NODES a block's shared memory may not hold its cells.
+// 10^4 nodes: 109 -> 54 us a call (bound by its chains of dependent FP64
+// operations: a division, a logarithm and a barrier after another); beyond CS_MAX_NODES a block's shared memory may not hold its cells.
 // Included inside namespace qm of qm_kernels.cu, after the helpers it uses.
 
 constexpr int CS_CTAS = 8, CS_THREADS = 512;
@@ -32,31 +31,11 @@ struct CompareSmallArgs {
     int *out_status;
 };
 
-// Every thread of the cluster has arrived, and sees the others' global and
-// shared writes from before.  (A hardware barrier of the resident cluster.)
-__device__ __forceinline__ void cluster_sync()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// Warp total of a 128-bit sum (modulo 2^128, valid in every lane): five 27-bit
-// chunks, each added by one redux.
-__device__ __forceinline__ i128 warp_sum_i128_redux(i128 v)
-{
-    constexpr unsigned M = (1u << 27) - 1u;
-    const u128 u = (u128)v;
-    u128 r = 0;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) r += (u128)__reduce_add_sync(0xffffffffu, (unsigned)(u >> (27 * k)) & M) << (27 * k);
-    return (i128)r;
-}
-
 __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS) k_compare_small(CompareSmallArgs a)
 {
     extern __shared__ __align__(16) unsigned sm_small[];
     __shared__ int s_cells;
-    __shared__ unsigned wait_s[CS_THREADS / 32][64];
+    __shared__ __align__(8) unsigned wait_s[CS_THREADS / 32][64];
     __shared__ unsigned late_s[CS_THREADS / 32][LATE_CELL_WORDS];
     __shared__ double s_ones[2];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, rank = blockIdx.x;
@@ -212,39 +191,24 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS) k_
         acc.ka += 1;
     }
     __syncwarp();
-    // every count is below 2^32 here (C(n, 2) of at most 2^14.2 nodes)
-    const i128 v4[4] = {acc.vi, acc.hnum, acc.hden, acc.f};
-    const int at4[4] = {GC_VI, GC_HNUM, GC_HDEN, GC_F};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const i128 t = warp_sum_i128_redux(v4[k]);
-        if (lane == 0 && t != 0) limbs_add(a.g + at4[k], t);
-    }
-    const unsigned long long u7[7] = {acc.a11, acc.sa, acc.sb, acc.nvd, acc.cells, acc.ka, acc.kb};
-    const int at7[7] = {GC_A11, GC_SA, GC_SB, GC_NVD, GC_CELLS, GC_KA, GC_KB};
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        const unsigned t = __reduce_add_sync(0xffffffffu, (unsigned)u7[k]);
-        if (lane == 0 && t) atomicAdd(a.g + at7[k], (unsigned long long)t);
+    static_assert(2 * GC_COUNT <= 64, "a warp's words take the place of its waiting keys");
+    unsigned long long *const words = (unsigned long long *)wait_s[wid];
+    compare_words_warp(acc, words);
+    block_sync();
+    if (tid < GC_COUNT) {
+        unsigned long long t = 0;
+        for (int w = 0; w < CS_THREADS / 32; ++w) t += ((const unsigned long long *)wait_s[w])[tid];
+        if (t) atomicAdd(a.g + tid, t);
     }
     cluster_sync();
+    if (rank == 0 && wid == 0) {
+        if (lane < GC_COUNT) words[lane] = __ldcg(&a.g[lane]);
+        __syncwarp();
+        compare_warp(words, a.n, a.out);
+        __threadfence_system();
+        __syncwarp();
+    }
     if (gt == 0) {
-        unsigned long long g[GC_COUNT];
-#pragma unroll
-        for (int k = 0; k < GC_COUNT; ++k) g[k] = __ldcg(&a.g[k]);
-        CompareTotals t;
-        t.vi = limbs_get(g + GC_VI);
-        t.hnum = limbs_get(g + GC_HNUM);
-        t.hden = limbs_get(g + GC_HDEN);
-        t.f = limbs_get(g + GC_F);
-        t.a11 = g[GC_A11];
-        t.sa = g[GC_SA];
-        t.sb = g[GC_SB];
-        t.nvd = g[GC_NVD];
-        t.cells = g[GC_CELLS];
-        t.ka = g[GC_KA];
-        t.kb = g[GC_KB];
-        make_compare(t, a.n, a.out);
         *a.out_status = 0;
         __threadfence_system();
     }

@@ -446,9 +446,8 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_count_w_big(CountWArgs a)
 __global__ void k_score_terms_w(const unsigned long long *cv, const unsigned long long *rec, const unsigned long long *recw,
                                 const unsigned long long *wl, int K, long long E, unsigned long long w_lo,
                                 unsigned long long w_hi, PerCommDev pc, unsigned long long *g, const int *status,
-                                Shard own)
+                                Shard own, ScoreOut o)
 {
-    __shared__ unsigned long long red[72];
     if (*status) return;
     ScoreAcc acc;
     score_acc_zero(acc);
@@ -495,9 +494,7 @@ __global__ void k_score_terms_w(const unsigned long long *cv, const unsigned lon
         if (pc.cond) pc.cond[c] = cond;
         if (pc.qds) pc.qds[c] = __dsub_rn(self, pen);
     }
-    flush_score_threads(acc, g, red);
-    const i128 t = group_sum_i128(qw, blockDim.x, red);
-    if (threadIdx.x == 0 && t != 0) limbs_add(g + GS_QW, t);
+    flush_terms(acc, qw, g, o);
 }
 
 // ---------------------------------------------------------------- load time
