@@ -37,74 +37,152 @@ __global__ void k_lpa_init(int *lab, long long n)
 // its own label when that is among the most frequent, and otherwise takes the
 // smallest of the tied labels.
 //
-// A warp takes 32 consecutive nodes (their row offsets and labels in one
-// coalesced load each, the results in one store) and gathers for LPA_NODES of
-// them at a time, a lane per sampled neighbour, so that the chain offset ->
-// neighbour -> label is waited for once for all of them.  Two ballots decide
-// most nodes: the own label when at least half of the sample carries it
-// (nothing can be more frequent), the first neighbour's when more than half
-// does.  The rest match their lanes and reduce (redux) the counts, then the
-// smallest label among the largest.  Bound by the instructions of the shuffles
-// and votes (DRAM: 1.0 GB a round).  Measured at 10^7 nodes (renumbered, mean
-// degree 19, ten rounds): 1.29-1.75 ms a round with a warp per node and a
-// 64-bit shuffle reduction, 0.78-1.16 ms so; 2, 4 and 8 nodes at a time: 8.60,
-// 8.63 and 9.42 ms a call.
+// A warp takes 32 consecutive nodes.  First their samples one after another in
+// slots, 32 slots a step whatever the degrees are (a bit per node's first slot
+// and a popcount give a lane the node of its slot): a vote a step tells which
+// labels equal the own one, and each node's lane then counts its bits.  A node
+// with its own label in at least half of the sample keeps it (nothing can be more
+// frequent).  The others are gathered LPA_NODES at a time, a lane per neighbour:
+// the first neighbour's label wins if more than half of the sample carries it;
+// else the lanes match and reduce (redux) the counts, then the smallest label
+// among the largest.  In the first rounds hardly a node keeps its label, so
+// those (`all`) skip the first part.
+// Bound in the first rounds by the pipe of votes, matches and redux (80 % busy;
+// DRAM 7 %), later by the gathers' latency.  Measured at 10^7 nodes (renumbered,
+// mean degree 19, ten rounds), ms a call: a warp per node and a 64-bit shuffle
+// reduction 14.2; a vote or two per node 8.62; so 7.79.  Steps in flight 2, 4, 8:
+// 8.08, 7.87, 8.15; blocks per SM 5, 6, 7: 7.87, 7.87, 8.12; rounds with `all` 2
+// and 3: 7.87, 7.79.
 constexpr int LPA_NODES = 4;
+constexpr int LPA_STEPS = 4;   // steps of 32 slots whose gathers are in flight together
+constexpr int LPA_ALL_ROUNDS = 3;
+constexpr int LPA_BLOCKS = 6;  // resident blocks per SM (40 registers), and those launched
 
-__global__ void __launch_bounds__(256) k_lpa_round(const long long *__restrict__ row_ptr, const int *__restrict__ col,
-                                                   long long n, const int *__restrict__ cur, int *__restrict__ nxt)
+struct LpaNode {
+    long long at;   // first arc less the first slot; or (sampled) -1 - the first arc
+    unsigned d, off;
+};
+
+__global__ void __launch_bounds__(256, LPA_BLOCKS) k_lpa_round(const long long *__restrict__ row_ptr, const int *__restrict__ col,
+                                                   long long n, const int *__restrict__ cur, int *__restrict__ nxt,
+                                                   int all)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ LpaNode s_node[8][32];
+    __shared__ int s_own[8][32];
+    __shared__ unsigned s_first[8][32 + LPA_STEPS], s_eq[8][32 + LPA_STEPS + 1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    LpaNode *const node = s_node[wid];
+    int *const nown = s_own[wid];
+    unsigned *const first_bits = s_first[wid], *const eq_bits = s_eq[wid];
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long u0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; u0 < n; u0 += nw * 32) {
         const long long u = u0 + lane;
         const long long rs = __ldg(&row_ptr[min(u, n)]);
         const unsigned deg = (unsigned)(__ldg(&row_ptr[min(u + 1, n)]) - rs);  // 0 past the last node
         const int own = u < n ? __ldg(&cur[u]) : -1;
+        const unsigned ds = min(deg, 32u);
         int res = own;
-        const int cnt = (int)min(32LL, n - u0);
-        for (int i0 = 0; i0 < cnt; i0 += LPA_NODES) {
-            int lab[LPA_NODES];
+        unsigned wait;  // nodes not decided yet
+        if (all) {
+            wait = __ballot_sync(0xffffffffu, deg != 0u);
+        } else {
+            unsigned off = ds;
+#pragma unroll
+            for (int k = 1; k < 32; k <<= 1) {
+                const unsigned t = __shfl_up_sync(0xffffffffu, off, k);
+                if (lane >= k) off += t;
+            }
+            const unsigned total = __shfl_sync(0xffffffffu, off, 31);  // at most 1024
+            off -= ds;
+            const unsigned some = __ballot_sync(0xffffffffu, deg != 0u);
+            first_bits[lane] = 0u;
+            if (lane < LPA_STEPS) first_bits[32 + lane] = 0u;
+            __syncwarp();
+            if (deg) {
+                const int k = __popc(some & ((1u << lane) - 1u));
+                node[k] = deg <= 32u ? LpaNode{rs - (long long)off, 0u, 0u} : LpaNode{-1 - rs, deg, off};
+                nown[k] = own;
+                atomicOr(&first_bits[off >> 5], 1u << (off & 31u));
+            }
+            __syncwarp();
+            int before = -1;  // nodes that began before this step, less one
+            for (unsigned t0 = 0; t0 < total; t0 += 32u * LPA_STEPS) {
+                int lab[LPA_STEPS], k[LPA_STEPS];
+#pragma unroll
+                for (int q = 0; q < LPA_STEPS; ++q) {
+                    const unsigned m = first_bits[t0 / 32u + q], t = t0 + 32u * q + lane;
+                    k[q] = max(before + __popc(m & (0xFFFFFFFFu >> (31 - lane))), 0);
+                    before += __popc(m);
+                    const LpaNode x = node[k[q]];
+                    const long long a =
+                        x.at >= 0 ? x.at + t : -1 - x.at + (long long)((unsigned long long)(t - x.off) * x.d / 32u);
+                    lab[q] = t < total ? __ldg(&col[a]) : -1;
+                }
+#pragma unroll
+                for (int q = 0; q < LPA_STEPS; ++q)
+                    if (lab[q] >= 0) lab[q] = __ldg(&cur[lab[q]]);
+#pragma unroll
+                for (int q = 0; q < LPA_STEPS; ++q) {
+                    const unsigned eq = __ballot_sync(0xffffffffu, lab[q] == nown[k[q]]);
+                    if (lane == 0) eq_bits[t0 / 32u + q] = eq;
+                }
+            }
+            __syncwarp();
+            unsigned no = 0;
+            if (ds) {
+                const unsigned w = off >> 5;
+                const unsigned b = __funnelshift_r(eq_bits[w], eq_bits[w + 1], off & 31u);
+                no = __popc(b & (0xFFFFFFFFu >> (32u - ds)));
+            }
+            wait = __ballot_sync(0xffffffffu, 2u * no < ds);
+            __syncwarp();
+        }
+        while (wait) {
+            int lab[LPA_NODES], id[LPA_NODES];
 #pragma unroll
             for (int q = 0; q < LPA_NODES; ++q) {
-                const long long r = __shfl_sync(0xffffffffu, rs, i0 + q);
-                const unsigned d = __shfl_sync(0xffffffffu, deg, i0 + q);
+                id[q] = wait ? __ffs(wait) - 1 : -1;
+                wait &= wait - 1u;
+                const long long r = __shfl_sync(0xffffffffu, rs, id[q] & 31);
+                const unsigned d = __shfl_sync(0xffffffffu, deg, id[q] & 31);
                 const unsigned j = d <= 32u ? (unsigned)lane : (unsigned)((unsigned long long)lane * d / 32u);
-                lab[q] = (unsigned)lane < d ? __ldcs(&col[r + j]) : -1;
+                lab[q] = id[q] >= 0 && (unsigned)lane < d ? __ldcs(&col[r + j]) : -1;
             }
 #pragma unroll
             for (int q = 0; q < LPA_NODES; ++q)
                 if (lab[q] >= 0) lab[q] = __ldg(&cur[lab[q]]);
 #pragma unroll
             for (int q = 0; q < LPA_NODES; ++q) {
-                const int mine = __shfl_sync(0xffffffffu, own, i0 + q);
-                const int nv = __popc(__ballot_sync(0xffffffffu, lab[q] >= 0));
-                const int no = __popc(__ballot_sync(0xffffffffu, lab[q] == mine));
+                if (id[q] < 0) break;
+                const int mine = __shfl_sync(0xffffffffu, own, id[q]);
+                const unsigned peers = __match_any_sync(0xffffffffu, lab[q]);
+                const unsigned c = lab[q] >= 0 ? 2u * (unsigned)__popc(peers) + (lab[q] == mine ? 1u : 0u) : 0u;
+                const unsigned most = __reduce_max_sync(0xffffffffu, c);  // odd: the own label is among them
                 int win = mine;
-                if (2 * no < nv) {
-                    const int first = __shfl_sync(0xffffffffu, lab[q], 0);
-                    if (2 * __popc(__ballot_sync(0xffffffffu, lab[q] == first)) > nv) {
-                        win = first;
-                    } else {
-                        const unsigned peers = __match_any_sync(0xffffffffu, lab[q]);
-                        const unsigned c = lab[q] >= 0 ? (unsigned)__popc(peers) : 0u;
-                        const unsigned most = __reduce_max_sync(0xffffffffu, c);
-                        const unsigned low =
-                            __reduce_min_sync(0xffffffffu, c == most ? (unsigned)lab[q] : 0xFFFFFFFFu);
-                        if ((unsigned)no < most) win = (int)low;
-                    }
-                }
-                if (lane == i0 + q) res = win;
+                if (!(most & 1u)) win = (int)__reduce_min_sync(0xffffffffu, c == most ? (unsigned)lab[q] : 0xFFFFFFFFu);
+                if (lane == id[q]) res = win;
             }
         }
         if (u < n) nxt[u] = res;
     }
 }
 
+// Nodes per label.  Neighbours in the stored order mostly share theirs, so the
+// first of each stretch of one label in a warp adds the stretch.
 __global__ void k_count_ids(const int *__restrict__ lab, long long n, int *hist)
 {
-    for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += (long long)gridDim.x * blockDim.x)
-        atomicAdd(&hist[lab[u]], 1);
+    const int lane = threadIdx.x & 31;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    for (long long u0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); u0 < n; u0 += step) {
+        const long long u = u0 + lane;
+        const int x = u < n ? __ldg(&lab[u]) : -1;
+        const int prev = __shfl_up_sync(0xffffffffu, x, 1);
+        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || x != prev);
+        if (x >= 0 && ((heads >> lane) & 1u)) {
+            const unsigned after = heads & (0xFFFFFFFEu << lane);
+            atomicAdd(&hist[x], (after ? __ffs(after) - 1 : 32) - lane);
+        }
+    }
 }
 
 // New position of every node: its cluster's offset plus a slot taken in the
@@ -208,12 +286,12 @@ int launch_label_propagation(const GraphDev &g, int rounds, int num_sms, cudaStr
                              int *hist, int *tmp, size_t tmp_elems, int *out)
 {
     const long long n = g.n;
-    const int g1 = grid_of(n, 512, num_sms, 8), gw = grid_of(n * 32, 256, num_sms, 8);
+    const int g1 = grid_of(n, 512, num_sms, 8), gl = grid_of(n, 256, num_sms, LPA_BLOCKS);
     int L = 0;
     k_lpa_init_ids<<<g1, 512, 0, s>>>(lab0, g.inv, n);
     ++L;
     for (int r = 0; r < rounds; ++r) {
-        k_lpa_round<<<gw, 256, 0, s>>>(g.row_ptr, g.col, n, lab0, lab1);
+        k_lpa_round<<<gl, 256, 0, s>>>(g.row_ptr, g.col, n, lab0, lab1, r < LPA_ALL_ROUNDS);
         std::swap(lab0, lab1);
         ++L;
     }
@@ -260,11 +338,12 @@ int reorder_graph(const GraphDev &g, int rounds, int num_sms, cudaStream_t s, lo
     if ((e = cudaMalloc(&perm, (size_t)n * 4)) != cudaSuccess) return -bad(e);
     if ((e = cudaMalloc(&inv, (size_t)n * 4)) != cudaSuccess) return -bad(e);
     if ((e = cudaMalloc(&tmp, tmp_elems * 4)) != cudaSuccess) return -bad(e);
-    const int g1 = grid_of(n, 512, num_sms, 8), gw = grid_of(n * 32, 256, num_sms, 8);
+    const int g1 = grid_of(n, 512, num_sms, 8), gw = grid_of(n * 32, 256, num_sms, 8),
+              gl = grid_of(n, 256, num_sms, LPA_BLOCKS);
     k_lpa_init<<<g1, 512, 0, s>>>(lab0, n);
     ++L;
     for (int r = 0; r < rounds; ++r) {
-        k_lpa_round<<<gw, 256, 0, s>>>(g.row_ptr, g.col, n, lab0, lab1);
+        k_lpa_round<<<gl, 256, 0, s>>>(g.row_ptr, g.col, n, lab0, lab1, r < LPA_ALL_ROUNDS);
         std::swap(lab0, lab1);
         ++L;
     }
