@@ -48,3 +48,17 @@ def test_candidates_per_cluster(qm, oracle_mod, count):
         assert oc[p] == qm.compare(truth, L[p], 40, k)
         check_quality(oq[p], oracle_mod.score(rp, col, L[p].cpu().numpy(), k), f"p={p}")
         check_compare(oc[p], oracle_mod.compare(truth.cpu().numpy(), L[p].cpu().numpy(), 40, k), f"p={p}")
+
+
+@pytest.mark.parametrize("k", [1, 2, 31, 33, 64, 129, 300])
+def test_candidate_counters_around_the_run_length(qm, oracle_mod, k):
+    """Runs with as many entries as counters above the community's id, fewer and
+    more: counters read in order, or through the run's entries again."""
+    n = 600
+    rng = np.random.default_rng(k)
+    rp, col = random_graph(n, 9 * n, seed=5)
+    L = torch.from_numpy(rng.integers(0, k, (5, n)).astype(np.int32)).cuda()
+    graph = qm.Graph(*to_dev(rp, col))
+    for p, q in enumerate(qm.score_batched(graph, L, [k] * 5)):
+        assert q == qm.score(graph, L[p], k)
+        check_quality(q, oracle_mod.score(rp, col, L[p].cpu().numpy(), k), f"p={p}")
