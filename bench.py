@@ -48,7 +48,7 @@ FALLBACK_HBM = 6800.0
 # permutation of renumbered graphs included), with the headers they include;
 # the DRAM records under profiles/ name their hash.
 STEP_SOURCES = ("qm_kernels.cu", "qm_community.cuh", "qm_device.cuh", "qm_finalize.cuh", "qm_expand.cuh",
-                "qm_binned.cuh", "qm_weighted.cuh", "qm_internal.h", "qm_reorder.cu")
+                "qm_rows.cuh", "qm_count.cuh", "qm_binned.cuh", "qm_weighted.cuh", "qm_internal.h", "qm_reorder.cu")
 
 
 def kernel_source_hash() -> str:
@@ -112,7 +112,7 @@ def algorithmic_bytes(kernel: str, n: int, E: int, K: int, q: dict) -> float:
     stream the adjacency with its label gathers carry all of them (they read
     every arc, every row offset and every node's label); the others carry none
     (pair counting and finalisation add no method bytes)."""
-    if kernel in ("k_expand", "k_score_cm", "k_expand_half"):
+    if kernel in ("k_rows", "k_score_cm", "k_expand_half"):
         return method_bytes(n, E)
     return 0.0
 
@@ -125,11 +125,10 @@ def pipeline_bytes(kernel: str, n: int, E: int, K: int, q: dict) -> float:
     cut = 2.0 * q["cut_edges_total"]
     table = {
         "k_score_cm": 8.0 * E + 12.0 * n,
-        "k_expand": 8.0 * E + 20.0 * n + 4.0 * cut,
-        "k_count": 20.0 * cut + 64.0 * K,
-        "k_scatter_deg": 20.0 * n,
+        "k_rows": 8.0 * E + 12.0 * n + 2.0 * cut,  # (of each cut edge's two entries, the one above is packed)
+        "k_count_tab": 2.0 * cut + 64.0 * K,
         "k_permute_labels": 12.0 * n,
-        "k_permute_hist": 12.0 * n,
+        "k_permute_vol": 20.0 * n,
     }
     return table.get(kernel, 0.0)
 
@@ -434,7 +433,7 @@ def bench_headline(args, world, rank, local):
         assert q6 == q, "sorted and hashed counts disagree"
         count_variants = {
             "what": "phase B of the two-phase pipeline: each community's packed run hashed (algorithm 1, "
-                    "k_count + k_count_long) or radix-sorted and run-length counted (algorithm 6, "
+                    "k_count_tab + k_count_big) or radix-sorted and run-length counted (algorithm 6, "
                     "k_count_sort + k_count_long); same graph, partition and launch shape, identical results",
             "hash": {"ms_per_step": ms_max / args.steps, "kernel_ms": per_kernel(step_kernels, args.steps)},
             "sort": {"ms_per_step": ms6 / vsteps, "kernel_ms": per_kernel(tr6, vsteps)}}

@@ -382,11 +382,13 @@ qm_status qm_debug_set_perm_buckets(int32_t window_bits, int32_t tile_bits, int6
  * (log2 n_nodes, log2 n_arcs, log2 K).  qm_get_tuning reports the shape the
  * next call of that bucket will use: threads per block, shared-memory bytes per
  * block, and the community size above which a whole block (not a warp) scores a
- * community (used by algorithm 0 only).  algorithm selects the scoring pipeline:
+ * community (used by algorithm 0 only).  The two-phase pipelines use the threads
+ * and shared memory for algorithm 6's sort and when K reaches 2^20; below that
+ * their kernels have fixed shapes.  algorithm selects the scoring pipeline:
  *   0  one kernel visits every community's members and gathers their
  *      neighbours' labels itself;
- *   1  (default) the neighbour labels are first written out in community
- *      order (one streaming pass over the arcs), then a second kernel counts
+ *   1  (default) the neighbour labels are first written out by community
+ *      (one streaming pass over the arcs in stored node order), then a second kernel counts
  *      each community's contiguous segment and a third forms the FP64 terms of
  *      all communities in parallel;
  *   2  as 1, but an arc whose far end is not close to its near end in node-id
@@ -401,11 +403,11 @@ qm_status qm_debug_set_perm_buckets(int32_t window_bits, int32_t tile_bits, int6
  *      21-bit ids to a 64-bit word (8/3 bytes a node instead of 4, so a larger
  *      share of it stays in L2); algorithm 1 does this on graphs of more than
  *      2^22 nodes.  On a graph loaded with QM_REORDER the gathers first try a
- *      block encoding built per call (per 16 consecutive nodes two labels and
- *      a 16-bit mask, blocks of three or more labels apart: half a byte a
- *      node when the partition follows the stored order, so that it stays in
- *      L2), falling back to the packed copy when too many blocks hold three
- *      or more labels; algorithm 1 does this above 2^26 nodes;
+ *      block encoding built per call (a 32-bit word per 16 consecutive nodes:
+ *      their label, or where two labels and a 16-bit mask, or 16 labels, lie:
+ *      a quarter of a byte a node when the partition follows the stored order,
+ *      so that it stays in L2), falling back to the packed copy when too many
+ *      blocks hold several labels; algorithm 1 does this above 2^26 nodes;
  *   5  as 1, never packed;
  *   6  as 1, but the second kernel sorts each community's segment by label
  *      (a radix sort in shared memory, 8-bit digits) and counts the equal-label

@@ -527,8 +527,8 @@ __global__ void __launch_bounds__(256) k_bu_scatter(const BatchItem *items, int 
     }
 }
 
-// A warp's share of phase A for the batched pipeline: expand_chunk, except
-// that when the chunk's members are not a few runs of consecutive node ids
+// A warp's share of phase A for the batched pipeline, 32 member positions.  When
+// the chunk's members are not a few runs of consecutive node ids
 // (the usual case for candidate partitions), the owner of each arc of the
 // chunk is tabulated once (each lane writes its member's index over its arc
 // range, up to BU_OWN_CAP arcs) instead of searched for arc by arc.
@@ -557,7 +557,6 @@ __device__ __forceinline__ void bu_expand_chunk(long long p0, long long n, const
     const bool newrun = valid && (lane == 0 || cw[lane] != cw[lane - 1]);
     unsigned runs = __ballot_sync(0xffffffffu, newrun);
     const unsigned segs = __ballot_sync(0xffffffffu, newrun || (valid && u != u_prev + 1));
-    u128 w_in = 0, w_out = 0;
     if (__popc(segs) <= EXPAND_MAX_SEGS) {
         unsigned rem = segs;
         while (rem) {
@@ -569,9 +568,8 @@ __device__ __forceinline__ void bu_expand_chunk(long long p0, long long n, const
             const int c = cw[lo];
             const unsigned cbase = __ldg(&aoff[__ldg(&start[c])]);
             const long long cs = rsw[lo] - (long long)e_lo;  // CSR index of arc e is cs + e
-            expand_range<false, false, true>(e_lo, e_hi, c, cbase, [cs](unsigned e) { return cs + (long long)e; },
-                                             col, labels, nullptr, inter, inter_hi, nbr, keep, lane, nullptr, nullptr,
-                                             w_in, w_out);
+            expand_range(e_lo, e_hi, c, cbase, [cs](unsigned e) { return cs + (long long)e; },
+                                             col, labels, inter, inter_hi, nbr, keep, lane);
         }
     } else {
         const bool tab = offw[nm] <= (unsigned)BU_OWN_CAP;
@@ -589,21 +587,21 @@ __device__ __forceinline__ void bu_expand_chunk(long long p0, long long n, const
             const int c = cw[m_lo];
             const unsigned cbase = __ldg(&aoff[__ldg(&start[c])]);
             if (tab)
-                expand_range<false, false, true>(
+                expand_range(
                     e_lo, e_hi, c, cbase,
                     [=](unsigned e) {
                         const int o = own[e];
                         return rsw[o] + (long long)(e - offw[o]);
                     },
-                    col, labels, nullptr, inter, inter_hi, nbr, keep, lane, nullptr, nullptr, w_in, w_out);
+                    col, labels, inter, inter_hi, nbr, keep, lane);
             else
-                expand_range<false, false, true>(
+                expand_range(
                     e_lo, e_hi, c, cbase,
                     [=](unsigned e) {
                         const int o = m_lo + upper_bound_smem(offw + m_lo, m_hi - m_lo, e) - 1;
                         return rsw[o] + (long long)(e - offw[o]);
                     },
-                    col, labels, nullptr, inter, inter_hi, nbr, keep, lane, nullptr, nullptr, w_in, w_out);
+                    col, labels, inter, inter_hi, nbr, keep, lane);
         }
     }
     __syncwarp();

@@ -20,7 +20,7 @@
 // 128-byte pieces, and lists each chunk when it is closed.  The chunk list is
 // then ordered by bin.
 #pragma once
-// Included by qm_kernels.cu inside namespace qm, after k_expand.
+// Included by qm_kernels.cu inside namespace qm, after the plain pipeline's kernels.
 
 constexpr int BIN_MAX = 16;        // destination windows at most
 constexpr int BIN_CHUNK = 256;     // records per pool chunk (2 KB)
@@ -183,7 +183,7 @@ __device__ __forceinline__ void expand_range_bin(unsigned e_lo, unsigned e_hi, i
     }
 }
 
-// Phase A of the binned path: k_expand's walk over member positions, with the
+// Phase A of the binned path: a walk over member positions, with the
 // far arcs binned instead of gathered.
 __global__ void __launch_bounds__(EXPAND_THREADS) k_expand_bin(const long long *__restrict__ row_ptr,
                                                                const int *__restrict__ col,

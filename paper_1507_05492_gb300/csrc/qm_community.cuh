@@ -593,8 +593,8 @@ __device__ __forceinline__ void compare_cells_community(const CompareCtx &x, int
 
 // ---------------------------------------------------------------- two-phase scoring
 //
-// Phase A (k_expand) visits every member of every community in member order
-// and looks up the labels of its neighbours.  Arcs to the member's own
+// Phase A (k_rows; in community order for batches and the other gathers) looks up
+// the labels of every node's neighbours.  Arcs to the member's own
 // community are only counted; the labels of the other arcs are packed densely
 // at the front of the community's arc segment, nbr[aoff[start[c]] ..
 // aoff[start[c]] + inter[c]), in no particular order.  Phase B

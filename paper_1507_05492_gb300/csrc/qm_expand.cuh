@@ -1,7 +1,7 @@
-// qm_expand.cuh -- phase A of the two-phase scoring pipeline (the far-end
-// label gathers), shared by the single-partition pipeline (k_expand in
-// qm_kernels.cu) and the batched pipeline over many candidate partitions
-// (qm_batched.cu).
+// qm_expand.cuh -- parts of phase A of the two-phase scoring pipeline (the
+// far-end label gathers): the label encodings, the gathers in community order of
+// the batched pipeline (qm_batched.cu) and of the half-edge variant
+// (qm_kernels.cu).  The single-partition default, in node order, is in qm_rows.cuh.
 #pragma once
 
 #include <climits>
@@ -11,7 +11,7 @@
 namespace qm {
 using namespace qmk;
 
-// Phase A: for each member position p (community order) the labels of the
+// Phase A in community order: for each member position p the labels of the
 // neighbours of members[p] are looked up.  A warp takes 32 consecutive member
 // positions; they hold one or more runs of members of one community each.  For
 // a run of community c the warp spreads the run's arcs over its lanes,
@@ -83,62 +83,42 @@ __host__ __device__ inline unsigned blk_slots_at(long long n) { return 3u * blk_
 enum { LAB_PLAIN = 0, LAB_PACK3 = 1, LAB_BLOCKS = 2 };
 
 // Gathers the labels of arcs [e_lo, e_hi) of a run of community c (loc(e) is
-// the CSR index of arc e; plab is the packed copy or the block encoding, as
-// LAB says), counts those != c in inter[c] (the cut arcs of c)
-// and packs them into c's segment at cbase; with HI only the labels above c are
-// packed (each unordered pair of communities is counted by its smaller id), and
-// hi[c] counts them.  On a weighted graph (WT) the arc weights travel with the
-// packed labels (nbrw) and each lane sums the fixed-point weights of its intra
-// and cut arcs.
-template <bool WT, int LAB, bool HI, class LOC>
+// the CSR index of arc e), counts those != c in inter[c] (the cut arcs of c)
+// and packs those above c into c's segment at cbase (each unordered pair of
+// communities is counted by its smaller id); hi[c] counts them.
+template <class LOC>
 __device__ __forceinline__ void expand_range(unsigned e_lo, unsigned e_hi, int c, unsigned cbase, LOC loc,
                                              const int *__restrict__ col, const int *__restrict__ labels,
-                                             const unsigned long long *__restrict__ plab,
                                              int *inter, int *hi, int *__restrict__ nbr, unsigned long long keep,
-                                             int lane, const float *__restrict__ wt, float *__restrict__ nbrw,
-                                             u128 &w_in, u128 &w_out)
+                                             int lane)
 {
     const unsigned lt = (1u << lane) - 1u;
     for (unsigned e0 = e_lo; e0 < e_hi; e0 += 32u * EXPAND_UNROLL) {
         int lab[EXPAND_UNROLL];
-        float wv[EXPAND_UNROLL];
 #pragma unroll
         for (int k = 0; k < EXPAND_UNROLL; ++k) {
             const unsigned e = e0 + lane + 32u * k;
             lab[k] = e < e_hi ? __ldcs(&col[loc(e)]) : -1;
-            if (WT) wv[k] = e < e_hi ? __ldcs(&wt[loc(e)]) : 0.0f;
         }
 #pragma unroll
         for (int k = 0; k < EXPAND_UNROLL; ++k)
-            if (lab[k] >= 0)
-                lab[k] = LAB == LAB_PACK3 ? ld_label3(plab, lab[k], keep) : ld_hint(&labels[lab[k]], keep);
-        if (WT) {
-#pragma unroll
-            for (int k = 0; k < EXPAND_UNROLL; ++k)
-                if (lab[k] >= 0) {
-                    const unsigned long long f = w_fixed(wv[k]);
-                    if (lab[k] == c) w_in += f; else w_out += f;
-                }
-        }
+            if (lab[k] >= 0) lab[k] = ld_hint(&labels[lab[k]], keep);
         unsigned msk[EXPAND_UNROLL];
         int tot = 0, cut = 0;
 #pragma unroll
         for (int k = 0; k < EXPAND_UNROLL; ++k) {
-            if (HI) cut += __popc(__ballot_sync(0xffffffffu, lab[k] >= 0 && lab[k] != c));
-            msk[k] = __ballot_sync(0xffffffffu, HI ? lab[k] > c : (lab[k] >= 0 && lab[k] != c));
+            cut += __popc(__ballot_sync(0xffffffffu, lab[k] >= 0 && lab[k] != c));
+            msk[k] = __ballot_sync(0xffffffffu, lab[k] > c);
             tot += __popc(msk[k]);
         }
-        if (HI && cut && lane == 0) atomicAdd(&inter[c], cut);
+        if (cut && lane == 0) atomicAdd(&inter[c], cut);
         if (tot == 0) continue;
         int pos = 0;
-        if (lane == 0) pos = atomicAdd(HI ? &hi[c] : &inter[c], tot);
+        if (lane == 0) pos = atomicAdd(&hi[c], tot);
         unsigned at = cbase + (unsigned)__shfl_sync(0xffffffffu, pos, 0);
 #pragma unroll
         for (int k = 0; k < EXPAND_UNROLL; ++k) {
-            if ((msk[k] >> lane) & 1u) {
-                __stcs(&nbr[at + __popc(msk[k] & lt)], lab[k]);
-                if (WT) __stcs(&nbrw[at + __popc(msk[k] & lt)], wv[k]);
-            }
+            if ((msk[k] >> lane) & 1u) __stcs(&nbr[at + __popc(msk[k] & lt)], lab[k]);
             at += __popc(msk[k]);
         }
     }
@@ -255,7 +235,7 @@ __device__ __forceinline__ void expand_range_half(unsigned e_lo, unsigned e_hi, 
     }
 }
 
-// One warp's share of the half-edge phase A: as expand_chunk, over the
+// One warp's share of the half-edge phase A: 32 member positions, over the
 // members' upper rows (up_ptr / up_col), with the in-chunk arc offsets summed
 // in the warp and each community's segment base read from cbase.
 template <bool PACK, bool FULL>

@@ -8,6 +8,7 @@
 //               by whole blocks, the rest by single warps
 //   k_score_cm  again over the communities whose warp table overflowed
 //   k_score_fin exact sums -> qm_quality
+// (tuning algorithm 0; the default pipeline's kernels are listed at launch_score2).
 // qm_compare_partitions runs the same counting sort on the detected labels,
 // hashes the ground-truth labels of each detected community's members into the
 // contingency cells, then walks the ground-truth communities for the row maxima.
@@ -730,7 +731,7 @@ static int grid_for(long long n, int threads, int num_sms, int per_sm)
 // the row-offset reads are coalesced).  The lanes of a warp that hold one label
 // take their places with a single atomic, in node order: on a graph whose nodes
 // are numbered cluster by cluster (QM_REORDER) consecutive member positions
-// are then mostly consecutive nodes, whose rows are adjacent (see k_expand).
+// are then mostly consecutive nodes, whose rows are adjacent.
 __global__ void k_scatter_deg(const int *__restrict__ labels, const long long *__restrict__ row_ptr, long long n,
                               int *cursor, int *members, int *degm, const int *status)
 {
