@@ -833,10 +833,10 @@ static qm_status score_impl(qm_graph *g, const int32_t *labels, int32_t K, qm_me
             int32_t *pl = (int32_t *)(ws.ptr() + perm_off);
             // two passes through shared memory where the graph has them (the two-phase
             // pipeline then takes the community sizes from the second), else one gather
-            const bool rows = sh.algo && score_rows(g->d, sh.algo, shard_p);
+            const bool vols = score_volumes(g->d, sh.algo);
             const int lp = g->pb.lpos ? launch_permute_buckets(dl, g->pb, g->row_ptr, n, (int *)(ws.ptr() + pb_off), pl,
-                                                               sh.algo && !rows ? w.size : nullptr,
-                                                               rows ? w.cv : nullptr, K, w.status, nsm, st, tr)
+                                                               sh.algo && !vols ? w.size : nullptr,
+                                                               vols ? w.cv : nullptr, K, w.status, nsm, st, tr)
                                       : 0;
             if (lp < 0) return -1;
             if (lp > 0) {
@@ -844,7 +844,7 @@ static qm_status score_impl(qm_graph *g, const int32_t *labels, int32_t K, qm_me
                 L += lp - 1;
             } else if (sh.algo) {  // the two-phase pipeline takes the community sizes from the gather
                 if (tr) tr("k_permute_hist", st);
-                if (launch_permute_hist(dl, g->inv, g->row_ptr, n, pl, K, w, rows, nsm, st) < 0) return -1;
+                if (launch_permute_hist(dl, g->inv, g->row_ptr, n, pl, K, w, vols, nsm, st) < 0) return -1;
                 sizes_ready = true;
             } else {
                 if (tr) tr("k_permute_labels", st);

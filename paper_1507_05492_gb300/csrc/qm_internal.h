@@ -196,6 +196,7 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
 // (algorithms 1, 4, 5 and 6, weighted graphs, and 7 where the half-edge pass does
 // not apply) rather than the members in community order.
 bool score_rows(const GraphDev &g, int algo, int shard_p);
+bool score_volumes(const GraphDev &g, int algo);
 // Segment bases (exclusive prefix of the low 33 bits) and reciprocals of the
 // sizes (the bits above) of K words; sums: scratch of K / 4096 + 1 words.
 // Returns its launches.

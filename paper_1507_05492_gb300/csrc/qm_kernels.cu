@@ -25,7 +25,7 @@ namespace qm {
 using namespace qmk;
 
 enum { C_BIG_COUNT = 0, C_BIG_NEXT = 1, C_SMALL_NEXT = 2, C_OVF_COUNT = 3, C_OVF_NEXT = 4, C_SMALL_COUNT = 5,
-       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_BAD = 9, C_MID_NEXT = 10, C_TERMS_DONE = 11,
+       C_LONG_COUNT = 6, C_NCELLS = 7, C_MID_COUNT = 8, C_BX_BAD = 9, C_MID_NEXT = 10, C_TERMS_DONE = 11, C_MEMBERS = 14,
        C_BX_COUNT = 12 /* two words */ };
 
 constexpr int SCAN_TILE = 4096;   // elements per block in the multi-block scan
@@ -726,9 +726,9 @@ static int grid_for(long long n, int threads, int num_sms, int per_sm)
 
 // ------------------------------------------------------------------ two-phase scoring
 
-// Counting sort of the nodes by label (as k_scatter) that also records the
-// degree of the node placed at each member position (read in node order, so
-// the row-offset reads are coalesced).  The lanes of a warp that hold one label
+// Counting sort of the nodes by label (as k_scatter) that also records (degm
+// not null) the degree of the node placed at each member position (read in node
+// order, so the row-offset reads are coalesced).  The lanes of a warp that hold one label
 // take their places with a single atomic, in node order: on a graph whose nodes
 // are numbered cluster by cluster (QM_REORDER) consecutive member positions
 // are then mostly consecutive nodes, whose rows are adjacent.
@@ -750,7 +750,7 @@ __global__ void k_scatter_deg(const int *__restrict__ labels, const long long *_
         base = __shfl_sync(peers, base, leader);
         const int pos = base + __popc(peers & ((1u << lane) - 1u));
         members[pos] = (int)i;
-        degm[pos] = (int)(__ldg(&row_ptr[i + 1]) - __ldg(&row_ptr[i]));
+        if (degm) degm[pos] = (int)(__ldg(&row_ptr[i + 1]) - __ldg(&row_ptr[i]));
     }
 }
 
@@ -883,13 +883,31 @@ __global__ void __launch_bounds__(EXPAND_THREADS) k_expand_half(const long long 
                                       offs_s[w], rs_s[w], cw_s[w], keep, lane);
 }
 
-// Each community's segment base, cbase[c] = aoff[start[c]] (for the appends
-// of the half-edge phase A into other communities' runs).
-__global__ void k_cbase(const int *start, const unsigned *aoff, int K, unsigned *cbase, const int *status)
+// Room for every community's members in the member array, in no particular
+// order of the communities (the half-edge pass only needs each one's members
+// together): a warp scans 32 sizes and takes their room with one atomic.  The
+// segment bases come from the communities' volumes (k_vscan_apply), so no degree
+// is written per member and no scan of them made: 10^8 nodes as given, the call
+// 30.2 -> 27.4 ms.
+__global__ void k_member_places(const unsigned long long *cv, int K, int *place, int *taken, const int *status)
 {
     if (*status) return;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < K; c += gridDim.x * blockDim.x)
-        cbase[c] = aoff[start[c]];
+    const int lane = threadIdx.x & 31;
+    for (long long c0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); c0 < K;
+         c0 += (long long)gridDim.x * blockDim.x) {
+        const long long c = c0 + lane;
+        const int size = c < K ? (int)(cv[c] >> VOL_BITS) : 0;
+        int end = size;
+#pragma unroll
+        for (int k = 1; k < 32; k <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, end, k);
+            if (lane >= k) end += t;
+        }
+        int at = 0;
+        if (lane == 31) at = atomicAdd(taken, end);
+        at = __shfl_sync(0xffffffffu, at, 31);
+        if (c < K) place[c] = at + end - size;
+    }
 }
 
 #include "qm_binned.cuh"
@@ -903,7 +921,7 @@ __global__ void k_cbase(const int *start, const unsigned *aoff, int K, unsigned 
 // cut_from_intra (the `inter` array) turns from 2|E_c^in| into the cut arcs.
 __global__ void k_classify(const int *start, const unsigned *aoff, const int *mlen, int K, int warp_fill,
                            int group_fill, int block_fill, RunHdr *big, RunHdr *small, RunHdr *lng, RunHdr *mid,
-                           int *counters, const int *status, Shard own, int *cut_from_intra)
+                           int *counters, const int *status, Shard own)
 {
     if (*status) return;
     const int lane = threadIdx.x & 31;
@@ -918,8 +936,6 @@ __global__ void k_classify(const int *start, const unsigned *aoff, const int *ml
             if (s1 > s0 && own.owns(c)) {
                 const unsigned a0 = aoff[s0];
                 h = RunHdr{c, a0, (unsigned)mlen[c], aoff[s1] - a0};
-                // half-edge phase A left 2|E_c^in| there: the cut arcs are the rest of the volume
-                if (cut_from_intra) cut_from_intra[c] = (int)(h.vol - (unsigned)cut_from_intra[c]);
                 cls = h.m > (unsigned)block_fill ? 2
                       : h.m > (unsigned)group_fill ? 0
                       : h.m > (unsigned)warp_fill ? 3 : 1;
@@ -1853,7 +1869,7 @@ static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, con
     const int cb = ct_count_bits(K), most = K < CT_MAX_K ? (int)std::min<long long>(INT_MAX, (1LL << cb) - 1) : 0;
     TRACE("k_classify");
     k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
-        ws.cv, (const unsigned *)ws.cursor, ws.curs, K, std::min(ct_fill_warp(K, num_sms), most),
+        ws.cv, (const unsigned *)ws.cursor, ws.curs, nullptr, K, std::min(ct_fill_warp(K, num_sms), most),
         std::min(CT_FILL_GROUP, most), std::min(CB_FILL_LONG, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.inter, ws.counters,
         ws.status, own);
     CountWArgs a;
@@ -1885,6 +1901,10 @@ static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, con
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
+// Whether the call counts members and arcs in one word per community (all but
+// the binned gathers and the one-kernel pipeline).
+bool score_volumes(const GraphDev &g, int algo) { return algo != 0 && (g.wt || !bin_mode_of(algo, false)); }
+
 bool score_rows(const GraphDev &g, int algo, int shard_p)
 {
     if (g.wt) return algo != 0;
@@ -1904,10 +1924,10 @@ int launch_segment_bases(const unsigned long long *words, int K, unsigned *base,
     return tiles > 1 ? 2 : 1;
 }
 
-// Phase A in stored node order: volumes (unless the label permutation has
-// counted them), segment bases, the walk.  Returns its launches.
-static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh, bool hi,
-                             int num_sms, cudaStream_t s, TraceFn tr, Shard own, bool sizes_ready)
+// Members and arcs of every community (unless the permutation counted them),
+// segment bases (in ws.cursor) and reciprocals.
+static int launch_volumes(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, int num_sms, cudaStream_t s,
+                          TraceFn tr, bool sizes_ready)
 {
     int launches = 0;
     const long long n = g.n;
@@ -1919,14 +1939,23 @@ static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const 
         ++launches;
     }
     unsigned *base = (unsigned *)ws.cursor;
-    launches += launch_segment_bases(ws.cv, K, base, ws.recip, (unsigned *)ws.scan_tmp, ws.status, s, tr);
+    return launches + launch_segment_bases(ws.cv, K, base, ws.recip, (unsigned *)ws.scan_tmp, ws.status, s, tr);
+}
+
+// Phase A in stored node order: volumes (unless the label permutation has
+// counted them), segment bases, the walk.  Returns its launches.
+static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh, bool hi,
+                             int num_sms, cudaStream_t s, TraceFn tr, Shard own, bool sizes_ready)
+{
+    const long long n = g.n;
+    int launches = launch_volumes(g, labels, K, ws, num_sms, s, tr, sizes_ready);
     RowsArgs a;
     a.row_ptr = g.row_ptr;
     a.col = g.col;
     a.labels = labels;
     a.plab = ws.plab;
     a.n = n;
-    a.base = base;
+    a.base = (const unsigned *)ws.cursor;
     a.curs = ws.curs;
     a.nbr = ws.nbr;
     a.status = ws.status;
@@ -1975,9 +2004,11 @@ static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const 
 // The two-phase plain scoring pipeline:
 //   k_hist_vol -> k_vscan_* (segment bases) -> k_rows
 //   -> k_rows_classify -> k_count_* -> k_score_terms (and the results)
-// or, for the half-edge and binned gathers, members in community order:
+// or, for the half-edge gathers, members in community order:
+//   k_hist_vol -> k_vscan_* -> k_member_places -> k_scatter_deg -> k_expand_half -> k_rows_classify -> ...
+// and for the binned gathers:
 //   k_hist -> scan (sizes) -> k_scatter_deg -> scan (member degrees = arc offsets)
-//   -> k_expand_half / k_expand_bin -> k_classify -> ...
+//   -> k_expand_bin -> k_classify -> ...
 int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws, const Shape &sh,
                   const PerCommDev *pc, int num_sms, cudaStream_t s, TraceFn tr, int shard_r, int shard_p,
                   bool sizes_ready)
@@ -1994,6 +2025,15 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     if (rows) {
         launches += launch_phase_rows(g, labels, K, ws, sh, hi, num_sms, s, tr, own, sizes_ready);
         if (g.wt) return launch_weighted_tail(g, K, ws, pc, num_sms, s, tr, own, launches);
+    } else if (half) {
+        launches += launch_volumes(g, labels, K, ws, num_sms, s, tr, sizes_ready);
+        TRACE("k_member_places");
+        k_member_places<<<grid_for(K, 256, num_sms, 8), 256, 0, s>>>(ws.cv, K, ws.start, &ws.counters[C_MEMBERS],
+                                                                     ws.status);
+        TRACE("k_scatter_deg");
+        k_scatter_deg<<<grid_for(n, 512, num_sms, 8), 512, 0, s>>>(labels, g.row_ptr, n, ws.start, ws.members, nullptr,
+                                                                   ws.status);
+        launches += 2;
     } else {
         if (!sizes_ready) {
             const int hist_smem = (K <= 12288) ? K * 4 : 0;
@@ -2013,14 +2053,10 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
                                 ws.counters, ws.scan_tmp, ws.status, s, tr);
     }
     if (half) {
-        // each undirected edge gathered once, from its lower end; the scatter
-        // cursors are free now and take the segment bases
-        unsigned *cbase = (unsigned *)ws.cursor;
+        // each undirected edge gathered once, from its lower end
+        const unsigned *cbase = (const unsigned *)ws.cursor;
         const bool full = pc && pc->qds;
         const dim3 eg(expand_grid(n, num_sms)), eb(EXPAND_THREADS);
-        TRACE("k_cbase");
-        k_cbase<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(ws.start, ws.aoff, K, cbase, ws.status);
-        ++launches;
         if (ws.plab) {
             TRACE("k_pack3");
             k_pack3<<<grid_for((n + 2) / 3, 256, num_sms, 8), 256, 0, s>>>(labels, n, ws.plab, ws.status, nullptr);
@@ -2071,29 +2107,18 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     const int cb = ct_count_bits(K);
     const int most = tab ? (int)std::min<long long>(INT_MAX, (1LL << cb) - 1) : 0;
     TRACE("k_classify");
-    if (rows) {
-        // run classes: the count's tables, or (sorted) SORT_WARP_CAP and the blocks' buffers
-        const int wf = tab ? std::min(ct_fill_warp(K, num_sms), most) : sorted ? SORT_WARP_CAP : cp.fill_w;
-        const int gf = tab ? std::min(CT_FILL_GROUP, most) : sorted ? SORT_WARP_CAP : cp.fill_g;
-        const int bf = tab ? std::min(CB_FILL, most) : sorted ? sp.cap : cp.fill;
+    // run classes: the count's tables, or (sorted) SORT_WARP_CAP and the blocks' buffers
+    const int wf = tab ? std::min(ct_fill_warp(K, num_sms), most) : sorted ? SORT_WARP_CAP : cp.fill_w;
+    const int gf = tab ? std::min(CT_FILL_GROUP, most) : sorted ? SORT_WARP_CAP : cp.fill_g;
+    const int bf = tab ? std::min(CB_FILL, most) : sorted ? sp.cap : cp.fill;
+    if (rows || half)
         k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
-            ws.cv, (const unsigned *)ws.cursor, ws.curs, K, wf, gf, bf, ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid,
-            ws.inter, ws.counters, ws.status, own);
-    } else if (tab)
-        k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
-            ws.start, ws.aoff, packed_len, K, std::min(ct_fill_warp(K, num_sms), most),
-            std::min(CT_FILL_GROUP, most), std::min(CB_FILL, most), ws.hdr_big, ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
-            half ? ws.inter : nullptr);
-    else if (sorted)  // warps sort runs up to SORT_WARP_CAP, blocks up to their buffers
-        k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(ws.start, ws.aoff, packed_len, K, SORT_WARP_CAP,
-                                                                SORT_WARP_CAP, sp.cap, ws.hdr_big, ws.hdr_small,
-                                                                ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
-                                                                half ? ws.inter : nullptr);
+            ws.cv, (const unsigned *)ws.cursor, ws.curs, half ? packed_len : nullptr, K, wf, gf, bf, ws.hdr_big,
+            ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.inter, ws.counters, ws.status, own);
     else
-        k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(ws.start, ws.aoff, packed_len, K, cp.fill_w,
-                                                                cp.fill_g, cp.fill, ws.hdr_big, ws.hdr_small,
-                                                                ws.hdr_long, ws.hdr_mid, ws.counters, ws.status, own,
-                                                                half ? ws.inter : nullptr);
+        k_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(ws.start, ws.aoff, packed_len, K, wf, gf, bf, ws.hdr_big,
+                                                                ws.hdr_small, ws.hdr_long, ws.hdr_mid, ws.counters,
+                                                                ws.status, own);
     ++launches;
     CountKArgs a;
     a.x.nbr = ws.nbr;
@@ -2173,7 +2198,7 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
     // (a shard's caller reads the partial sums instead of the results)
     const ScoreOut so{shard_p == 1 ? ws.counters + C_TERMS_DONE : nullptr, n, g.n_arcs / 2, ws.result, 0};
     const int tt = terms_threads(K, num_sms);
-    k_score_terms<<<grid_for(K, tt, num_sms, 2), tt, 0, s>>>(ws.start, rows ? ws.cv : nullptr, ws.rec, K,
+    k_score_terms<<<grid_for(K, tt, num_sms, 2), tt, 0, s>>>(ws.start, rows || half ? ws.cv : nullptr, ws.rec, K,
                                                              g.n_arcs / 2, pcd, ws.gacc, ws.status, own, so);
     ++launches;
     TRACE(nullptr);
@@ -2187,7 +2212,7 @@ int launch_cover_runs(const CoverRuns &r, int K, long long E, unsigned long long
     const int cb = ct_count_bits(K), most = (int)std::min<long long>(INT_MAX, (1LL << cb) - 1);
     const Shard own{0, 1};
     k_rows_classify<<<grid_for(K, 256, num_sms, 4), 256, 0, s>>>(
-        r.cv, r.base, r.curs, K, std::min(ct_fill_warp(K, num_sms), most), std::min(CT_FILL_GROUP, most),
+        r.cv, r.base, r.curs, nullptr, K, std::min(ct_fill_warp(K, num_sms), most), std::min(CT_FILL_GROUP, most),
         std::min(CB_FILL, most), r.hdr[0], r.hdr[1], r.hdr[2], r.hdr[3], r.inter, r.counters, r.gate, own);
     CountTabArgs t;
     t.x.nbr = r.nbr;

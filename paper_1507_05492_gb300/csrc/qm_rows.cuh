@@ -437,7 +437,8 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
 // One header per non-empty owned community, by run length (as k_classify), from
 // the volumes and cursors of the walk; the cut arcs go to inter[] for the
 // records.
-__global__ void k_rows_classify(const unsigned long long *cv, const unsigned *base, const unsigned long long *curs, int K,
+__global__ void k_rows_classify(const unsigned long long *cv, const unsigned *base, const unsigned long long *curs,
+                                const int *half_len, int K,
                                 int warp_fill, int group_fill, int block_fill, RunHdr *big, RunHdr *small, RunHdr *lng,
                                 RunHdr *mid, int *inter, int *counters, const int *status, Shard own)
 {
@@ -452,9 +453,15 @@ __global__ void k_rows_classify(const unsigned long long *cv, const unsigned *ba
             const int c = (int)cl;
             const unsigned long long v = cv[c];
             if ((v >> VOL_BITS) != 0ull && own.owns(c)) {
-                const unsigned long long q = curs[c];
-                h = RunHdr{c, base[c], (unsigned)q, (unsigned)(v & VOL_MASK)};
-                inter[c] = (int)(q >> 32);
+                const unsigned vol = (unsigned)(v & VOL_MASK);
+                if (half_len) {  // half-edge gathers left 2|E_c^in|: the cut arcs are the rest of the volume
+                    h = RunHdr{c, base[c], (unsigned)half_len[c], vol};
+                    inter[c] = (int)(vol - (unsigned)inter[c]);
+                } else {
+                    const unsigned long long q = curs[c];
+                    h = RunHdr{c, base[c], (unsigned)q, vol};
+                    inter[c] = (int)(q >> 32);
+                }
                 cls = h.m > (unsigned)block_fill ? 2
                       : h.m > (unsigned)group_fill ? 0
                       : h.m > (unsigned)warp_fill ? 3 : 1;

@@ -62,3 +62,21 @@ def test_candidate_counters_around_the_run_length(qm, oracle_mod, k):
     for p, q in enumerate(qm.score_batched(graph, L, [k] * 5)):
         assert q == qm.score(graph, L[p], k)
         check_quality(q, oracle_mod.score(rp, col, L[p].cpu().numpy(), k), f"p={p}")
+
+
+@pytest.mark.parametrize("K", [1, 31, 32, 33, 255, 257, 1100])
+@pytest.mark.parametrize("reorder", [False, True])
+def test_half_edge_members(qm, oracle_mod, K, reorder):
+    """Members of each community placed together by warps of 32 ids, empty ones
+    among them (algorithm 7), on graphs as given and renumbered."""
+    n = 1000
+    rng = np.random.default_rng(K)
+    rp, col = random_graph(n, 5 * n, seed=K + 1)
+    lab = (rng.integers(0, (K + 1) // 2, n) * 2 % K).astype(np.int32)  # about every other id is empty
+    graph, d = qm.Graph(*to_dev(rp, col), reorder=reorder), torch.from_numpy(lab).cuda()
+    ref = qm.score(graph, d, K)
+    check_quality(ref, oracle_mod.score(rp, col, lab, K), f"K={K}")
+    qm.set_tuning(graph, K, 512, 96 * 1024, 48, 7)
+    assert qm.score(graph, d, K) == ref
+    q = qm.score(graph, d, K, per_community=True)
+    assert int(q.pop("per_community")["size"].sum()) == n and q == ref
