@@ -459,8 +459,7 @@ static Shape shape_for(qm_graph *g, int K, bool batched)
     Shape s = it != m.end() ? it->second : (batched ? default_batch_shape() : default_shape());
     if (!batched && g->wt && s.algo != 1) s = default_shape();  // weighted graphs: two-phase pipeline, direct gathers
     // untuned large graphs in their given (unclustered) node order: each edge
-    // gathered once pays there (measured at 10^8 nodes; slower at 3.2*10^7,
-    // whose packed labels stay in L2, and on reordered graphs)
+    // gathered once pays there (HALF_MIN_NODES; not on reordered graphs)
     if (!batched && it == m.end() && g->up_ptr && !g->inv && g->n > HALF_MIN_NODES) s.algo = ALGO_HALF;
     return batched ? resolve_batched(s) : resolve_plain(s);
 }

@@ -50,8 +50,11 @@ constexpr int ALGO_SORT = 6;
 // upper rows; others run algorithm 1.
 constexpr int ALGO_HALF = 7;
 // Untuned calls take ALGO_HALF on graphs in their given node order with more
-// nodes than this.
-constexpr long long HALF_MIN_NODES = 1LL << 26;
+// nodes than this: about where the packed labels (8/3 bytes a node) outgrow L2
+// and the gathers go to DRAM.  Both ends gathered against half-edge, ms a call in
+// random node order, mean degree 19: 3*10^7 nodes 5.40 and 6.87, 4.4*10^7 9.93 and
+// 10.55, 5.1*10^7 12.19 and 12.42, 6*10^7 16.90 and 15.11, 10^8 39.1 and 27.4.
+constexpr long long HALF_MIN_NODES = 13LL << 22;
 
 // Carving of the dynamic shared memory of a community-major block.
 struct SmemPlan {
