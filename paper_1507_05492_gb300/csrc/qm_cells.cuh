@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(CELL_THREADS) k_cells_split(CellArgs a)
 {
     extern __shared__ __align__(16) unsigned sm_cells[];
     __shared__ unsigned long long red[72];
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     unsigned *const buf = sm_cells;                    // the tile's pairs, by bucket
     int *const cur = (int *)(buf + CELL_TILE);         // local cursors; at the end each group's end
     int *const go = cur + (1 << CELL_BITS);            // global place of each group
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
     __shared__ unsigned long long red[72];
     __shared__ unsigned late_s[CELL_TAB_THREADS / 32][32 * 5];
     __shared__ int s_b, s_used, s_at, s_over;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     unsigned *const key = sm_tab, *const cnt = sm_tab + CELL_SLOTS;
     const int tid = threadIdx.x, lane = tid & 31;
     const int range = 1 << a.sh;

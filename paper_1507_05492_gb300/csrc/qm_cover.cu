@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_score(CoverScoreArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_c;
-    if (*a.status || (a.run_if && !*a.run_if)) return;
+    if (block_stopped(a.status) || (a.run_if && !*a.run_if)) return;
     const SmemPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);
@@ -691,7 +691,7 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_cells(CoverCmpArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_c;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const SmemPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);

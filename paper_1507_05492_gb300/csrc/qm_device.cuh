@@ -657,6 +657,16 @@ __device__ __forceinline__ void block_sync()
     __syncwarp();
 }
 
+// Whether a status word is set, one answer for the whole block (all its threads
+// call this).  For kernels with block barriers that may set the word themselves:
+// a block that starts late reads it while earlier blocks write it, and warps that
+// each acted on their own read would leave the others at the barriers, with
+// their part of the shared memory unwritten.
+__device__ __forceinline__ bool block_stopped(const int *status)
+{
+    return __syncthreads_or(*(const volatile int *)status) != 0;
+}
+
 __device__ __forceinline__ void group_sync(int group)
 {
     if (group == 32) __syncwarp();

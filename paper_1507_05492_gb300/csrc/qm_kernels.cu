@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(1024) k_score_cm(ScoreKArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_item;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const SmemPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(1024) k_compare_cm(CompareKArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_item;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const SmemPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);
@@ -992,7 +992,7 @@ __global__ void __launch_bounds__(1024) k_count(CountKArgs a)
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ RunHdr ring[3];
     __shared__ int s_timeout;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const CountPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);
@@ -1190,7 +1190,7 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_count_big(CountTabArgs a)
     __shared__ unsigned long long red[256];
     __shared__ RunHdr ring[3];
     __shared__ int s_timeout;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const int nbig = a.counters[C_BIG_COUNT], nlong = a.counters[C_LONG_COUNT];
     const long long G = gridDim.x, b = blockIdx.x;
     if (b >= nbig && b >= nlong) return;
@@ -1279,7 +1279,7 @@ __global__ void __launch_bounds__(1024) k_count_long(CountCtx x, const RunHdr *l
                                                       SmemPlan p, const int *status)
 {
     extern __shared__ __align__(16) unsigned char sm[];
-    if (*status) return;
+    if (block_stopped(status)) return;
     const int n = counters[C_LONG_COUNT];
     if ((int)blockIdx.x >= n) return;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
@@ -1446,7 +1446,7 @@ __global__ void __launch_bounds__(1024) k_count_sort(CountSortArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ int s_i;
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const SortPlan &p = a.plan;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     unsigned *hist = (unsigned *)(sm + p.hist_off);

@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_count_w_big(CountWArgs a)
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ unsigned late[CB_THREADS / 32][CT_LATE];
     __shared__ unsigned long long red[6 * (CB_THREADS / 32)];
-    if (*a.status) return;
+    if (block_stopped(a.status)) return;
     const int nbig = a.counters[C_BIG_COUNT], nlong = a.counters[C_LONG_COUNT], tid = threadIdx.x;
     const int G = gridDim.x, b = blockIdx.x;
     if (b >= nbig && b >= nlong) return;
