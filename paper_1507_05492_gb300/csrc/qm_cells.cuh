@@ -272,7 +272,9 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                 if (lane == 0 && fresh) atomicAdd(&s_used, (int)fresh);
             }
             {
-                const unsigned fresh = nl && !*(volatile int *)&s_over ? follow(nl) : 0u;
+                // (other warps may be setting the flag: one answer for the warp, which follow() needs whole)
+                const bool over = __any_sync(0xffffffffu, *(volatile int *)&s_over);
+                const unsigned fresh = nl && !over ? follow(nl) : 0u;
                 nl = 0;
                 if (lane == 0 && fresh) atomicAdd(&s_used, (int)fresh);
             }
