@@ -232,17 +232,18 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
         block_sync();
         const int bk = s_b;
         if (bk >= a.nb) break;
-        const int p0 = a.off[(long long)bk * a.ntiles], p1 = a.off[(long long)(bk + 1) * a.ntiles];
+        // (unsigned: the steps of the walk pass 2^31 in the last bucket of that many nodes)
+        const unsigned p0 = a.off[(long long)bk * a.ntiles], p1 = a.off[(long long)(bk + 1) * a.ntiles];
         // classes still to do: hash class r of R, split in two when it overflows
         // (the second halves wait as bits of `todo`, one per doubling)
         unsigned r = 0, R = 1;
         unsigned long long todo = 0;
         while (p0 < p1) {
-            for (int i0 = p0 + (tid & ~31); i0 < p1; i0 += 4 * CELL_TAB_THREADS) {
+            for (unsigned i0 = p0 + (tid & ~31); i0 < p1; i0 += 4 * CELL_TAB_THREADS) {
                 unsigned k[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const int i = i0 + lane + q * CELL_TAB_THREADS;
+                    const unsigned i = i0 + lane + q * CELL_TAB_THREADS;
                     k[q] = i < p1 ? __ldcs(&a.pairs[i]) + 1u : 0u;
                     if (R > 1 && tab_split(k[q], R) != r) k[q] = 0u;
                 }

@@ -611,9 +611,9 @@ __global__ void k_compare_cells(CompareCtx x, const Cell *cells, const int *coun
     CompareAcc acc;
     compare_acc_zero(acc);
     LateCells lc = late_cells(late[threadIdx.x >> 5], x.logt);
-    const int nc = counters[C_NCELLS];
-    for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < nc; i0 += gridDim.x * blockDim.x) {
-        const int i = i0 + (threadIdx.x & 31);
+    const unsigned nc = (unsigned)counters[C_NCELLS];  // (below 2^31; i0 may step past that)
+    for (unsigned i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < nc; i0 += gridDim.x * blockDim.x) {
+        const unsigned i = i0 + (threadIdx.x & 31u);
         Cell c{0, 0, 0u, 0u};
         if (i < nc) c = cells[i];
         const bool in = i < nc && QM_CHK(c.a, x.ka, 30) && QM_CHK(c.b, x.kb, 31);
