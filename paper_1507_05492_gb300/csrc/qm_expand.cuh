@@ -135,15 +135,33 @@ __device__ __forceinline__ u128 warp_sum_u81(u128 v)
     return (u128)a + ((u128)b << 27) + ((u128)c << 54);
 }
 
-// Adds a warp's intra and cut weight sums of community c to its limbs (wl:
+// A community's sum of fixed-point weights in global memory: v = L2 * 2^64 +
+// L1 * 2^32 + L0, updated with 64-bit atomics, where L0 and L1 add up 32-bit
+// chunks and L2 the rest.  Every addition brings at least one arc, of which there
+// are fewer than 2^32, each below 2^63: no word passes 2^64, however a community's
+// nodes lie (limbs_add holds only 2^21 additions).
+__device__ __forceinline__ void wsum_add(unsigned long long *L, u128 v)
+{
+    const unsigned long long l0 = (unsigned)v, l1 = (unsigned)(v >> 32), l2 = (unsigned long long)(v >> 64);
+    if (l0) atomicAdd(&L[0], l0);
+    if (l1) atomicAdd(&L[1], l1);
+    if (l2) atomicAdd(&L[2], l2);
+}
+
+__device__ __forceinline__ i128 wsum_get(const unsigned long long *L)
+{
+    return (i128)(((u128)L[2] << 64) + ((u128)L[1] << 32) + (u128)L[0]);
+}
+
+// Adds a warp's intra and cut weight sums of community c to its sums (wl:
 // six words per community, intra then cut).
 __device__ __forceinline__ void flush_weights(unsigned long long *wl, int c, u128 w_in, u128 w_out, int lane)
 {
     w_in = warp_sum_u81(w_in);
     w_out = warp_sum_u81(w_out);
     if (lane == 0) {
-        if (w_in) limbs_add(wl + (size_t)c * 6, (i128)w_in);
-        if (w_out) limbs_add(wl + (size_t)c * 6 + 3, (i128)w_out);
+        if (w_in) wsum_add(wl + (size_t)c * 6, w_in);
+        if (w_out) wsum_add(wl + (size_t)c * 6 + 3, w_out);
     }
 }
 

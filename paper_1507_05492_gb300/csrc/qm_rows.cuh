@@ -363,7 +363,7 @@ __device__ __forceinline__ void rows_mixed(const RowsArgs &a, const int *col, co
 
 // Intra and cut weight sums of a mixed chunk, a lane per node over its arcs
 // [rel, end) (the chunk's weights are in L1 by then), added to its community's
-// limbs.
+// sums.
 __device__ __forceinline__ void rows_mixed_weights(const RowsArgs &a, const float *wt, const unsigned char *own,
                                                    unsigned rel, unsigned end, int c, bool node)
 {
@@ -373,8 +373,8 @@ __device__ __forceinline__ void rows_mixed_weights(const RowsArgs &a, const floa
         const unsigned long long f = w_fixed(__ldg(&wt[e]));
         if (own[e] & ROWS_CUT) w_out += f; else w_in += f;
     }
-    if (w_in) limbs_add(a.wl + (size_t)c * 6, (i128)w_in);
-    if (w_out) limbs_add(a.wl + (size_t)c * 6 + 3, (i128)w_out);
+    if (w_in) wsum_add(a.wl + (size_t)c * 6, w_in);
+    if (w_out) wsum_add(a.wl + (size_t)c * 6 + 3, w_out);
 }
 
 template <bool WT, int LAB, bool HI>

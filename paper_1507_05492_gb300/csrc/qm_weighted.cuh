@@ -10,7 +10,7 @@
 // Weights are float32 (0 or in [2^-20, 2^20)); each is an exact fixed-point
 // integer w * 2^43, so every weight sum below is exact:
 //   - k_rows<true> sums each community's intra-arc weights (2 W_c^in) and
-//     cut-arc weights (W_c^out) into three-limb integers, and packs the cut
+//     cut-arc weights (W_c^out) into three-word integers, and packs the cut
 //     arcs' weights beside their labels;
 //   - k_count_w_tab and k_count_w_big count each community's run in a
 //     shared-memory table (|E_ci,cj| for every neighbour cj) and then, in a
@@ -461,7 +461,7 @@ __global__ void k_score_terms_w(const unsigned long long *cv, const unsigned lon
         const long long ein = (long long)(same / 2), eout = (long long)(vol - same);
         double qs_unweighted, dens, contr, expn, cond;
         community_terms(ein, eout, size, E, qs_unweighted, dens, contr, expn, cond);
-        const i128 win2 = limbs_get(wl + (size_t)c * 6), wout = limbs_get(wl + (size_t)c * 6 + 3);
+        const i128 win2 = wsum_get(wl + (size_t)c * 6), wout = wsum_get(wl + (size_t)c * 6 + 3);
         const double fin = __ddiv_rn(i128_to_double(win2), W2);          // W_c^in / W
         const double fvol = __ddiv_rn(i128_to_double(win2 + wout), W2);  // (2 W_c^in + W_c^out) / (2W)
         const double qwt = __dsub_rn(fin, __dmul_rn(fvol, fvol));

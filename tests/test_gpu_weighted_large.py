@@ -1,0 +1,63 @@
+"""Weighted sums of communities of millions of nodes.  Nodes of one parity are
+linked among themselves only (u to u +- 2, 4, ..) and the labels are the parity,
+so the two communities alternate along the node order, every node's weights are
+added to its community's sum apart, and Q_w follows from the weights' exact sums:
+    Q_w = sum_c W_c / W - (W_c / W)^2
+with fractional weights, whose fixed-point values fill every bit of a sum's low
+word.  Then a hub whose row sums to more than 2^81 in a lane."""
+from fractions import Fraction
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def qm():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1507_05492_gb300 import qm as q
+    return q
+
+
+def fixed_sum(x):
+    """Exact sum of float32 weights as an integer multiple of 2^-43."""
+    v = (x.double() * 2.0 ** 43).long()
+    return (int((v >> 24).sum()) << 24) + int((v & 0xFFFFFF).sum())
+
+
+# degree 6: a warp's 32 nodes are walked together; 80: their rows exceed what it
+# tabulates, and each stretch of a label is walked apart
+@pytest.mark.parametrize("n,half", [(12_000_000, 3), (10_000_000, 40)])
+def test_alternating_communities(qm, n, half):
+    gen = torch.Generator(device="cuda").manual_seed(half)
+    deg = 2 * half
+    u = torch.arange(n, dtype=torch.int32, device="cuda")
+    edge = torch.rand(half, n, generator=gen, device="cuda") * 4.95 + 0.05  # edge[d - 1][u]: weight of (u, u + 2d)
+    col = torch.empty(n, deg, dtype=torch.int32, device="cuda")
+    wt = torch.empty(n, deg, dtype=torch.float32, device="cuda")
+    for d in range(1, half + 1):
+        col[:, half - d] = (u - 2 * d) % n
+        wt[:, half - d] = edge[d - 1].roll(2 * d)
+        col[:, half + d - 1] = (u + 2 * d) % n
+        wt[:, half + d - 1] = edge[d - 1]
+    for part in (slice(0, deg), slice(n - deg, n)):  # the rows that wrap around
+        order = col[part].argsort(dim=1)
+        col[part], wt[part] = col[part].gather(1, order), wt[part].gather(1, order)
+    row_ptr = torch.arange(n + 1, dtype=torch.int64, device="cuda") * deg
+    graph = qm.Graph(row_ptr, col.view(-1), weights=wt.view(-1))
+    W = [sum(fixed_sum(edge[d][p::2]) for d in range(half)) for p in (0, 1)]
+    share = [Fraction(x, sum(W)) for x in W]
+    dens = Fraction(deg, n // 2 - 1)  # 2 E_in / (s (s - 1))
+    for K in (2, 7):
+        q = qm.score(graph, (u % 2).contiguous(), K)
+        Q = sum(x - x * x for x in share)
+        Qds = sum(x * dens - (x * dens) ** 2 for x in share)
+        assert abs(q["modularity"] - float(Q)) <= 1e-12 * 2
+        assert abs(q["modularity_density"] - float(Qds)) <= 1e-12 * 2 * float(dens)
+        assert q["cut_edges_total"] == 0 and q["intra_edges_total"] == n * half
+    parts = [qm.score_part(graph, (u % 2).contiguous(), 2, r, 2) for r in range(2)]  # a shard per community
+    q = qm.finalize_part(qm.combine_parts(parts))
+    assert abs(q["modularity"] - float(Q)) <= 1e-12 * 2
+    graph.close()
