@@ -124,15 +124,16 @@ __device__ __forceinline__ void expand_range(unsigned e_lo, unsigned e_hi, int c
     }
 }
 
-// Warp total of a value below 2^76 (a lane's sum of a few fixed-point weights
-// below 2^63): three 27-bit chunks, each added by one redux.
-__device__ __forceinline__ u128 warp_sum_u81(u128 v)
+// Warp total of lane sums of fixed-point weights: four 27-bit chunks, each added
+// by one redux.  A lane holds a 32nd of the arcs of a stretch of rows, fewer than
+// 2^27 weights below 2^63, so its sum is below 2^90.
+__device__ __forceinline__ u128 warp_sum_u108(u128 v)
 {
     constexpr unsigned M = (1u << 27) - 1u;
-    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)v & M);
-    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 27) & M);
-    const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 54) & M);
-    return (u128)a + ((u128)b << 27) + ((u128)c << 54);
+    u128 r = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r += (u128)__reduce_add_sync(0xffffffffu, (unsigned)(v >> (27 * k)) & M) << (27 * k);
+    return r;
 }
 
 // A community's sum of fixed-point weights in global memory: v = L2 * 2^64 +
@@ -157,8 +158,8 @@ __device__ __forceinline__ i128 wsum_get(const unsigned long long *L)
 // six words per community, intra then cut).
 __device__ __forceinline__ void flush_weights(unsigned long long *wl, int c, u128 w_in, u128 w_out, int lane)
 {
-    w_in = warp_sum_u81(w_in);
-    w_out = warp_sum_u81(w_out);
+    w_in = warp_sum_u108(w_in);
+    w_out = warp_sum_u108(w_out);
     if (lane == 0) {
         if (w_in) wsum_add(wl + (size_t)c * 6, w_in);
         if (w_out) wsum_add(wl + (size_t)c * 6 + 3, w_out);

@@ -61,3 +61,22 @@ def test_alternating_communities(qm, n, half):
     q = qm.finalize_part(qm.combine_parts(parts))
     assert abs(q["modularity"] - float(Q)) <= 1e-12 * 2
     graph.close()
+
+
+def test_heavy_hub(qm):
+    """A star of 10^7 leaves with the largest weights, one leaf in a community of its own:
+    W_0 / W = (m - 1) / m, and vol_0 = (2 m - 1) w, vol_1 = w of 2 W = 2 m w."""
+    m = 10_000_000
+    leaf = torch.arange(1, m + 1, dtype=torch.int32, device="cuda")
+    row_ptr = torch.cat([torch.zeros(1, dtype=torch.int64, device="cuda"),
+                         m + torch.arange(m + 1, dtype=torch.int64, device="cuda")])
+    weights = torch.full((2 * m,), 1048575.9375, device="cuda")
+    labels = torch.zeros(m + 1, dtype=torch.int32, device="cuda")
+    labels[m] = 1
+    graph = qm.Graph(row_ptr, torch.cat([leaf, torch.zeros_like(leaf)]), weights=weights)
+    q = qm.score(graph, labels, 2)
+    Q = Fraction(m - 1, m) - Fraction(2 * m - 1, 2 * m) ** 2 - Fraction(1, 2 * m) ** 2
+    assert q["intra_edges_total"] == m - 1
+    # (m - 1) / m, (2 m - 1) / (2 m) and its square are rounded once each
+    assert abs(q["modularity"] - float(Q)) <= 1e-12 * 2
+    graph.close()
