@@ -221,6 +221,7 @@ __device__ __forceinline__ void ct_count_run(const CountCtx &x, const RunHdr &h,
     // one step of CT_UNROLL entries a lane from e0 (warp-uniform) on
     auto step = [&](int e0, auto last) {
         constexpr bool LAST = decltype(last)::value;
+        constexpr bool EVERY = !LAST && MODE != CT_MIXED && !QM_CHECKED;  // no entry is skipped
         int lv[CT_UNROLL];
         unsigned cur[CT_UNROLL];
         Rcp rj[CT_UNROLL];
@@ -229,8 +230,8 @@ __device__ __forceinline__ void ct_count_run(const CountCtx &x, const RunHdr &h,
             lv[k] = nx[k];
             if ((LAST && e0 + lane + GS * k >= m) || (MODE == CT_MIXED && lv[k] < c) || !QM_CHK(lv[k], x.K, 6))
                 lv[k] = -1;
-            if (LAST || MODE == CT_MIXED) rj[k] = Rcp{0ull, 0ull};
-            if ((!LAST && MODE != CT_MIXED) || lv[k] >= 0) rj[k] = ld_rcp(&x.recip[lv[k]]);
+            if (!EVERY) rj[k] = Rcp{0ull, 0ull};
+            if (EVERY || lv[k] >= 0) rj[k] = ld_rcp(&x.recip[lv[k]]);
         }
         if (!LAST)
 #pragma unroll
@@ -240,7 +241,7 @@ __device__ __forceinline__ void ct_count_run(const CountCtx &x, const RunHdr &h,
         for (int k = 0; k < CT_UNROLL; ++k) {
             const unsigned hs = ((unsigned)lv[k] * 0x9E3779B1u) >> shift;
             cur[k] = 0u;
-            if ((!LAST && MODE != CT_MIXED) || lv[k] >= 0) cur[k] = atomicCAS(&slot[hs], 0u, (unsigned)lv[k] * one + one);
+            if (EVERY || lv[k] >= 0) cur[k] = atomicCAS(&slot[hs], 0u, (unsigned)lv[k] * one + one);
         }
 #pragma unroll
         for (int k = 0; k < CT_UNROLL; ++k) {
@@ -258,7 +259,7 @@ __device__ __forceinline__ void ct_count_run(const CountCtx &x, const RunHdr &h,
                 rj[k].lo = above ? rj[k].lo : 0ull;
                 rj[k].hi = above ? rj[k].hi : 0ull;
                 counts[2] += above ? 1u : 0u;
-            } else if (MODE == CT_MIXED) {
+            } else if (MODE == CT_MIXED || QM_CHECKED) {
                 counts[2] += lv[k] >= 0 ? 1u : 0u;
             }
             u192_add_chain(inner, rj[k]);
@@ -273,7 +274,7 @@ __device__ __forceinline__ void ct_count_run(const CountCtx &x, const RunHdr &h,
         reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
     ct_totals<FULL, GS>(counts, inner, inner_full, red);
     if (gtid == 0) {
-        const unsigned long long entries = MODE == CT_ABOVE ? (unsigned)m : counts[2];
+        const unsigned long long entries = MODE == CT_ABOVE && !QM_CHECKED ? (unsigned)m : counts[2];
         put_record(x, c, h.vol, h.m, entries - counts[0], entries + counts[1], inner, inner_full);
     }
     ct_sync<GS>();  // the cleared slots and `red` are free for the next run

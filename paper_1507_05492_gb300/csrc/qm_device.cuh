@@ -48,10 +48,12 @@ __device__ __forceinline__ bool qm_chk_ex(long long i, long long n, int site, lo
     atomicAdd(&qm_dbg_rec[3], 1ull);
     return false;
 }
+constexpr bool QM_CHECKED = true;
 #define QM_CHK(i, n, site) qm_chk_ex((long long)(i), (long long)(n), (site), 0, 0, 0, 0)
 #define QM_CHKX(i, n, site, a, b, c, d) \
     qm_chk_ex((long long)(i), (long long)(n), (site), (long long)(a), (long long)(b), (long long)(c), (long long)(d))
 #else
+constexpr bool QM_CHECKED = false;
 #define QM_CHK(i, n, site) true
 #define QM_CHKX(i, n, site, a, b, c, d) true
 #endif
