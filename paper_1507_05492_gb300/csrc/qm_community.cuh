@@ -1017,7 +1017,9 @@ __device__ __forceinline__ void count_run_general(const CountCtx &x, const RunHd
     const bool full = x.full != 0;
     const int *src = x.nbr + h.a0;
     const unsigned cap_keys = (unsigned)tab.max_used;
-    unsigned R = m <= cap_keys ? 1u : (unsigned)min((unsigned long long)R_MAX, (5ull * m + 4ull * cap_keys - 1) / (4ull * cap_keys));
+    // distinct keys at most: the labels counted, or the entries
+    const unsigned keys = min(m, (unsigned)(full ? x.K - 1 : x.K - 1 - c));
+    unsigned R = keys <= cap_keys ? 1u : (unsigned)min((unsigned long long)R_MAX, (5ull * keys + 4ull * cap_keys - 1) / (4ull * cap_keys));
     for (;;) {
         unsigned long long slots = 0, cnt2 = 0;
         U192 inner, inner_full;

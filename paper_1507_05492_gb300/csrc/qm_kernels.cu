@@ -1124,12 +1124,12 @@ struct CountTabArgs {
     const RunHdr *mid;    // runs for whole blocks of k_count_tab
     const RunHdr *small;  // runs for single warps
     const RunHdr *big;    // runs for k_count_big, staged
-    const RunHdr *lng;    // runs longer than those, counted in hash classes
+    const RunHdr *lng;    // runs longer than those
+    RunHdr *over;         // where k_count_big lists the ones beyond its table (k_count_tab's `mid`, done by then)
     int *counters;
     const int *status;
     int cb;               // bits of a table word left for the repeats
     unsigned stage_wait;  // k_count_big: polls of each staging wait before the block gives up
-    SmemPlan plan;        // k_count_big: tables of the hash-class count
 };
 
 template <int MODE>
@@ -1178,8 +1178,15 @@ __global__ void __launch_bounds__(CT_THREADS, CT_BLOCKS) k_count_tab(CountTabArg
 // wait; the next copy is issued only after the current one has landed, so at
 // most one is in flight when a wait expires).  Then the list of the runs beyond
 // that: up to CB_FILL_LONG entries (and below 2^cb) with one table in the whole
-// shared memory, longer ones by hash classes (count_run_general).
+// shared memory; longer ones are k_count_long's.
 constexpr int CB_SMEM = 16 + CB_WORDS * 4 + 2 * CB_STAGE * 4;
+
+// The longest run that the one-word tables count.
+__host__ __device__ static inline int tab_longest(int cb)
+{
+    return cb < 31 && (1 << cb) - 1 < CB_FILL_LONG ? (1 << cb) - 1 : CB_FILL_LONG;
+}
+
 static_assert(CB_SMEM >= 16 + CB_WORDS_LONG * 4, "the unstaged table fits");
 
 template <int MODE>
@@ -1247,40 +1254,34 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_count_big(CountTabArgs a)
     }
     if (b >= nlong) return;
     block_sync();
-    const unsigned most = min((unsigned)CB_FILL_LONG, (1u << a.cb) - 1u);
-    bool general = false;
     for (int i = tid; i < CB_WORDS_LONG / 4; i += CB_THREADS)
         reinterpret_cast<uint4 *>(slot)[i] = make_uint4(0u, 0u, 0u, 0u);
     block_sync();
+    const unsigned most = (unsigned)tab_longest(a.cb);
     for (long long i = b; i < nlong; i += G) {
         const RunHdr h = a.lng[i];
         if (h.m <= most) ct_count_run<MODE, false, CB_THREADS>(a.x, h, a.x.nbr + h.a0, slot, a.cb, tid, late[tid >> 5], red);
-        else general = true;
+        else if (tid == 0) a.over[atomicAdd(&a.counters[C_OVF_COUNT], 1)] = h;
     }
-    if (!general) return;
-    block_sync();
-    const SmemPlan &p = a.plan;
-    int *ctl = (int *)(sm + p.ctl_off);
-    unsigned long long *lslot = (unsigned long long *)(sm + p.slot_off);
-    int *used = (int *)(sm + p.used_off);
-    for (int i = tid; i < p.cap; i += CB_THREADS) lslot[i] = 0ull;
-    if (tid < 2) ctl[tid] = 0;
-    block_sync();
-    const SmemTable tb{lslot, used, &ctl[0], &ctl[1], p.cap, p.max_used};
-    for (long long i = b; i < nlong; i += G)
-        if (a.lng[i].m > most)
-            count_run_general(a.x, a.lng[i], tb, tid, CB_THREADS, (unsigned long long *)(sm + p.red_off));
 }
 
 // Runs longer than the block tables of k_count hold at 3/4 load (and any run
-// of 2^24 entries or more), one block each, with 64-bit counts
-// (count_run_general).
-__global__ void __launch_bounds__(1024) k_count_long(CountCtx x, const RunHdr *lng, const int *counters,
+// of 2^24 entries or more), or than k_count_big's table takes: one block each
+// with all of an SM's threads and shared memory, claimed one at a time, with
+// 64-bit counts (count_run_general).  The passes over a run are as many as its
+// distinct keys need of this table (13,984 keys; in the 82 KB that a block of
+// k_count_big has, three times as many).  The call at 5*10^5 nodes, labels at
+// random: in hash classes of k_count_big, sized by the entries, 870 ms with two
+// communities and 842 ms with one community of half the nodes; here 81 and 2.8 ms
+// (in k_count_long with classes sized by the entries 239 and 163 ms).  Without such
+// runs it adds a launch, 1.5 us.
+__global__ void __launch_bounds__(1024) k_count_long(CountCtx x, const RunHdr *lng, int *counters, int which,
                                                       SmemPlan p, const int *status)
 {
     extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int s_i;
     if (block_stopped(status)) return;
-    const int n = counters[C_LONG_COUNT];
+    const int n = counters[which];
     if ((int)blockIdx.x >= n) return;
     unsigned long long *red = (unsigned long long *)(sm + p.red_off);
     int *ctl = (int *)(sm + p.ctl_off);
@@ -1288,9 +1289,15 @@ __global__ void __launch_bounds__(1024) k_count_long(CountCtx x, const RunHdr *l
     int *used = (int *)(sm + p.used_off);
     for (int i = threadIdx.x; i < p.cap; i += blockDim.x) slot[i] = 0ull;
     if (threadIdx.x < 2) ctl[threadIdx.x] = 0;
-    block_sync();
     const SmemTable tb{slot, used, &ctl[0], &ctl[1], p.cap, p.max_used};
-    for (int i = blockIdx.x; i < n; i += gridDim.x) count_run_general(x, lng[i], tb, threadIdx.x, blockDim.x, red);
+    for (;;) {
+        block_sync();
+        if (threadIdx.x == 0) s_i = atomicAdd(&counters[C_OVF_NEXT], 1);
+        block_sync();
+        const int i = s_i;
+        if (i >= n) return;
+        count_run_general(x, lng[i], tb, threadIdx.x, blockDim.x, red);
+    }
 }
 
 // ------------------------------------------------------------------ phase B by sorting (algorithm 6)
@@ -2146,13 +2153,12 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
         t.small = ws.hdr_small;
         t.big = ws.hdr_big;
         t.lng = ws.hdr_long;
+        t.over = ws.hdr_mid;
         t.counters = ws.counters;
         t.status = ws.status;
         t.cb = cb;
         t.stage_wait = a.stage_wait;
-        t.plan = plan_smem(CB_THREADS, CB_SMEM);
         const int tg = (int)std::min<long long>((long long)num_sms * CT_BLOCKS, K), bg = std::min(2 * num_sms, K);
-        TRACE("k_count_tab");
         // the binned gathers pack every label, the others only those counted
         const int mode = a.x.full ? CT_FULL : ws.bin_pool ? CT_MIXED : CT_ABOVE;
         TRACE("k_count_tab");
@@ -2186,12 +2192,11 @@ int launch_score2(const GraphDev &g, const int *labels, int K, const ScoreWs &ws
         if (a.x.full) k_count<EpochTable, true><<<count_grid, sh.threads, sh.smem_bytes, s>>>(a);
         else k_count<EpochTable, false><<<count_grid, sh.threads, sh.smem_bytes, s>>>(a);
     }
-    if (!tab) {
-        TRACE("k_count_long");
-        k_count_long<<<std::min(num_sms, K), 1024, MAX_DYN_SMEM, s>>>(a.x, ws.hdr_long, ws.counters,
-                                                                      plan_smem(1024, MAX_DYN_SMEM), ws.status);
-    }
-    launches += 2;
+    TRACE("k_count_long");
+    k_count_long<<<std::min(num_sms, K), 1024, MAX_DYN_SMEM, s>>>(a.x, tab ? ws.hdr_mid : ws.hdr_long, ws.counters,
+                                                                  tab ? C_OVF_COUNT : C_LONG_COUNT,
+                                                                  plan_smem(1024, MAX_DYN_SMEM), ws.status);
+    launches += tab ? 3 : 2;
     PerCommDev pcd{};
     if (pc) pcd = *pc;
     TRACE("k_score_terms");
@@ -2227,18 +2232,20 @@ int launch_cover_runs(const CoverRuns &r, int K, long long E, unsigned long long
     t.big = r.hdr[0];
     t.small = r.hdr[1];
     t.lng = r.hdr[2];
+    t.over = r.hdr[3];
     t.mid = r.hdr[3];
     t.counters = r.counters;
     t.status = r.gate;
     t.cb = cb;
     t.stage_wait = g_stage_wait.load();
-    t.plan = plan_smem(CB_THREADS, CB_SMEM);
     k_count_tab<CT_ABOVE><<<(int)std::min<long long>((long long)num_sms * CT_BLOCKS, K), CT_THREADS, 0, s>>>(t);
     k_count_big<CT_ABOVE><<<std::min(2 * num_sms, K), CB_THREADS, CB_SMEM, s>>>(t);
+    k_count_long<<<std::min(num_sms, K), 1024, MAX_DYN_SMEM, s>>>(t.x, t.over, r.counters, C_OVF_COUNT,
+                                                                  plan_smem(1024, MAX_DYN_SMEM), r.gate);
     const int tt = terms_threads(K, num_sms);
     k_score_terms<<<grid_for(K, tt, num_sms, 2), tt, 0, s>>>(nullptr, r.cv, r.rec, K, E, PerCommDev{}, gacc, r.gate, own,
                                                              ScoreOut{});
-    return cudaGetLastError() == cudaSuccess ? 4 : -1;
+    return cudaGetLastError() == cudaSuccess ? 5 : -1;
 }
 
 int launch_score_fin(const unsigned long long *gacc, const int *status, long long n, long long E, qm_quality *out,
