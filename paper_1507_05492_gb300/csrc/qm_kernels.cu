@@ -1810,8 +1810,9 @@ int launch_permute_hist(const int *labels, const int *inv, const long long *row_
                         const ScoreWs &ws, bool rows, int num_sms, cudaStream_t s)
 {
     if (rows) {
-        k_permute_vol<<<grid_for((n + HIST_UNROLL - 1) / HIST_UNROLL, 256, num_sms, 8), 256, 0, s>>>(
-            labels, inv, row_ptr, n, out, K, ws.cv, ws.status);
+        const int smem = K <= VOL_SMEM_IDS ? K * 8 : 0;
+        k_permute_vol<<<grid_for((n + HIST_UNROLL - 1) / HIST_UNROLL, 256, num_sms, 8), 256, smem, s>>>(
+            labels, inv, row_ptr, n, out, K, ws.cv, ws.status, smem ? 1 : 0);
         return cudaGetLastError() == cudaSuccess ? 1 : -1;
     }
     const int hist_smem = (K <= 12288) ? K * 4 : 0;

@@ -605,7 +605,7 @@ __global__ void k_pb_tile(const int *__restrict__ labels, const unsigned short *
 template <int B, bool V4>
 __global__ void k_pb_window(const int *__restrict__ tmp, const unsigned short *__restrict__ dloc, long long n, int wb,
                             int nw, int *__restrict__ out, int *size, int K, const long long *__restrict__ row_ptr,
-                            unsigned long long *cv);
+                            unsigned long long *cv, int counts_at);
 
 template <int B, bool V4>
 static cudaError_t pb_set_smem_v(size_t smem_max)
@@ -809,16 +809,19 @@ __global__ void __launch_bounds__(PB_THREADS, 2) k_pb_tile(const int *__restrict
 
 // Pass 2, one window per block step: slots into shared memory at their new
 // ids, then the window out in order.  With `size`, the labels are counted as
-// k_hist does, with `cv` as k_hist_vol does (pass 1 has checked them).
+// k_hist does, with `cv` as k_permute_vol does (in shared memory from byte
+// counts_at on, where that is not 0; pass 1 has checked the labels).
 template <int B, bool V4>
 __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restrict__ tmp,
                                                           const unsigned short *__restrict__ dloc, long long n,
                                                           int wb, int nw, int *__restrict__ out, int *size, int K,
                                                           const long long *__restrict__ row_ptr,
-                                                          unsigned long long *cv)
+                                                          unsigned long long *cv, int counts_at)
 {
     extern __shared__ __align__(16) unsigned char smb[];
     const int T = blockDim.x, tid = threadIdx.x;
+    unsigned *const shv = counts_at ? (unsigned *)(smb + counts_at) : nullptr;
+    if (shv) vol_smem_zero(shv, K);
     for (int w = blockIdx.x; w < nw; w += gridDim.x) {
         const long long base = (long long)w << wb;
         const int len = (int)min(n - base, 1LL << wb);
@@ -838,7 +841,9 @@ __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restri
 #pragma unroll
             for (int q = 0; q < PB_UNROLL; ++q) {
                 const bool ok = (unsigned)l[q] < (unsigned)K;
-                if (cv) {
+                if (shv) {
+                    vol_smem_add_warp(shv, K, l[q], d[q], ok);
+                } else if (cv) {
                     vol_add_warp(cv, l[q], d[q], ok);
                 } else if (size) {
                     const unsigned act = __ballot_sync(0xffffffffu, ok);
@@ -851,6 +856,7 @@ __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restri
         }
         __syncthreads();
     }
+    if (shv) vol_smem_flush(shv, K, cv);
 }
 
 int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long long *row_ptr, long long n, int *tmp,
@@ -860,15 +866,20 @@ int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long 
     const int B = narrow ? 3 : 4;
     const size_t p1 = pb_pass1_smem(pb.tb, pb.nw, B), p2 = pb_pass2_smem(pb.wb, B);
     if (p1 > pb.smem_max || p2 > pb.smem_max) return 0;  // 4-byte labels do not fit: gather them instead
+    const size_t at = (p2 + 15) / 16 * 16;  // the counters behind the window
+    const bool counts = cv && K <= VOL_SMEM_IDS && at + (size_t)K * 8 <= pb.smem_max;
+    const size_t p2c = counts ? at + (size_t)K * 8 : p2;
     // resident blocks per SM: two of PB_THREADS at most, and what shared memory allows
     auto per_sm = [](size_t smem) { return (int)std::max<size_t>(1, std::min<size_t>(2, 233472 / (smem + 1024))); };
-    const int g1 = std::min(pb.ntiles, num_sms * per_sm(p1)), g2 = std::min(pb.nw, num_sms * per_sm(p2));
+    const int g1 = std::min(pb.ntiles, num_sms * per_sm(p1)), g2 = std::min(pb.nw, num_sms * per_sm(p2c));
     // four at a time where every tile (window) start keeps the 16-byte alignment
     const bool v1 = pb.tb >= 2 && ((uintptr_t)labels & 15) == 0, v2 = pb.wb >= 2;
     auto pass1 = [&](auto kern) {
         kern<<<g1, PB_THREADS, p1, s>>>(labels, pb.lpos, pb.toff, pb.tlb, n, pb.tb, pb.nw, pb.ntiles, K, tmp, status);
     };
-    auto pass2 = [&](auto kern) { kern<<<g2, PB_THREADS, p2, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K, row_ptr, cv); };
+    auto pass2 = [&](auto kern) { 
+        kern<<<g2, PB_THREADS, p2c, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K, row_ptr, cv, counts ? (int)at : 0);
+    };
     if (tr) tr("k_pb_tile", s);
     if (narrow)
         v1 ? pass1(k_pb_tile<3, true>) : pass1(k_pb_tile<3, false>);
