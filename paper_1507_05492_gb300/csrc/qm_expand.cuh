@@ -154,16 +154,43 @@ __device__ __forceinline__ i128 wsum_get(const unsigned long long *L)
     return (i128)(((u128)L[2] << 64) + ((u128)L[1] << 32) + (u128)L[0]);
 }
 
-// Adds a warp's intra and cut weight sums of community c to its sums (wl:
-// six words per community, intra then cut).
-__device__ __forceinline__ void flush_weights(unsigned long long *wl, int c, u128 w_in, u128 w_out, int lane)
+// The same sum below 2^96 in three 32-bit words of shared memory, the carries
+// passed on by whoever causes them.
+__device__ __forceinline__ void wsum_add_smem(unsigned *L, u128 v)
+{
+    const unsigned l0 = (unsigned)v;
+    unsigned carry = l0 && atomicAdd(&L[0], l0) > ~l0 ? 1u : 0u;
+    const unsigned l1 = (unsigned)(v >> 32) + carry;
+    if (l1) carry = atomicAdd(&L[1], l1) > ~l1 ? 1u : 0u;  // (else the carry, if any, went through l1)
+    const unsigned l2 = (unsigned)(v >> 64) + carry;
+    if (l2) atomicAdd(&L[2], l2);
+}
+
+// Where a kernel adds up the communities' weights: six words per community,
+// intra then cut, in global memory, or (few communities) in a block's shared
+// memory, whose sums it adds to the global ones at its end.
+struct WeightSums {
+    unsigned long long *wl;
+    unsigned *smem;  // null: straight to wl
+
+    __device__ __forceinline__ void add(int c, u128 w_in, u128 w_out) const
+    {
+        if (smem) {
+            if (w_in) wsum_add_smem(smem + c * 6, w_in);
+            if (w_out) wsum_add_smem(smem + c * 6 + 3, w_out);
+        } else {
+            if (w_in) wsum_add(wl + (size_t)c * 6, w_in);
+            if (w_out) wsum_add(wl + (size_t)c * 6 + 3, w_out);
+        }
+    }
+};
+
+// Adds a warp's intra and cut weight sums of community c.
+__device__ __forceinline__ void flush_weights(const WeightSums &ws, int c, u128 w_in, u128 w_out, int lane)
 {
     w_in = warp_sum_u108(w_in);
     w_out = warp_sum_u108(w_out);
-    if (lane == 0) {
-        if (w_in) wsum_add(wl + (size_t)c * 6, w_in);
-        if (w_out) wsum_add(wl + (size_t)c * 6 + 3, w_out);
-    }
+    if (lane == 0) ws.add(c, w_in, w_out);
 }
 
 // ---------------------------------------------------------------- half-edge gathers

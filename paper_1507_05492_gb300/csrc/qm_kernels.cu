@@ -1972,6 +1972,7 @@ static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const 
     a.wt = g.wt;
     a.nbrw = ws.nbrw;
     a.wl = ws.wl;
+    a.K = K;
     if (g.wt) {
         TRACE("k_rows");
         launch_rows<true, LAB_PLAIN, false>(a, num_sms, s);

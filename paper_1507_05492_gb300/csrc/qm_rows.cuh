@@ -197,6 +197,7 @@ struct RowsArgs {
     const float *wt;                  // weighted graphs
     float *nbrw;
     unsigned long long *wl;
+    int K;
 };
 
 // Labels of U far-end nodes v (with CHECK some may be -1: none, and stay so),
@@ -368,8 +369,8 @@ __device__ __forceinline__ void rows_mixed(const RowsArgs &a, const int *col, co
 // Intra and cut weight sums of a mixed chunk, a lane per node over its arcs
 // [rel, end) (the chunk's weights are in L1 by then), added to its community's
 // sums.
-__device__ __forceinline__ void rows_mixed_weights(const RowsArgs &a, const float *wt, const unsigned char *own,
-                                                   unsigned rel, unsigned end, int c, bool node)
+__device__ __forceinline__ void rows_mixed_weights(const RowsArgs &a, const WeightSums &ws, const float *wt,
+                                                   const unsigned char *own, unsigned rel, unsigned end, int c, bool node)
 {
     if (!node || rel == end || !a.own.owns(c)) return;
     u128 w_in = 0, w_out = 0;
@@ -377,9 +378,15 @@ __device__ __forceinline__ void rows_mixed_weights(const RowsArgs &a, const floa
         const unsigned long long f = w_fixed(__ldg(&wt[e]));
         if (own[e] & ROWS_CUT) w_out += f; else w_in += f;
     }
-    if (w_in) wsum_add(a.wl + (size_t)c * 6, w_in);
-    if (w_out) wsum_add(a.wl + (size_t)c * 6 + 3, w_out);
+    ws.add(c, w_in, w_out);
 }
+
+// Up to this many label ids a block adds up their weights in shared memory: a
+// node of a mixed chunk (a stretch, where rows are long) adds up to six words,
+// and with few communities all SMs' additions queue for few of them.  The call at
+// 2*10^6 nodes as given, two communities in turn, global words against shared: 2.59
+// and 0.37 ms; ten 1.60 and 0.37, a hundred 0.52 and 0.37 (a thousand, global: 0.38).
+constexpr int ROWS_W_IDS = 256;
 
 template <bool WT, int LAB, bool HI>
 __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows(RowsArgs a)
@@ -387,8 +394,14 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
     __shared__ int cw_s[ROWS_THREADS / 32][32];
     __shared__ unsigned bw_s[ROWS_THREADS / 32][32];
     __shared__ unsigned char own_s[ROWS_THREADS / 32][ROWS_OWN_CAP];
+    __shared__ unsigned wsum_s[WT ? ROWS_W_IDS * 6 : 1];
     if (*a.status) return;
     if (a.bx_bad && (LAB == LAB_BLOCKS) == (*a.bx_bad != 0)) return;
+    const WeightSums ws{a.wl, WT && a.K <= ROWS_W_IDS ? wsum_s : nullptr};
+    if (WT && ws.smem) {
+        for (int i = threadIdx.x; i < a.K * 6; i += ROWS_THREADS) wsum_s[i] = 0u;
+        block_sync();
+    }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned long long keep = l2_policy_evict_last();
     const long long nwarps = (long long)gridDim.x * (ROWS_THREADS / 32);
@@ -417,7 +430,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
                 if (e_lo == e_hi || !a.own.owns(cc)) continue;
                 u128 w_in = 0, w_out = 0;
                 rows_one<WT, LAB, HI>(a, col, WT ? a.wt + r0 : nullptr, e_lo, e_hi, cc, cb, keep, lane, w_in, w_out);
-                if (WT) flush_weights(a.wl, cc, w_in, w_out, lane);
+                if (WT) flush_weights(ws, cc, w_in, w_out, lane);
             }
         } else {
             __syncwarp();
@@ -431,9 +444,16 @@ __global__ void __launch_bounds__(ROWS_THREADS, (rows_blocks<WT, LAB>())) k_rows
             rows_mixed<WT, LAB, HI>(a, col, WT ? a.wt + r0 : nullptr, total, own_s[w], cw_s[w], bw_s[w], keep, lane);
             __syncwarp();
             if (WT) {
-                rows_mixed_weights(a, a.wt + r0, own_s[w], rel, end, c, lane < nm);
+                rows_mixed_weights(a, ws, a.wt + r0, own_s[w], rel, end, c, lane < nm);
                 __syncwarp();
             }
+        }
+    }
+    if (WT && ws.smem) {
+        block_sync();
+        for (int i = threadIdx.x; i < a.K * 2; i += ROWS_THREADS) {  // intra and cut sums
+            const unsigned *L = wsum_s + 3 * i;
+            wsum_add(a.wl + 3 * (size_t)i, ((u128)L[2] << 64) | ((u128)L[1] << 32) | (u128)L[0]);
         }
     }
 }

@@ -45,3 +45,24 @@ def test_counts_beside_the_permutation(qm, oracle_mod, K, bits):
         qm.score(graph, bad, K)
     assert e.value.status == qm.QM_EINVAL
     graph.close()
+
+
+# 256 ids: the most whose weights a block adds up in shared memory; 600,000 edges: long rows
+@pytest.mark.parametrize("K", [2, 9, 255, 256, 257])
+@pytest.mark.parametrize("n,m", [(20_011, 60_000), (6_007, 600_000)])
+@pytest.mark.parametrize("reorder", [False, True])
+def test_weights_of_few_communities(qm, oracle_mod, K, n, m, reorder):
+    rp, col = random_graph(n, m, seed=K)
+    src = np.repeat(np.arange(n), np.diff(rp))
+    key = np.minimum(src, col) * np.int64(n) + np.maximum(src, col)
+    rng = np.random.default_rng(K)
+    # over the whole accepted range, so that sums carry from word to word
+    w = np.exp2(rng.uniform(-20, 19.99, n * 3))[key % (3 * n)].astype(np.float32)
+    graph = qm.Graph(*to_dev(rp, col), weights=torch.from_numpy(w).cuda(), reorder=reorder, validate=True)
+    for lab in (rng.integers(0, K, n), np.arange(n) * K // n, np.arange(n) // 12 % K):
+        lab = lab.astype(np.int32)
+        o = oracle_mod.score_weighted(rp, col, w.astype(np.float64), lab, K)
+        q = qm.score(graph, torch.from_numpy(lab).cuda(), K)
+        for name, cond in (("modularity", "cond_modularity"), ("modularity_density", "cond_modularity_density")):
+            assert abs(q[name] - o[name]) <= 1e-12 * max(abs(o[name]), abs(o[cond])), (name, q[name], o[name])
+    graph.close()
