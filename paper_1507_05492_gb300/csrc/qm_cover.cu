@@ -15,8 +15,8 @@
 // unordered pair is charged to its smaller id).  A run's segment is sized by
 // the list lengths of its members' neighbours (k_cover_cap).  The counting,
 // the terms and the sums are the partition path's, so a cover with one
-// community per node gives the partition's bits.  Covers whose segments do not
-// fit the scratch (long lists), and ones of 2^20 ids or more, are transposed
+// community per node gives the partition's bits.  Covers with long lists, ones
+// whose segments do not fit the scratch, and ones of 2^20 ids or more, are transposed
 // into member lists and scored by one block per community (k_cover_score).
 // Measured, 10^6 nodes, a tenth of them in two communities: 2.46 ms by member
 // lists, 0.60 by runs (k_cover_walk 0.27, k_cover_cap 0.14, counting 0.07); the
@@ -45,6 +45,12 @@ namespace {
 
 constexpr int COVER_THREADS = 256;
 constexpr int COVER_SMEM = 48 * 1024;
+// Covers with a longer list than this are scored by member lists: k_cover_walk
+// turns the two ends' lists in step over the 32 arcs of a warp, so that one arc's
+// pairs of communities are walked by all.  5*10^5 nodes, every 500th in L
+// communities, by runs and by member lists, ms: L = 8 0.46 and 1.50, 16 0.74 and
+// 1.59, 32 2.53 and 1.78, 128 88 and 4.6.
+constexpr int COVER_LIST_MAX = 16;
 constexpr int OVL_CAP = 2048;  // overlapping members of one community paired in shared memory
 
 // extra accumulator words after the GC_* words of a comparison
@@ -181,11 +187,13 @@ CoverWs carve_cover_compare_ws(void *base, long long n, long long ma, int ka, lo
 // ------------------------------------------------------------------ bringing a cover to the stored order
 
 // List length of every stored node (its caller node's list when the graph is
-// renumbered), with the offsets' checks (non-decreasing from 0 to m).
-__global__ void k_cover_len(const long long *mptr, long long n, long long m, const int *inv, int *len, int *status)
+// renumbered), with the offsets' checks (non-decreasing from 0 to m).  *too_long
+// (when wanted) is set where a list is longer than COVER_LIST_MAX.
+__global__ void k_cover_len(const long long *mptr, long long n, long long m, const int *inv, int *len, int *status,
+                            int *too_long)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    bool bad = false;
+    bool bad = false, above = false;
     for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) {
         const long long u = inv ? (long long)__ldg(&inv[j]) : j;
         const long long b = __ldg(&mptr[u]), e = __ldg(&mptr[u + 1]);
@@ -194,10 +202,12 @@ __global__ void k_cover_len(const long long *mptr, long long n, long long m, con
             len[j] = 0;
         } else {
             len[j] = (int)(e - b);
+            above |= e - b > COVER_LIST_MAX;
         }
         if (j == 0 && (__ldg(&mptr[0]) != 0 || __ldg(&mptr[n]) != m)) bad = true;
     }
     if (bad) atomicOr(status, 1);
+    if (too_long && above) *too_long = 1;
 }
 
 // Copies every stored node's list to its new offset, checks it (ids in [0, K),
@@ -295,8 +305,6 @@ __device__ __forceinline__ int claim_next(int *counter, int *slot)
 
 // ------------------------------------------------------------------ scoring in node order
 
-constexpr int COVER_LIST_MAX = 1 << 20;  // longer lists are scored by k_cover_score
-
 // Length of node v's list from its head word.
 __device__ __forceinline__ int head_len(int h, const int *off, int v)
 {
@@ -311,10 +319,10 @@ __device__ __forceinline__ int head_len(int h, const int *off, int v)
 __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__ row_ptr, const int *__restrict__ col,
                                                    const int *__restrict__ off, const int *__restrict__ memb,
                                                    const int *__restrict__ head, long long n, unsigned long long *cv,
-                                                   unsigned long long *capw, unsigned long long *total, int *too_long,
-                                                   const int *status)
+                                                   unsigned long long *capw, unsigned long long *total,
+                                                   const int *too_long, const int *status)
 {
-    if (*status) return;
+    if (*status || *too_long) return;
     const int lane = threadIdx.x & 31;
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
     unsigned long long sum = 0;
@@ -333,9 +341,7 @@ __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__
                 const unsigned d = i0 + q < cnt ? __shfl_sync(0xffffffffu, deg, i0 + q) : 0u;
                 if ((unsigned)lane < d) {
                     const int v = __ldg(&col[ri + lane]);
-                    const int l = head_len(__ldg(&head[v]), off, v);
-                    if (l > COVER_LIST_MAX) *too_long = 1;
-                    s[q] = (unsigned)min(l, COVER_LIST_MAX);
+                    s[q] = (unsigned)head_len(__ldg(&head[v]), off, v);
                 }
                 more |= d > 32u;
             }
@@ -352,9 +358,7 @@ __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__
                         unsigned x = 0u;
                         if (e0 + lane < d) {
                             const int v = __ldg(&col[ri + e0 + lane]);
-                            const int l = head_len(__ldg(&head[v]), off, v);
-                            if (l > COVER_LIST_MAX) *too_long = 1;
-                            x = (unsigned)min(l, COVER_LIST_MAX);
+                            x = (unsigned)head_len(__ldg(&head[v]), off, v);
                         }
                         const unsigned t = __reduce_add_sync(0xffffffffu, x);
                         if (lane == i0 + q) mine += t;
@@ -939,10 +943,10 @@ int members_of_side(const CoverSide &c, long long n, const CoverWs &w, int num_s
 // Brings one cover to the stored order and builds its member lists (members).
 int prepare_side(const long long *mptr, const int *memb, long long m, long long n, const int *inv,
                  const CoverSide &c, const CoverWs &w, int num_sms, cudaStream_t s, int *head = nullptr,
-                 bool members = true)
+                 int *too_long = nullptr, bool members = true)
 {
     int L = 0;
-    k_cover_len<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(mptr, n, m, inv, c.len, w.status);
+    k_cover_len<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(mptr, n, m, inv, c.len, w.status, too_long);
     ++L;
     const int l1 = scan_offsets(c.len, (int)n, c.off, w.scan_tmp, w.counters + CC_SCAN, w.status, s);
     if (l1 < 0) return -1;
@@ -970,7 +974,8 @@ int launch_cover_score(const GraphDev &g, const long long *mptr, const int *memb
 {
     const long long n = g.n;
     const bool runs = w.run_entries > 0;
-    int L = prepare_side(mptr, memb, m, n, g.inv, w.a, w, num_sms, s, runs ? w.head : nullptr, !runs);
+    int L = prepare_side(mptr, memb, m, n, g.inv, w.a, w, num_sms, s, runs ? w.head : nullptr,
+                         runs ? w.counters + CC_LONG : nullptr, !runs);
     if (L < 0) return -1;
     const int *run_if = nullptr;
     if (runs) {

@@ -1,0 +1,38 @@
+"""Covers around the list length up to which they are scored in node order (16): the
+longest list just at it and just beyond, on nodes apart and on neighbours."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import check_quality, random_graph, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def qm():
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1507_05492_gb300 import qm as q
+    return q
+
+
+@pytest.mark.parametrize("longest", [15, 16, 17, 300])
+@pytest.mark.parametrize("where", ["first", "last", "every 100th", "neighbours"])
+def test_longest_list(qm, oracle_mod, longest, where):
+    n, K = 5003, 700
+    rp, col = random_graph(n, 40_000, seed=longest)
+    rng = np.random.default_rng(longest)
+    lengths = rng.integers(0, 3, n)
+    at = {"first": [0], "last": [n - 1], "every 100th": range(0, n, 100),
+          "neighbours": np.unique(np.append(col[rp[7]:rp[8]], 7))}[where]
+    lengths[list(at)] = longest
+    mptr = np.zeros(n + 1, np.int64)
+    mptr[1:] = np.cumsum(lengths)
+    memb = np.concatenate([np.sort(rng.choice(K, int(x), replace=False)) for x in lengths]).astype(np.int32)
+    o = oracle_mod.score_cover(rp, col, mptr, memb, K)
+    dev = (torch.from_numpy(mptr).cuda(), torch.from_numpy(memb).cuda())
+    for reorder in (False, True):
+        graph = qm.Graph(*to_dev(rp, col), reorder=reorder)
+        check_quality(qm.score_cover(graph, dev, K), o, f"{where} reorder={reorder}")
+        graph.close()
