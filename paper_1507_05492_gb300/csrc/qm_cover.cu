@@ -878,10 +878,17 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_pairs(CoverCmpArgs a)
         const bool in_smem = L <= OVL_CAP;
         // pairs of overlapping members (from shared memory, or the whole member
         // list filtered again when there are too many to hold)
-        // a warp per first member, its lanes over the later ones
-        const int Lp = in_smem ? L : me - mb;
-        for (int pp = tid >> 5; pp < Lp - 1; pp += T >> 5)
-        for (int qq = pp + 1 + (tid & 31); qq < Lp; qq += 32) {
+        // The pairs (p, q), p < q < Lp, as a rectangle: with Lp rounded up to an even
+        // number E, rows p and E - 1 - p hold E - 1 pairs together, so E / 2 rows of
+        // E - 1 columns hold all (those with q = Lp are none where Lp is odd).  Every
+        // thread steps through it T places at a time, without a division a pair.
+        const unsigned Lp = in_smem ? L : me - mb, E = Lp + (Lp & 1u), width = E - 1u;
+        const unsigned dr = T / width, dq = T % width;
+        unsigned row = tid / width, at = tid % width;
+        for (; row < E / 2u; row += dr, at += dq, row += at >= width ? 1u : 0u, at -= at >= width ? width : 0u) {
+            const bool upper = at >= row;
+            const unsigned pp = upper ? row : E - 1u - row, qq = upper ? at + 1u : E - row + at;
+            if (qq >= Lp) continue;
             const int i = in_smem ? ovl[pp] : __ldg(&xcmem[mb + pp]);
             const int j = in_smem ? ovl[qq] : __ldg(&xcmem[mb + qq]);
             const int li = __ldg(&xoff[i + 1]) - __ldg(&xoff[i]), lj = __ldg(&xoff[j + 1]) - __ldg(&xoff[j]);

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import check_quality, random_graph, to_dev
+from helpers import check_compare, check_quality, random_graph, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -36,3 +36,24 @@ def test_longest_list(qm, oracle_mod, longest, where):
         graph = qm.Graph(*to_dev(rp, col), reorder=reorder)
         check_quality(qm.score_cover(graph, dev, K), o, f"{where} reorder={reorder}")
         graph.close()
+
+
+# members of one community that are in others too: their pairs are enumerated as a
+# rectangle; beyond 2,048 of them the whole member list is
+@pytest.mark.parametrize("L", [1, 2, 3, 32, 33, 255, 256, 257, 1000, 2048, 2049])
+def test_pairs_of_overlapping_members(qm, oracle_mod, L):
+    n = 2600
+    rng = np.random.default_rng(L)
+
+    def side(shared):
+        lists = [[2 + int(rng.integers(0, 40))] for _ in range(n)]
+        for u in rng.choice(n, shared, replace=False):  # in community 0 and its own, some in 1 too
+            lists[u] = [0] + ([1] if rng.random() < 0.5 else []) + lists[u]
+        mptr = np.zeros(n + 1, np.int64)
+        mptr[1:] = np.cumsum([len(x) for x in lists])
+        return mptr, np.concatenate(lists).astype(np.int32)
+
+    a, b = side(L), side(max(1, L // 2))
+    o = oracle_mod.compare_cover(a[0], a[1], 42, b[0], b[1], 42)
+    dev = [tuple(torch.from_numpy(x).cuda() for x in s) for s in (a, b)]
+    check_compare(qm.compare_covers(dev[0], 42, dev[1], 42, n), o, f"L={L}")
