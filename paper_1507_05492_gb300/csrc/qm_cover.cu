@@ -56,7 +56,7 @@ constexpr int OVL_CAP = 2048;  // overlapping members of one community paired in
 // extra accumulator words after the GC_* words of a comparison
 enum { GC_SAME_A_CORR = GC_COUNT, GC_SAME_B_CORR = GC_COUNT + 1, GC_A11_CORR = GC_COUNT + 2, GC_WORDS = GC_COUNT + 3 };
 enum { CC_NEXT_A = 0, CC_NEXT_B = 1, CC_NEXT_C = 2, CC_GATE = 3, CC_OLD = 4, CC_LONG = 5, CC_TOTAL = 6 /* two words */,
-       CC_SCAN = 8, CC_RUNS = 16 };
+       CC_SCAN = 8, CC_RUNS = 16, CC_HUBS = 32 };
 
 size_t al(size_t x) { return (x + 255) / 256 * 256; }
 
@@ -124,6 +124,8 @@ CoverWs carve_cover_score_ws(void *base, long long n, long long m, int K, long l
     if (run_entries) {
         w.head = (int *)p;
         p += al((size_t)n * 4);
+        w.hubs = (int *)p;
+        p += al((size_t)(run_entries / COVER_HUB + 1) * 4);  // (run_entries exceeds the arcs)
         w.base = (unsigned *)p;
         p += al((size_t)K * 4);
         w.inter = (int *)p;
@@ -213,9 +215,11 @@ __global__ void k_cover_len(const long long *mptr, long long n, long long m, con
 // Copies every stored node's list to its new offset, checks it (ids in [0, K),
 // strictly increasing) and counts the community sizes.
 // head[j] (when wanted): the id of a list of one, -1 for an empty list, else the
-// list's offset with the sign bit set.
+// list's offset with the sign bit set; and the nodes of more than COVER_HUB arcs
+// are listed in hubs.
 __global__ void k_cover_copy(const long long *mptr, const int *memb, long long n, const int *inv, int K,
-                             const int *off, int *out, int *size, int *status, int *head)
+                             const int *off, int *out, int *size, int *status, int *head,
+                             const long long *__restrict__ row_ptr, int *hubs, int *nhubs)
 {
     if (*(volatile int *)status) return;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -235,7 +239,10 @@ __global__ void k_cover_copy(const long long *mptr, const int *memb, long long n
             out[o + k] = c;
             atomicAdd(&size[c], 1);
         }
-        if (head) head[j] = len == 1 ? prev : len == 0 ? -1 : (int)(0x80000000u | (unsigned)o);
+        if (head) {
+            head[j] = len == 1 ? prev : len == 0 ? -1 : (int)(0x80000000u | (unsigned)o);
+            if (__ldg(&row_ptr[j + 1]) - __ldg(&row_ptr[j]) > COVER_HUB) hubs[atomicAdd(nhubs, 1)] = (int)j;
+        }
     }
     if (bad) atomicOr(status, 1);
 }
@@ -312,14 +319,18 @@ __device__ __forceinline__ int head_len(int h, const int *off, int v)
     return h == -1 ? 0 : __ldg(&off[v + 1]) - (h & 0x7FFFFFFF);
 }
 
+// Pieces of the rows of hubs (see COVER_HUB), which all warps take in turn.
+constexpr unsigned HUB_PIECE = 2048;
+
 // Members and arcs (cv) of every community, and members and segment size
 // (capw): for each of its members the list lengths of the neighbours, summed.
-// A warp takes 32 nodes, a lane per arc of one node at a time.  The segments'
-// total goes to *total.
+// A warp takes 32 nodes, a lane per arc of one node at a time, then the hubs'
+// rows in pieces.  The segments' total goes to *total.
 __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__ row_ptr, const int *__restrict__ col,
                                                    const int *__restrict__ off, const int *__restrict__ memb,
                                                    const int *__restrict__ head, long long n, unsigned long long *cv,
                                                    unsigned long long *capw, unsigned long long *total,
+                                                   const int *__restrict__ hubs, const int *nhubs,
                                                    const int *too_long, const int *status)
 {
     if (*status || *too_long) return;
@@ -338,7 +349,8 @@ __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const long long ri = __shfl_sync(0xffffffffu, r, i0 + q);
-                const unsigned d = i0 + q < cnt ? __shfl_sync(0xffffffffu, deg, i0 + q) : 0u;
+                unsigned d = i0 + q < cnt ? __shfl_sync(0xffffffffu, deg, i0 + q) : 0u;
+                if (d > (unsigned)COVER_HUB) d = 0u;
                 if ((unsigned)lane < d) {
                     const int v = __ldg(&col[ri + lane]);
                     s[q] = (unsigned)head_len(__ldg(&head[v]), off, v);
@@ -354,7 +366,7 @@ __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__
                 for (int q = 0; q < 4 && i0 + q < cnt; ++q) {
                     const long long ri = __shfl_sync(0xffffffffu, r, i0 + q);
                     const unsigned d = __shfl_sync(0xffffffffu, deg, i0 + q);
-                    for (unsigned e0 = 32u; e0 < d; e0 += 32u) {
+                    for (unsigned e0 = 32u; e0 < d && d <= (unsigned)COVER_HUB; e0 += 32u) {
                         unsigned x = 0u;
                         if (e0 + lane < d) {
                             const int v = __ldg(&col[ri + e0 + lane]);
@@ -373,6 +385,22 @@ __global__ void __launch_bounds__(256) k_cover_cap(const long long *__restrict__
                 atomicAdd(&capw[c], (1ull << VOL_BITS) | mine);  // (a sum beyond 33 bits is beyond the scratch too)
             }
             sum += mine * (unsigned long long)(e - b);
+        }
+    }
+    const long long wg = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for (int i = 0; i < *nhubs; ++i) {
+        const int u = __ldg(&hubs[i]), b = __ldg(&off[u]), len = __ldg(&off[u + 1]) - b;
+        const long long r = __ldg(&row_ptr[u]), end = __ldg(&row_ptr[u + 1]);
+        for (long long e0 = r + (wg + i) % nw * HUB_PIECE; e0 < end; e0 += nw * HUB_PIECE) {
+            unsigned x = 0u;
+#pragma unroll 4
+            for (unsigned e = lane; e < HUB_PIECE; e += 32u) {
+                const int v = e0 + e < end ? __ldg(&col[e0 + e]) : -1;
+                if (v >= 0) x += (unsigned)head_len(__ldg(&head[v]), off, v);
+            }
+            const unsigned long long t = __reduce_add_sync(0xffffffffu, x);
+            for (int k = lane; k < len; k += 32) atomicAdd(&capw[__ldg(&memb[b + k])], t);
+            if (lane == 0) sum += t * (unsigned long long)len;
         }
     }
     sum = warp_sum_u64(sum);
@@ -396,6 +424,7 @@ struct CoverWalkArgs {
     const unsigned *base;
     unsigned long long *curs;  // cut arcs << 32 | packed entries of each community
     int *nbr;
+    const int *hubs, *nhubs;
     const int *gate;
 };
 
@@ -486,9 +515,31 @@ __global__ void __launch_bounds__(CW_THREADS) k_cover_walk(CoverWalkArgs a)
         } else {
             for (int i = 0; i < nm; ++i) {
                 const unsigned b = __shfl_sync(0xffffffffu, rel, i), z = __shfl_sync(0xffffffffu, end, i);
+                if (z - b > (unsigned)COVER_HUB) continue;  // below, in pieces
                 cover_arcs(a, a.col + r0 + b, z - b, aoff_s[w], [i](unsigned) { return i; }, lane);
             }
         }
+        __syncwarp();
+    }
+}
+
+// The same for the hubs' rows, in pieces (apart from k_cover_walk, whose
+// registers a second walk would raise).
+__global__ void __launch_bounds__(CW_THREADS) k_cover_walk_hubs(CoverWalkArgs a)
+{
+    __shared__ int aoff_s[CW_THREADS / 32][2];
+    if (*a.gate) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, n = *a.nhubs;
+    const long long nwarps = (long long)gridDim.x * (CW_THREADS / 32);
+    const long long wg = (long long)blockIdx.x * (CW_THREADS / 32) + w;
+    for (int i = 0; i < n; ++i) {
+        const int u = __ldg(&a.hubs[i]);
+        const long long r = __ldg(&a.row_ptr[u]), end = __ldg(&a.row_ptr[u + 1]);
+        if (lane < 2) aoff_s[w][lane] = __ldg(&a.off[u + lane]);
+        __syncwarp();
+        for (long long e0 = r + (wg + i) % nwarps * HUB_PIECE; e0 < end; e0 += nwarps * HUB_PIECE)
+            cover_arcs(a, a.col + e0, (unsigned)min((long long)HUB_PIECE, end - e0), aoff_s[w],
+                       [](unsigned) { return 0; }, lane);
         __syncwarp();
     }
 }
@@ -950,7 +1001,7 @@ int members_of_side(const CoverSide &c, long long n, const CoverWs &w, int num_s
 // Brings one cover to the stored order and builds its member lists (members).
 int prepare_side(const long long *mptr, const int *memb, long long m, long long n, const int *inv,
                  const CoverSide &c, const CoverWs &w, int num_sms, cudaStream_t s, int *head = nullptr,
-                 int *too_long = nullptr, bool members = true)
+                 int *too_long = nullptr, const long long *row_ptr = nullptr, bool members = true)
 {
     int L = 0;
     k_cover_len<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(mptr, n, m, inv, c.len, w.status, too_long);
@@ -959,7 +1010,7 @@ int prepare_side(const long long *mptr, const int *memb, long long m, long long 
     if (l1 < 0) return -1;
     L += l1;
     k_cover_copy<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(mptr, memb, n, inv, c.K, c.off, c.memb, c.size,
-                                                            w.status, head);
+                                                            w.status, head, row_ptr, w.hubs, w.counters + CC_HUBS);
     ++L;
     if (!members) return L;
     const int l2 = members_of_side(c, n, w, num_sms, s, nullptr);
@@ -982,14 +1033,15 @@ int launch_cover_score(const GraphDev &g, const long long *mptr, const int *memb
     const long long n = g.n;
     const bool runs = w.run_entries > 0;
     int L = prepare_side(mptr, memb, m, n, g.inv, w.a, w, num_sms, s, runs ? w.head : nullptr,
-                         runs ? w.counters + CC_LONG : nullptr, !runs);
+                         runs ? w.counters + CC_LONG : nullptr, g.row_ptr, !runs);
     if (L < 0) return -1;
     const int *run_if = nullptr;
     if (runs) {
         int *const gate = w.counters + CC_GATE, *const old_path = w.counters + CC_OLD;
         unsigned long long *const total = (unsigned long long *)(w.counters + CC_TOTAL);
         k_cover_cap<<<grid_of(n, 256, num_sms, 8), 256, 0, s>>>(g.row_ptr, g.col, w.a.off, w.a.memb, w.head, n, w.cv, w.capw,
-                                                               total, w.counters + CC_LONG, w.status);
+                                                               total, w.hubs, w.counters + CC_HUBS,
+                                                               w.counters + CC_LONG, w.status);
         k_cover_gate<<<1, 1, 0, s>>>(w.status, total, w.run_entries, w.counters + CC_LONG, gate, old_path);
         L += 2 + launch_segment_bases(w.capw, K, w.base, w.recip, (unsigned *)w.scan_tmp, gate, s);
         CoverWalkArgs a;
@@ -1002,8 +1054,11 @@ int launch_cover_score(const GraphDev &g, const long long *mptr, const int *memb
         a.base = w.base;
         a.curs = w.curs;
         a.nbr = w.nbr;
+        a.hubs = w.hubs;
+        a.nhubs = w.counters + CC_HUBS;
         a.gate = gate;
         k_cover_walk<<<grid_of(n, CW_THREADS, num_sms, 5), CW_THREADS, 0, s>>>(a);
+        k_cover_walk_hubs<<<5 * num_sms, CW_THREADS, 0, s>>>(a);
         CoverRuns r;
         r.cv = w.cv;
         r.curs = w.curs;
@@ -1018,7 +1073,7 @@ int launch_cover_score(const GraphDev &g, const long long *mptr, const int *memb
         r.err = w.status;
         const int lr = launch_cover_runs(r, K, g.n_arcs / 2, w.gacc, num_sms, s);
         if (lr < 0) return -1;
-        L += 1 + lr;
+        L += 2 + lr;
         run_if = old_path;  // the kernels below work only when the runs did not fit
         const int lm = members_of_side(w.a, n, w, num_sms, s, run_if);
         if (lm < 0) return -1;

@@ -25,6 +25,11 @@ struct CoverSide {
     int K;
 };
 
+// Rows of more arcs than this are taken in pieces by all warps of a pass over the
+// rows, not by the warp that meets them: a star of 10^6 leaves in a thousand
+// communities, the call 41 ms by that warp, 0.81 so (29.7 by member lists).
+constexpr int COVER_HUB = 8192;
+
 struct CoverWs {
     int *status;               // bit 0: a malformed list or an id out of range; bit 1: too many distinct keys
     int *counters;             // claim counters and scan counters (zeroed)
@@ -40,6 +45,7 @@ struct CoverWs {
     unsigned long long *cv, *capw;  // [K] members << 33 | arcs, members << 33 | segment size (zeroed)
     unsigned long long *curs;  // [K] cut arcs << 32 | packed entries (zeroed)
     int *head;                 // [n] each node's list: its id, -1, or its offset with the sign bit
+    int *hubs;                 // nodes of more than COVER_HUB arcs (at most run_entries / COVER_HUB)
     unsigned *base;            // [K] segment bases
     int *inter;                // [K] cut arcs
     unsigned long long *rec;   // [K][8] count records

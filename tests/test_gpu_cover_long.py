@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import check_compare, check_quality, random_graph, to_dev
+from helpers import check_compare, check_quality, csr_from_edges, random_graph, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +57,24 @@ def test_pairs_of_overlapping_members(qm, oracle_mod, L):
     o = oracle_mod.compare_cover(a[0], a[1], 42, b[0], b[1], 42)
     dev = [tuple(torch.from_numpy(x).cuda() for x in s) for s in (a, b)]
     check_compare(qm.compare_covers(dev[0], 42, dev[1], 42, n), o, f"L={L}")
+
+
+@pytest.mark.parametrize("m", [8191, 8192, 8193, 60_000])  # 8,192 arcs: the longest row a warp walks alone
+def test_hub_rows(qm, oracle_mod, m):
+    rng = np.random.default_rng(m)
+    n = m + 3
+    edges = [np.stack([np.full(m, h), rng.permutation(n)[:m]], 1) for h in (0, n // 2, n - 1)]
+    # hubs of m arcs or a few more (the other hubs'), and some other edges
+    rp, col = csr_from_edges(n, np.concatenate(edges + [rng.integers(0, n, (2 * n, 2))]))
+    K = 300
+    lengths = rng.integers(0, 3, n)
+    lengths[[0, n // 2]] = [5, 0]
+    mptr = np.zeros(n + 1, np.int64)
+    mptr[1:] = np.cumsum(lengths)
+    memb = np.concatenate([np.sort(rng.choice(K, int(x), replace=False)) for x in lengths]).astype(np.int32)
+    o = oracle_mod.score_cover(rp, col, mptr, memb, K)
+    dev = (torch.from_numpy(mptr).cuda(), torch.from_numpy(memb).cuda())
+    for reorder in (False, True):
+        graph = qm.Graph(*to_dev(rp, col), reorder=reorder)
+        check_quality(qm.score_cover(graph, dev, K), o, f"m={m} reorder={reorder}")
+        graph.close()
