@@ -37,16 +37,16 @@ __global__ void k_lpa_init(int *lab, long long n)
 // its own label when that is among the most frequent, and otherwise takes the
 // smallest of the tied labels.
 //
-// A warp takes 32 consecutive nodes.  First their samples one after another in
+// A warp takes 32 consecutive nodes (fewer where those would not occupy the GPU,
+// see lpa_shape).  First their samples one after another in
 // slots, 32 slots a step whatever the degrees are (a bit per node's first slot
 // and a popcount give a lane the node of its slot): a vote a step tells which
 // labels equal the own one, and each node's lane then counts its bits.  A node
 // with its own label in at least half of the sample keeps it (nothing can be more
-// frequent).  The others are gathered LPA_NODES at a time, a lane per neighbour:
-// the first neighbour's label wins if more than half of the sample carries it;
-// else the lanes match and reduce (redux) the counts, then the smallest label
-// among the largest.  In the first rounds hardly a node keeps its label, so
-// those (`all`) skip the first part.
+// frequent).  The others are gathered LPA_NODES at a time, a lane per neighbour: the
+// lanes match their labels and reduce (redux) the largest count, the own label
+// counting half more, then the smallest label of that count.  In the first rounds
+// hardly a node keeps its label, so those (`all`) skip the first part.
 // Bound in the first rounds by the pipe of votes, matches and redux (80 % busy;
 // DRAM 7 %), later by the gathers' latency.  Measured at 10^7 nodes (renumbered,
 // mean degree 19, ten rounds), ms a call: a warp per node and a 64-bit shuffle
@@ -63,6 +63,7 @@ struct LpaNode {
     unsigned d, off;
 };
 
+template <int NODES>
 __global__ void __launch_bounds__(256, LPA_BLOCKS) k_lpa_round(const long long *__restrict__ row_ptr, const int *__restrict__ col,
                                                    long long n, const int *__restrict__ cur, int *__restrict__ nxt,
                                                    int all)
@@ -75,8 +76,8 @@ __global__ void __launch_bounds__(256, LPA_BLOCKS) k_lpa_round(const long long *
     int *const nown = s_own[wid];
     unsigned *const first_bits = s_first[wid], *const eq_bits = s_eq[wid];
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long u0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; u0 < n; u0 += nw * 32) {
-        const long long u = u0 + lane;
+    for (long long u0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * NODES; u0 < n; u0 += nw * NODES) {
+        const long long u = NODES == 32 || lane < NODES ? u0 + lane : n;
         const long long rs = __ldg(&row_ptr[min(u, n)]);
         const unsigned deg = (unsigned)(__ldg(&row_ptr[min(u + 1, n)]) - rs);  // 0 past the last node
         const int own = u < n ? __ldg(&cur[u]) : -1;
@@ -275,6 +276,36 @@ static int grid_of(long long work, int threads, int num_sms, int per_sm)
     return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
+// Nodes a warp of k_lpa_round takes, and its blocks.  Small graphs spread over the
+// GPU: down to four nodes a warp where there are not four times as many
+// warps as are resident.  Their labels are in L2 and the slots cost more than the
+// matches they save, so all their rounds go without.  Ten rounds at 10^4, 10^5 and
+// 6*10^5 nodes, mixing 0.5, us a call: a warp per node 126, 270, 1024; 32 nodes a
+// warp with slots 211, 297, 997; so 127, 252, 870 (0.1: 129, 242, 899; 164, 210,
+// 627; 126, 205, 627).  From 9*10^5 nodes on 32 (10^6 nodes, 0.1 and 0.5: a warp per
+// node 1408 and 1619, 32 with slots 929 and 1538).
+struct LpaShape {
+    int nodes, grid;
+    bool all(int round) const { return round < LPA_ALL_ROUNDS || nodes < 32; }
+};
+
+static LpaShape lpa_shape(long long n, int num_sms)
+{
+    LpaShape s{32, 0};
+    while (s.nodes > 4 && n < 4LL * s.nodes * num_sms * LPA_BLOCKS * 8) s.nodes /= 2;
+    s.grid = grid_of((n + s.nodes - 1) / s.nodes * 32, 256, num_sms, LPA_BLOCKS);
+    return s;
+}
+
+static void launch_lpa_round(const GraphDev &g, const int *cur, int *nxt, int round, const LpaShape &s, cudaStream_t st)
+{
+    auto run = [&](auto kern) { kern<<<s.grid, 256, 0, st>>>(g.row_ptr, g.col, g.n, cur, nxt, s.all(round)); };
+    if (s.nodes == 32) run(k_lpa_round<32>);
+    else if (s.nodes == 16) run(k_lpa_round<16>);
+    else if (s.nodes == 8) run(k_lpa_round<8>);
+    else run(k_lpa_round<4>);
+}
+
 int launch_permute_labels(const int *labels, const int *inv, long long n, int P, int *out, int num_sms,
                           cudaStream_t s)
 {
@@ -286,12 +317,13 @@ int launch_label_propagation(const GraphDev &g, int rounds, int num_sms, cudaStr
                              int *hist, int *tmp, size_t tmp_elems, int *out)
 {
     const long long n = g.n;
-    const int g1 = grid_of(n, 512, num_sms, 8), gl = grid_of(n, 256, num_sms, LPA_BLOCKS);
+    const int g1 = grid_of(n, 512, num_sms, 8);
+    const LpaShape ls = lpa_shape(n, num_sms);
     int L = 0;
     k_lpa_init_ids<<<g1, 512, 0, s>>>(lab0, g.inv, n);
     ++L;
     for (int r = 0; r < rounds; ++r) {
-        k_lpa_round<<<gl, 256, 0, s>>>(g.row_ptr, g.col, n, lab0, lab1, r < LPA_ALL_ROUNDS);
+        launch_lpa_round(g, lab0, lab1, r, ls, s);
         std::swap(lab0, lab1);
         ++L;
     }
@@ -338,12 +370,12 @@ int reorder_graph(const GraphDev &g, int rounds, int num_sms, cudaStream_t s, lo
     if ((e = cudaMalloc(&perm, (size_t)n * 4)) != cudaSuccess) return -bad(e);
     if ((e = cudaMalloc(&inv, (size_t)n * 4)) != cudaSuccess) return -bad(e);
     if ((e = cudaMalloc(&tmp, tmp_elems * 4)) != cudaSuccess) return -bad(e);
-    const int g1 = grid_of(n, 512, num_sms, 8), gw = grid_of(n * 32, 256, num_sms, 8),
-              gl = grid_of(n, 256, num_sms, LPA_BLOCKS);
+    const int g1 = grid_of(n, 512, num_sms, 8), gw = grid_of(n * 32, 256, num_sms, 8);
+    const LpaShape ls = lpa_shape(n, num_sms);
     k_lpa_init<<<g1, 512, 0, s>>>(lab0, n);
     ++L;
     for (int r = 0; r < rounds; ++r) {
-        k_lpa_round<<<gl, 256, 0, s>>>(g.row_ptr, g.col, n, lab0, lab1, r < LPA_ALL_ROUNDS);
+        launch_lpa_round(g, lab0, lab1, r, ls, s);
         std::swap(lab0, lab1);
         ++L;
     }
