@@ -2270,7 +2270,10 @@ int launch_weight_check(const GraphDev &g, const float *wt, int full, int *statu
 
 bool compare_small_ok(long long n, int ka, int kb)
 {
-    return n <= CS_MAX_NODES && ka <= CS_MAX_K && kb <= CS_MAX_K && bits_of(ka) + bits_of(kb) <= 31;
+    // cells, rows and columns of a node or two each are mostly FP64 work, which the
+    // whole GPU does sooner than eight SMs from about 10^4 nodes on
+    const bool fine = n > CS_FINE_NODES && 8LL * std::min(ka, kb) >= 3 * n;
+    return n <= CS_MAX_NODES && !fine && ka <= CS_MAX_K && kb <= CS_MAX_K && bits_of(ka) + bits_of(kb) <= 31;
 }
 
 int launch_compare_small(const int *truth, const int *found, long long n, int ka, int kb, const CompareWs &ws,

@@ -18,6 +18,11 @@ constexpr int CS_CTAS = 8, CS_THREADS = 512;
 constexpr int CS_MAX_SLOTS = 21504;  // 10 bytes each: a block may come to hold every cell
 constexpr int CS_MAX_NODES = CS_MAX_SLOTS * 3 / 4;
 constexpr int CS_MAX_K = 1 << 16;
+// Beyond this many nodes two labellings that both have communities of fewer than
+// 8/3 nodes on average go the other path.  Communities of two on both sides, this
+// path and the other, us: 10^4 nodes 103 and 108, 12,000 114 and 109, 16,128 141 and
+// 120 (of three, 16,128 nodes: 91 and 108; of two against 30 79 and 114).
+constexpr int CS_FINE_NODES = 10000;
 
 struct CompareSmallArgs {
     const int *truth, *found;
