@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
     __shared__ unsigned colmax[CELL_MAX_RANGE];
     __shared__ unsigned long long red[72];
     __shared__ unsigned late_s[CELL_TAB_THREADS / 32][32 * 5];
-    __shared__ int s_b, s_used, s_at, s_over;
+    __shared__ int s_b, s_used, s_done, s_at, s_over;
     if (block_stopped(a.status)) return;
     unsigned *const key = sm_tab, *const cnt = sm_tab + CELL_SLOTS;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
             nbs[i] = 0;
             colmax[i] = 0u;
         }
-        if (tid == 0) s_used = s_over = 0;
+        if (tid == 0) s_used = s_done = s_over = 0;
         block_sync();
         const int bk = s_b;
         if (bk >= a.nb) break;
@@ -247,7 +247,14 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                     k[q] = i < p1 ? __ldcs(&a.pairs[i]) + 1u : 0u;
                     if (R > 1 && tab_split(k[q], R) != r) k[q] = 0u;
                 }
-                if (*(volatile int *)&s_used > CELL_FILL) *(volatile int *)&s_over = 1;
+                // more keys than the table takes; or, once it is half as full, so many per entry
+                // that the rest would bring them (found at the end, a nearly full table of long
+                // probes would have been filled for nothing: 10^8 nodes, two labellings at
+                // random, this kernel 7.7 and 3.0 ms; 10^7 nodes 1.04 and 0.42)
+                const int have = *(volatile int *)&s_used, read = *(volatile int *)&s_done;
+                if (have > CELL_FILL ||
+                    (have > CELL_FILL / 2 && (long long)have * (p1 - p0) > (long long)CELL_FILL * read))
+                    *(volatile int *)&s_over = 1;
                 if (__any_sync(0xffffffffu, *(volatile int *)&s_over)) break;  // this class does not fit: stop reading it
                 // first slots of all four: own key or free; the others are followed 32 at a time
                 unsigned fresh = 0;
@@ -270,7 +277,10 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                 }
                 __syncwarp();
                 while (nl >= 32u) fresh += follow(32u);
-                if (lane == 0 && fresh) atomicAdd(&s_used, (int)fresh);
+                if (lane == 0) {
+                    atomicAdd(&s_done, 128);
+                    if (fresh) atomicAdd(&s_used, (int)fresh);
+                }
             }
             {
                 // (other warps may be setting the flag: one answer for the warp, which follow() needs whole)
@@ -327,7 +337,7 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                 R = 2u * top;
             }
             block_sync();
-            if (tid == 0) s_used = s_over = 0;
+            if (tid == 0) s_used = s_done = s_over = 0;
             block_sync();
         }
         block_sync();
