@@ -423,7 +423,7 @@ qm_status qm_debug_set_perm_buckets(int32_t window_bits, int32_t tile_bits, int6
  *      id, appended to that run's segment from wherever it is found.  Half the
  *      far-end gathers, at the price of scattered appends: faster on graphs in
  *      a random node order whose label array exceeds L2 (the default for
- *      untuned graphs loaded without QM_REORDER above 13 * 2^22 nodes), slower on
+ *      untuned graphs loaded without QM_REORDER above 11 * 2^22 nodes), slower on
  *      reordered or smaller graphs.  Sharded calls run 1 instead.
  * Packing needs K <= 2^21; with more label ids the 32-bit labels are gathered.
  * All give bit-identical results.  Weighted graphs take algorithm 1 whatever

@@ -51,10 +51,14 @@ constexpr int ALGO_SORT = 6;
 constexpr int ALGO_HALF = 7;
 // Untuned calls take ALGO_HALF on graphs in their given node order with more
 // nodes than this: about where the packed labels (8/3 bytes a node) outgrow L2
-// and the gathers go to DRAM.  Both ends gathered against half-edge, ms a call in
-// random node order, mean degree 19: 3*10^7 nodes 5.40 and 6.87, 4.4*10^7 9.93 and
-// 10.55, 5.1*10^7 12.19 and 12.42, 6*10^7 16.90 and 15.11, 10^8 39.1 and 27.4.
-constexpr long long HALF_MIN_NODES = 13LL << 22;
+// and the gathers go to DRAM.  Both ends gathered by members, both ends by rows and
+// half-edge, ms a call in random node order, mean degree 19: mixing 0.05 at 4*10^7
+// nodes 7.2, 7.1, 7.4, at 4.8*10^7 9.0, 9.4, 8.9, at 5.2*10^7 10.1, 10.5, 9.8;
+// mixing 0.3 9.7, 8.6, 9.5, then 12.6, 11.2, 11.7, then 14.0, 12.6, 12.8, and at
+// 6*10^7 17.0, 15.9, 14.9 (10^8, rows and half-edge: 39.1, 27.4).  The line lies where
+// no mixing loses against the members, not where half-edge gains at 0.3; nodes given
+// cluster by cluster lose a gain there (4.8*10^7: 6.9, 5.1, 6.9).
+constexpr long long HALF_MIN_NODES = 11LL << 22;
 
 // Carving of the dynamic shared memory of a community-major block.
 struct SmemPlan {
