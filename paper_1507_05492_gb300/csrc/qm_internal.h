@@ -160,6 +160,11 @@ inline int bin_mode_of(int algo, bool weighted) { return (!weighted && (algo == 
 // Graphs with more nodes than this gather packed labels by default (algorithm
 // 1): their label array is well beyond what L2 keeps.
 constexpr long long PACK_MIN_NODES = 1LL << 22;
+// Weighted graphs in their given node order: 3*10^7 nodes, mixing 0.02, 0.1 and 0.5,
+// ms a call with the 32-bit labels 7.29, 9.69, 15.1, packed 6.47, 8.72, 14.2 (by
+// members 6.78, 8.13, 23.9); 2*10^7 nodes, 0.02 and 0.1, 4.16 and 5.51, 3.75 and 5.20;
+// equal at 10^7.  Renumbered ones gather near their own row: 2.38 and 2.71 at 0.02.
+constexpr long long PACK_MIN_WEIGHTED = 1LL << 24;
 // Renumbered graphs of more nodes than this gather from the block encoding of
 // the labels (qm_expand.cuh) instead of the packed copy (tuning algorithm 4:
 // at any size): below it the packed copy mostly stays in L2 already and the
@@ -168,11 +173,12 @@ constexpr long long BLOCKS_MIN_NODES = 1LL << 26;
 inline bool label_blocks(int algo, long long n) { return algo == 4 || n > BLOCKS_MIN_NODES; }
 
 // Whether a two-phase call gathers from the packed copy: algorithm 4 always,
-// algorithms 1, ALGO_SORT and ALGO_HALF on graphs above PACK_MIN_NODES;
-// unweighted graphs and label ids below 2^21 only.
-inline bool packs_labels(int algo, bool weighted, long long n, int K)
+// algorithms 1, ALGO_SORT and ALGO_HALF on graphs above PACK_MIN_NODES, weighted
+// graphs above PACK_MIN_WEIGHTED that are not renumbered; label ids below 2^21 only.
+inline bool packs_labels(int algo, bool weighted, bool renumbered, long long n, int K)
 {
-    return !weighted && K <= (1 << 21) &&
+    if (weighted) return algo == 1 && !renumbered && K <= (1 << 21) && n > PACK_MIN_WEIGHTED;
+    return K <= (1 << 21) &&
            (algo == 4 || ((algo == 1 || algo == ALGO_SORT || algo == ALGO_HALF) && n > PACK_MIN_NODES));
 }
 // The autotuner tries the binned gathers on graphs with more nodes than this:

@@ -1723,7 +1723,7 @@ ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool w
 {
     ScoreWs w{};
     if (weighted) bin_mode = 0;
-    if (weighted || bin_mode || K > PACK_MAX_K) pack = false;
+    if (bin_mode || K > PACK_MAX_K) pack = false;
     const int tiles = scan_tiles((int)std::max<long long>(n, K));
     char *p = (char *)base;
     w.status = (int *)p;
@@ -1977,8 +1977,14 @@ static int launch_phase_rows(const GraphDev &g, const int *labels, int K, const 
     a.wl = ws.wl;
     a.K = K;
     if (g.wt) {
+        if (ws.plab) {
+            TRACE("k_pack3");
+            k_pack3<<<grid_for((n + 2) / 3, 256, num_sms, 8), 256, 0, s>>>(labels, n, ws.plab, ws.status, nullptr);
+            ++launches;
+        }
         TRACE("k_rows");
-        launch_rows<true, LAB_PLAIN, false>(a, num_sms, s);
+        if (ws.plab) launch_rows<true, LAB_PACK3, false>(a, num_sms, s);
+        else launch_rows<true, LAB_PLAIN, false>(a, num_sms, s);
         return launches + 1;
     }
     // on a renumbered graph above BLOCKS_MIN_NODES nodes (any size with

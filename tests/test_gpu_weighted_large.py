@@ -80,3 +80,34 @@ def test_heavy_hub(qm):
     # (m - 1) / m, (2 m - 1) / (2 m) and its square are rounded once each
     assert abs(q["modularity"] - float(Q)) <= 1e-12 * 2
     graph.close()
+
+
+# 2^24 nodes: the most whose labels a weighted call gathers as given; 2^21 ids: the
+# most that are packed beyond that
+@pytest.mark.parametrize("n", [1 << 24, (1 << 24) + 1, 17_500_000])
+@pytest.mark.parametrize("K", [200_000, (1 << 21) + 1])
+def test_ring_of_blocks(qm, n, K):
+    """A ring (u to u +- 1) with blocks of consecutive nodes as communities, ids in
+    a scattered order: every W_c^in and W_c^out is a sum of few weights."""
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    u = torch.arange(n, dtype=torch.int64, device="cuda")
+    edge = torch.rand(n, generator=gen, device="cuda") * 4.95 + 0.05  # edge[u]: weight of (u, u + 1)
+    block = u * min(K, 150_000) // n
+    labels = (block * 7919 % K).to(torch.int32)
+    col = torch.stack([(u - 1) % n, (u + 1) % n], 1).int()
+    wt = torch.stack([edge.roll(1), edge], 1)
+    for row in (0, n - 1):
+        col[row], wt[row] = col[row].flip(0), wt[row].flip(0)
+    graph = qm.Graph(torch.arange(n + 1, dtype=torch.int64, device="cuda") * 2, col.view(-1), weights=wt.view(-1))
+    v = (edge.double() * 2.0 ** 43).long()  # at most 118 edges a block: sums below 2^53
+    last = block != block.roll(-1)          # edges between blocks
+    B = int(block[-1]) + 1
+    w_in = torch.zeros(B, dtype=torch.int64, device="cuda").index_add_(0, block[~last], v[~last])
+    w_out = torch.zeros(B, dtype=torch.int64, device="cuda")
+    w_out.index_add_(0, block[last], v[last]).index_add_(0, block.roll(-1)[last], v[last])
+    W = fixed_sum(edge)
+    fin, vol = w_in.double() / float(W), (2 * w_in + w_out).double() / float(2 * W)
+    q = qm.score(graph, labels, K)
+    assert abs(q["modularity"] - float((fin - vol * vol).sum())) <= 1e-12 * 2
+    assert q["cut_edges_total"] == int(last.sum())
+    graph.close()
