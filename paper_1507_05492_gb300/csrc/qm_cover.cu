@@ -80,9 +80,14 @@ void carve_side(char *&p, CoverSide &c, long long n, long long m, int K)
 // Entries of the packed runs' scratch: what covers whose memberships do not
 // follow the degrees need (every arc once per pair of its ends' communities),
 // and a quarter more.
+// Small calls keep the member lists: the runs take nine launches more, and pay from
+// about 2^20 arcs on, or where a community's arcs are many for its one block (us a
+// call, lists and runs: 20,000 nodes 0.38*10^6 arcs 197-231 and 243-262, 40,000
+// nodes 244-275 and 248-271, 10^5 nodes 270-345 and 272-288; few communities, 5,000
+// nodes, 19,000 arcs each 379-931 and 218-372, 9,500 each 379-458 and 208-231).
 long long cover_run_entries(long long n, long long n_arcs, long long m, int K)
 {
-    if (!cover_runs_ok(K)) return 0;
+    if (!cover_runs_ok(K) || (n_arcs < (1LL << 20) && n_arcs < (1LL << 12) * K)) return 0;
     const double r = std::max(1.0, (double)m / (double)n);
     const double e = 1.25 * (double)n_arcs * r * r + 4096.0;
     return e < 4.0e9 ? (long long)e : 0;
