@@ -767,7 +767,8 @@ qm_status qm_workspace_bytes(const qm_graph *g, int32_t K, int32_t with_compare,
     if (!g || !bytes || K < 1 || (with_compare && k_truth < 1)) return fail(QM_EINVAL, "bad argument");
     const bool wt = g->wt != nullptr;
     size_t b = std::max(score_ws_bytes(g->n, K),
-                        score2_ws_bytes(g->n, g->n_arcs, K, wt, 0, packs_labels(1, wt, g->inv != nullptr, g->n, K))) +
+                        score2_ws_bytes(g->n, g->n_arcs, K, wt, 0, packs_labels(1, wt, g->inv != nullptr, g->n, K),
+                                        !wt)) +
                al256((size_t)g->n * 4);
     if (g->inv) b += al256((size_t)g->n * 4);
     if (g->pb.lpos) b += al256((size_t)g->n * 4);
@@ -796,8 +797,9 @@ static qm_status score_impl(qm_graph *g, const int32_t *labels, int32_t K, qm_me
     const bool weighted = g->wt != nullptr;
     const bool graphed = !pc && !t_trace.on && n <= kPlainGraphMaxN;
     const int bmode = bin_mode_of(sh.algo, weighted);
+    const bool half = sh.algo == ALGO_HALF && !weighted;
     const bool pack = packs_labels(sh.algo, weighted, g->inv != nullptr, n, K);
-    size_t need = sh.algo ? score2_ws_bytes(n, g->n_arcs, K, weighted, bmode, pack) : score_ws_bytes(n, K);
+    size_t need = sh.algo ? score2_ws_bytes(n, g->n_arcs, K, weighted, bmode, pack, half) : score_ws_bytes(n, K);
     const size_t lab_off = need;
     if (where == QM_HOST || graphed) need += al256((size_t)n * 4);
     const size_t perm_off = need;
@@ -811,7 +813,7 @@ static qm_status score_impl(qm_graph *g, const int32_t *labels, int32_t K, qm_me
     Lease pin(g_pool.acquire(al256(std::max(sizeof(qm_quality), (size_t)QM_PARTIAL_WORDS * 8)) + 256, g->device,
                              true));
     if (!ws.b || !pin.b) return fail(QM_ENOMEM, "scratch allocation failed");
-    ScoreWs w = sh.algo ? carve_score2_ws(ws.ptr(), n, g->n_arcs, K, weighted, bmode, pack)
+    ScoreWs w = sh.algo ? carve_score2_ws(ws.ptr(), n, g->n_arcs, K, weighted, bmode, pack, half)
                         : carve_score_ws(ws.ptr(), n, K);
     const int32_t *dl = labels;
     if (where == QM_HOST || graphed) {
@@ -1360,7 +1362,8 @@ static qm_status run_large_batched(qm_graph *g, int dev, long long n, const std:
             shapes[p] = shape_for(g, it.K, false);
             const Shape &sh = shapes[p];
             sb = std::max(sb, sh.algo ? score2_ws_bytes(n, g->n_arcs, it.K, wt, bin_mode_of(sh.algo, wt),
-                                                        packs_labels(sh.algo, wt, g->inv != nullptr, n, it.K))
+                                                        packs_labels(sh.algo, wt, g->inv != nullptr, n, it.K),
+                                                        sh.algo == ALGO_HALF && !wt)
                                       : score_ws_bytes(n, it.K));
         }
         if (it.flags & 2) cb = std::max(cb, compare_ws_bytes(n, it.kt, it.K));
@@ -1386,7 +1389,8 @@ static qm_status run_large_batched(qm_graph *g, int dev, long long n, const std:
         if (it.flags & 1) {
             const Shape &sh = shapes[p];
             const ScoreWs w = sh.algo ? carve_score2_ws(S, n, g->n_arcs, it.K, wt, bin_mode_of(sh.algo, wt),
-                                                        packs_labels(sh.algo, wt, g->inv != nullptr, n, it.K))
+                                                        packs_labels(sh.algo, wt, g->inv != nullptr, n, it.K),
+                                                        sh.algo == ALGO_HALF && !wt)
                                       : carve_score_ws(S, n, it.K);
             ok = cudaMemsetAsync(S, 0, w.zero_bytes, cs) == cudaSuccess;
             const int Li = !ok ? -1

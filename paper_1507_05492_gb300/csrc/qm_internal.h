@@ -150,10 +150,11 @@ size_t score_ws_bytes(long long n, int K);
 // Weighted graphs take mode 0.
 // pack (two-phase pipeline, direct gathers, K <= 2^21): the far-end gathers
 // read a copy of the labels packed three to a 64-bit word.
-size_t score2_ws_bytes(long long n, long long n_arcs, int K, bool weighted = false, int bin_mode = 0,
-                       bool pack = false);
-ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool weighted = false, int bin_mode = 0,
-                        bool pack = false);
+// members: the half-edge gathers may run, which need the member array (the binned
+// ones take it, and the arc offsets, in any case).
+size_t score2_ws_bytes(long long n, long long n_arcs, int K, bool weighted, int bin_mode, bool pack, bool members);
+ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool weighted, int bin_mode, bool pack,
+                        bool members);
 // The binning mode of a two-phase launch shape on a graph (algorithm 2 or 3
 // on an unweighted graph; 0 otherwise).
 inline int bin_mode_of(int algo, bool weighted) { return (!weighted && (algo == 2 || algo == 3)) ? algo : 0; }

@@ -1699,9 +1699,10 @@ int launch_score(const GraphDev &g, const int *labels, int K, const ScoreWs &ws,
     return cudaGetLastError() == cudaSuccess ? launches : -1;
 }
 
-size_t score2_ws_bytes(long long n, long long n_arcs, int K, bool weighted, int bin_mode, bool pack)
+size_t score2_ws_bytes(long long n, long long n_arcs, int K, bool weighted, int bin_mode, bool pack, bool members)
 {
-    return carve_score2_ws(reinterpret_cast<void *>(4096), n, n_arcs, K, weighted, bin_mode, pack).bytes;
+    return carve_score2_ws(reinterpret_cast<void *>(4096), n, n_arcs, K, weighted, bin_mode, pack, members)
+        .bytes;
 }
 
 // Window size, window count and nearness distance of the binned gathers.
@@ -1719,7 +1720,8 @@ static void bin_geometry(long long n, int mode, int *shift, int *nbins, int *nea
     *nbins = (int)(((std::max(n, 1LL) - 1) >> *shift) + 1);
 }
 
-ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool weighted, int bin_mode, bool pack)
+ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool weighted, int bin_mode, bool pack,
+                        bool members)
 {
     ScoreWs w{};
     if (weighted) bin_mode = 0;
@@ -1784,10 +1786,14 @@ ScoreWs carve_score2_ws(void *base, long long n, long long n_arcs, int K, bool w
     w.big_list = (int *)p;
     p += align_up((size_t)K * 4, 256);
     w.ovf_list = nullptr;
-    w.members = (int *)p;
-    p += align_up((size_t)n * 4, 256);
-    w.aoff = (unsigned *)p;
-    p += align_up((size_t)(n + 1) * 4, 256);
+    if (members || bin_mode) {
+        w.members = (int *)p;
+        p += align_up((size_t)n * 4, 256);
+    }
+    if (bin_mode) {
+        w.aoff = (unsigned *)p;
+        p += align_up((size_t)(n + 1) * 4, 256);
+    }
     w.nbr = (int *)p;
     p += align_up((size_t)n_arcs * 4, 256) + 256;
     w.rec = (unsigned long long *)p;
