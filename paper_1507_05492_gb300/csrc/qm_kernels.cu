@@ -1816,9 +1816,11 @@ int launch_permute_hist(const int *labels, const int *inv, const long long *row_
                         const ScoreWs &ws, bool rows, int num_sms, cudaStream_t s)
 {
     if (rows) {
-        const int smem = K <= VOL_SMEM_IDS ? K * 8 : 0;
-        k_permute_vol<<<grid_for((n + HIST_UNROLL - 1) / HIST_UNROLL, 256, num_sms, 8), 256, smem, s>>>(
-            labels, inv, row_ptr, n, out, K, ws.cv, ws.status, smem ? 1 : 0);
+        const int grid = grid_for((n + HIST_UNROLL - 1) / HIST_UNROLL, 256, num_sms, 8);
+        if (K <= VOL_SMEM_IDS)
+            k_permute_vol<true><<<grid, 256, (size_t)K * 8, s>>>(labels, inv, row_ptr, n, out, K, ws.cv, ws.status);
+        else
+            k_permute_vol<false><<<grid, 256, 0, s>>>(labels, inv, row_ptr, n, out, K, ws.cv, ws.status);
         return cudaGetLastError() == cudaSuccess ? 1 : -1;
     }
     const int hist_smem = (K <= 12288) ? K * 4 : 0;
@@ -1863,8 +1865,8 @@ static void launch_rows(const RowsArgs &a, int num_sms, cudaStream_t s)
 // 10.2 us, k_count_w_tab 18.4 -> 12.3 us).
 static int ct_fill_warp(int K, int num_sms) { return K <= num_sms * CT_BLOCKS ? 96 : CT_FILL_WARP; }
 
-// Weighted graphs after k_rows<true>: one block per community counts and
-// forms the weighted pair sums, then the weighted terms and the result.
+// Weighted graphs after k_rows<true>: runs classed by length, counted and their
+// weighted pair sums formed by warps and blocks, then the weighted terms and the result.
 
 static int launch_weighted_tail(const GraphDev &g, int K, const ScoreWs &ws, const PerCommDev *pc, int num_sms,
                                 cudaStream_t s, TraceFn tr, Shard own, int launches)

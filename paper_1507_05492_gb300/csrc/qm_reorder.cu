@@ -634,7 +634,7 @@ template <int B, bool V4>
 __global__ void k_pb_tile(const int *__restrict__ labels, const unsigned short *__restrict__ lpos,
                           const int *__restrict__ toff, const int *__restrict__ tlb, long long n, int tb, int nw,
                           int ntiles, int K, int *__restrict__ tmp, int *status);
-template <int B, bool V4>
+template <int B, bool V4, bool SHARED>
 __global__ void k_pb_window(const int *__restrict__ tmp, const unsigned short *__restrict__ dloc, long long n, int wb,
                             int nw, int *__restrict__ out, int *size, int K, const long long *__restrict__ row_ptr,
                             unsigned long long *cv, int counts_at);
@@ -645,7 +645,9 @@ static cudaError_t pb_set_smem_v(size_t smem_max)
     cudaError_t e =
         cudaFuncSetAttribute(k_pb_tile<B, V4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pb_window<B, V4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+        e = cudaFuncSetAttribute(k_pb_window<B, V4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+    if (e == cudaSuccess && B == 3)  // (few ids are narrow)
+        e = cudaFuncSetAttribute(k_pb_window<3, V4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
     return e;
 }
 
@@ -842,8 +844,8 @@ __global__ void __launch_bounds__(PB_THREADS, 2) k_pb_tile(const int *__restrict
 // Pass 2, one window per block step: slots into shared memory at their new
 // ids, then the window out in order.  With `size`, the labels are counted as
 // k_hist does, with `cv` as k_permute_vol does (in shared memory from byte
-// counts_at on, where that is not 0; pass 1 has checked the labels).
-template <int B, bool V4>
+// counts_at on with SHARED; pass 1 has checked the labels).
+template <int B, bool V4, bool SHARED>
 __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restrict__ tmp,
                                                           const unsigned short *__restrict__ dloc, long long n,
                                                           int wb, int nw, int *__restrict__ out, int *size, int K,
@@ -852,8 +854,8 @@ __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restri
 {
     extern __shared__ __align__(16) unsigned char smb[];
     const int T = blockDim.x, tid = threadIdx.x;
-    unsigned *const shv = counts_at ? (unsigned *)(smb + counts_at) : nullptr;
-    if (shv) vol_smem_zero(shv, K);
+    unsigned *const shv = (unsigned *)(smb + counts_at);
+    if (SHARED) vol_smem_zero(shv, K);
     for (int w = blockIdx.x; w < nw; w += gridDim.x) {
         const long long base = (long long)w << wb;
         const int len = (int)min(n - base, 1LL << wb);
@@ -873,7 +875,7 @@ __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restri
 #pragma unroll
             for (int q = 0; q < PB_UNROLL; ++q) {
                 const bool ok = (unsigned)l[q] < (unsigned)K;
-                if (shv) {
+                if (SHARED) {
                     vol_smem_add_warp(shv, K, l[q], d[q], ok);
                 } else if (cv) {
                     vol_add_warp(cv, l[q], d[q], ok);
@@ -888,7 +890,7 @@ __global__ void __launch_bounds__(PB_THREADS, 1) k_pb_window(const int *__restri
         }
         __syncthreads();
     }
-    if (shv) vol_smem_flush(shv, K, cv);
+    if (SHARED) vol_smem_flush(shv, K, cv);
 }
 
 int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long long *row_ptr, long long n, int *tmp,
@@ -910,7 +912,7 @@ int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long 
         kern<<<g1, PB_THREADS, p1, s>>>(labels, pb.lpos, pb.toff, pb.tlb, n, pb.tb, pb.nw, pb.ntiles, K, tmp, status);
     };
     auto pass2 = [&](auto kern) { 
-        kern<<<g2, PB_THREADS, p2c, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K, row_ptr, cv, counts ? (int)at : 0);
+        kern<<<g2, PB_THREADS, p2c, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K, row_ptr, cv, (int)at);
     };
     if (tr) tr("k_pb_tile", s);
     if (narrow)
@@ -918,10 +920,9 @@ int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long 
     else
         v1 ? pass1(k_pb_tile<4, true>) : pass1(k_pb_tile<4, false>);
     if (tr) tr("k_pb_window", s);
-    if (narrow)
-        v2 ? pass2(k_pb_window<3, true>) : pass2(k_pb_window<3, false>);
-    else
-        v2 ? pass2(k_pb_window<4, true>) : pass2(k_pb_window<4, false>);
+    if (counts) v2 ? pass2(k_pb_window<3, true, true>) : pass2(k_pb_window<3, false, true>);
+    else if (narrow) v2 ? pass2(k_pb_window<3, true, false>) : pass2(k_pb_window<3, false, false>);
+    else v2 ? pass2(k_pb_window<4, true, false>) : pass2(k_pb_window<4, false, false>);
     return cudaGetLastError() == cudaSuccess ? 2 : -1;
 }
 

@@ -67,13 +67,15 @@ __global__ void k_hist_vol(const int *__restrict__ labels, const long long *__re
 }
 
 // k_permute_hist with the communities' arcs: labels of a renumbered graph
-// gathered into its order, out[j] = labels[inv[j]], counted on the way.
+// gathered into its order, out[j] = labels[inv[j]], counted on the way (SHARED:
+// in shared memory, see VOL_SMEM_IDS).
+template <bool SHARED>
 __global__ void k_permute_vol(const int *__restrict__ labels, const int *__restrict__ inv,
                               const long long *__restrict__ row_ptr, long long n, int *__restrict__ out, int K,
-                              unsigned long long *cv, int *status, int use_smem)
+                              unsigned long long *cv, int *status)
 {
-    extern __shared__ unsigned shp[];  // with use_smem: [K] members, [K] arcs
-    if (use_smem) vol_smem_zero(shp, K);
+    extern __shared__ unsigned shp[];  // SHARED: [K] members, [K] arcs
+    if (SHARED) vol_smem_zero(shp, K);
     bool bad = false;
     const int lane = threadIdx.x & 31;
     const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
@@ -95,12 +97,12 @@ __global__ void k_permute_vol(const int *__restrict__ labels, const int *__restr
             const bool in = j < n, ok = in && (unsigned)l[q] < (unsigned)K;
             if (in) out[j] = l[q];
             if (in && !ok) bad = true;
-            if (use_smem) vol_smem_add_warp(shp, K, l[q], d[q], ok);
+            if (SHARED) vol_smem_add_warp(shp, K, l[q], d[q], ok);
             else vol_add_warp(cv, l[q], d[q], ok);
         }
     }
     if (bad) atomicOr(status, 1);
-    if (use_smem) vol_smem_flush(shp, K, cv);
+    if (SHARED) vol_smem_flush(shp, K, cv);
 }
 
 // ------------------------------------------------------------------ segment bases
