@@ -32,7 +32,9 @@ constexpr int CELL_TAB_THREADS = 1024;
 constexpr int CELL_SLOTS = 24576;              // slots of a bucket's table (8 bytes each), one block per SM
 constexpr int CELL_FILL = CELL_SLOTS * 3 / 4;
 constexpr int CELL_MAX_RANGE = 1024;           // found labels of a bucket
-constexpr long long CELL_MIN_NODES = 1LL << 21;  // (a tile a third of the SMs)
+// (A tile a third of the SMs.  20% moved, sort and buckets, us a call: 2.2*10^6 nodes
+// 252 and 152, 3*10^6 316 and 183.)
+constexpr long long CELL_MIN_NODES = 1LL << 21;
 
 struct CellPlan {
     int sh;      // bucket of a found label b: b >> sh
@@ -187,7 +189,8 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
     __shared__ unsigned colmax[CELL_MAX_RANGE];
     __shared__ unsigned long long red[72];
     __shared__ unsigned late_s[CELL_TAB_THREADS / 32][32 * 5];
-    __shared__ int s_b, s_used, s_done, s_at, s_over;
+    __shared__ int s_b, s_used, s_at, s_over;
+    __shared__ unsigned s_done;
     if (block_stopped(a.status)) return;
     unsigned *const key = sm_tab, *const cnt = sm_tab + CELL_SLOTS;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -228,7 +231,10 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
             nbs[i] = 0;
             colmax[i] = 0u;
         }
-        if (tid == 0) s_used = s_done = s_over = 0;
+        if (tid == 0) {
+            s_used = s_over = 0;
+            s_done = 0u;
+        }
         block_sync();
         const int bk = s_b;
         if (bk >= a.nb) break;
@@ -251,7 +257,8 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                 // that the rest would bring them (found at the end, a nearly full table of long
                 // probes would have been filled for nothing: 10^8 nodes, two labellings at
                 // random, this kernel 7.7 and 3.0 ms; 10^7 nodes 1.04 and 0.42)
-                const int have = *(volatile int *)&s_used, read = *(volatile int *)&s_done;
+                const int have = *(volatile int *)&s_used;
+                const unsigned read = *(volatile unsigned *)&s_done;
                 if (have > CELL_FILL ||
                     (have > CELL_FILL / 2 && (long long)have * (p1 - p0) > (long long)CELL_FILL * read))
                     *(volatile int *)&s_over = 1;
@@ -278,7 +285,7 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                 __syncwarp();
                 while (nl >= 32u) fresh += follow(32u);
                 if (lane == 0) {
-                    atomicAdd(&s_done, 128);
+                    atomicAdd(&s_done, 128u);
                     if (fresh) atomicAdd(&s_used, (int)fresh);
                 }
             }
@@ -337,7 +344,10 @@ __global__ void __launch_bounds__(CELL_TAB_THREADS, 1) k_cells_table(CellArgs a)
                 R = 2u * top;
             }
             block_sync();
-            if (tid == 0) s_used = s_done = s_over = 0;
+            if (tid == 0) {
+                s_used = s_over = 0;
+                s_done = 0u;
+            }
             block_sync();
         }
         block_sync();
