@@ -911,7 +911,7 @@ int launch_permute_buckets(const int *labels, const PermBuckets &pb, const long 
     auto pass1 = [&](auto kern) {
         kern<<<g1, PB_THREADS, p1, s>>>(labels, pb.lpos, pb.toff, pb.tlb, n, pb.tb, pb.nw, pb.ntiles, K, tmp, status);
     };
-    auto pass2 = [&](auto kern) { 
+    auto pass2 = [&](auto kern) {
         kern<<<g2, PB_THREADS, p2c, s>>>(tmp, pb.dloc, n, pb.wb, pb.nw, out, size, K, row_ptr, cv, (int)at);
     };
     if (tr) tr("k_pb_tile", s);
