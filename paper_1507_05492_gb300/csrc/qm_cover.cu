@@ -51,6 +51,8 @@ constexpr int COVER_SMEM = 48 * 1024;
 // communities, by runs and by member lists, ms: L = 8 0.46 and 1.50, 16 0.74 and
 // 1.59, 32 2.53 and 1.78, 128 88 and 4.6.
 constexpr int COVER_LIST_MAX = 16;
+// Memberships of both covers from which a comparison tabulates log(N / n) and n / N.
+constexpr long long COVER_TABLE_MEMB = 1 << 15;
 constexpr int OVL_CAP = 2048;  // overlapping members of one community paired in shared memory
 
 // extra accumulator words after the GC_* words of a comparison
@@ -713,7 +715,7 @@ struct CoverCmpArgs {
     int *next_a, *next_b, *next_c;
     unsigned long long *g;
     int *status;
-    const double *logt;  // log(N / n), then n / N, 1 <= n <= LOGT_MAX
+    const double *logt;  // log(N / n), then n / N, 1 <= n <= LOGT_MAX (null: formed per cell)
     SmemPlan plan;
 };
 
@@ -807,7 +809,7 @@ __global__ void __launch_bounds__(COVER_THREADS) k_cover_cells(CoverCmpArgs a)
                     part.cells += 1;
                     const double l1 = cell_log(n, na, nb);
                     part.vi += fp_from_double(vi_term_l(n, l1), SC_VI);
-                    const bool tb = n <= LOGT_MAX;
+                    const bool tb = a.logt && n <= LOGT_MAX;
                     part.hnum += fp_from_double(nmi_num_term_q(tb ? __ldg(&a.logt[LOGT_MAX + 1 + n]) : nmi_over(n, a.N), l1,
                                                                tb ? __ldg(&a.logt[n]) : log_ratio(a.N, n)),
                                                 SC_H);
@@ -1136,16 +1138,19 @@ int launch_cover_compare(const long long *aptr, const int *amemb, long long ma, 
     a.next_c = w.counters + CC_NEXT_C;
     a.g = w.gacc;
     a.status = w.status;
-    a.logt = w.logt;
+    // the tables are a launch more, which few cells do not repay (10^3 nodes in
+    // one community each: 207 us a call with them, 192 without)
+    const bool tables = ma + mb > COVER_TABLE_MEMB;
+    a.logt = tables ? w.logt : nullptr;
     a.plan = plan_smem(COVER_THREADS, COVER_SMEM);
-    launch_batch_logt(w.logt, n, s);
+    if (tables) launch_batch_logt(w.logt, n, s);
     k_cover_cells<<<std::min(num_sms * 4, std::max(ka, 1)), COVER_THREADS, COVER_SMEM, s>>>(a);
     k_cover_rows<<<grid_of(ka, 256, num_sms, 2), 256, 0, s>>>(a);
     k_cover_cols<<<grid_of(kb, 256, num_sms, 2), 256, 0, s>>>(a);
     k_cover_pairs<true><<<std::min(num_sms * 4, std::max(ka, 1)), COVER_THREADS, 0, s>>>(a);
     k_cover_pairs<false><<<std::min(num_sms * 4, std::max(kb, 1)), COVER_THREADS, 0, s>>>(a);
     k_cover_compare_fin<<<1, 32, 0, s>>>(w.gacc, w.status, n, (qm_compare *)w.result);
-    return cudaGetLastError() == cudaSuccess ? L1 + L2 + 7 : -1;
+    return cudaGetLastError() == cudaSuccess ? L1 + L2 + 6 + (tables ? 1 : 0) : -1;
 }
 
 }  // namespace qm

@@ -78,3 +78,16 @@ def test_hub_rows(qm, oracle_mod, m):
         graph = qm.Graph(*to_dev(rp, col), reorder=reorder)
         check_quality(qm.score_cover(graph, dev, K), o, f"m={m} reorder={reorder}")
         graph.close()
+
+
+# 32,768 memberships of both covers: the most whose logarithms are formed per cell
+@pytest.mark.parametrize("n", [16_384, 16_385])
+def test_comparisons_with_and_without_tables(qm, oracle_mod, n):
+    rng = np.random.default_rng(n)
+    a, b = rng.integers(0, 90, n).astype(np.int32), rng.integers(0, 70, n).astype(np.int32)
+    mptr = np.arange(n + 1, dtype=np.int64)
+    o = oracle_mod.compare_cover(mptr, a, 90, mptr, b, 70)
+    dev = [(torch.from_numpy(mptr).cuda(), torch.from_numpy(x).cuda()) for x in (a, b)]
+    c = qm.compare_covers(dev[0], 90, dev[1], 70, n)
+    check_compare(c, o, f"n={n}")
+    assert c == qm.compare(dev[0][1], dev[1][1], 90, 70)  # a cover of one community a node: the partition's bits
